@@ -204,7 +204,7 @@ template <class S, bool COH, bool OFF32 = false>
 __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typename S::T* fout, int64_t ns, int slot,
                                                 int64_t tile, const uint32_t* __restrict__ vox,
                                                 const int* __restrict__ grid, const int* __restrict__ tile_member,
-                                                Member* members, typename S::M sp, typename S::M sm,
+                                                Member* members, Rates<typename S::M> rates,
                                                 double* partials, unsigned* counters, double* sh) {
     using M = typename S::M;
     const int mi = tile_member[tile];
@@ -227,7 +227,7 @@ __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typena
         } else if (il >= m.n - m.a_out) {
             close_outlet(d, outlet_known(d) - M(m.drho_out));
         }
-        collide(d, sp, sm);
+        collide(d, rates);
         encode_node<S>(d, seed, i, [&](auto) { return r_own; }, [&](auto qc, typename S::T v) {
             constexpr int Q = decltype(qc)::value;
             fout[(int64_t)Q * ns + i] = v;
@@ -275,11 +275,11 @@ template <class S, int MINB, bool OFF32 = false>
 __global__ void __launch_bounds__(kTile, batch_min_blocks<S, MINB>())
 k_batch_step(const typename S::T* __restrict__ fin, typename S::T* __restrict__ fout, int64_t ns, int slot,
              const uint32_t* __restrict__ vox, const int* __restrict__ grid, const int* __restrict__ tile_member,
-             Member* members, typename S::M sp, typename S::M sm, double* __restrict__ partials,
+             Member* members, Rates<typename S::M> rates, double* __restrict__ partials,
              unsigned* __restrict__ counters) {
     __shared__ double sh[32];
     batch_prefetch(fin, ns, vox);
-    batch_tile_step<S, false, OFF32>(fin, fout, ns, slot, blockIdx.x, vox, grid, tile_member, members, sp, sm,
+    batch_tile_step<S, false, OFF32>(fin, fout, ns, slot, blockIdx.x, vox, grid, tile_member, members, rates,
                                      partials, counters, sh);
 }
 
@@ -333,7 +333,7 @@ template <class S, int MINB>
 __global__ void __launch_bounds__(kTile, batch_min_blocks<S, MINB>())
 k_batch_persistent(typename S::T* f0, typename S::T* f1, int64_t ns, int slot0, int nsteps, int64_t ntiles,
                    const uint32_t* __restrict__ vox, const int* __restrict__ grid,
-                   const int* __restrict__ tile_member, Member* members, typename S::M sp, typename S::M sm,
+                   const int* __restrict__ tile_member, Member* members, Rates<typename S::M> rates,
                    double* partials, unsigned* counters, GridBarrier* bar, long long limit) {
     __shared__ double sh[32];
     unsigned gen = 0;
@@ -343,7 +343,7 @@ k_batch_persistent(typename S::T* f0, typename S::T* f1, int64_t ns, int slot0, 
         const typename S::T* fin = slot ? f1 : f0;
         typename S::T* fout = slot ? f0 : f1;
         for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-            batch_tile_step<S, true>(fin, fout, ns, slot, tile, vox, grid, tile_member, members, sp, sm, partials,
+            batch_tile_step<S, true>(fin, fout, ns, slot, tile, vox, grid, tile_member, members, rates, partials,
                                      counters, sh);
         if (!grid_barrier(bar, gridDim.x, gen, limit)) return;
     }
@@ -385,8 +385,7 @@ struct Rows {
 template <class S, bool ODD, int MINB, bool OFF32 = false>
 __global__ void __launch_bounds__(kTile, batch_min_blocks<S, MINB>())
 k_batch_aa(const Rows<typename S::T> F, int slot, const uint32_t* __restrict__ vox,
-           const int* __restrict__ grid, const int* __restrict__ tile_member, Member* members, typename S::M sp,
-           typename S::M sm, double* __restrict__ partials, unsigned* __restrict__ counters) {
+           const int* __restrict__ grid, const int* __restrict__ tile_member, Member* members, Rates<typename S::M> rates, double* __restrict__ partials, unsigned* __restrict__ counters) {
     using M = typename S::M;
     __shared__ double sh[32];
     constexpr bool kStage = ODD && OFF32 && LBM_BATCH_AA_STAGE;
@@ -437,7 +436,7 @@ k_batch_aa(const Rows<typename S::T> F, int slot, const uint32_t* __restrict__ v
         } else if (il >= m.n - m.a_out) {
             close_outlet(d, outlet_known(d) - M(m.drho_out));
         }
-        collide(d, sp, sm);
+        collide(d, rates);
         // an opaque copy of the node index for the stores (sharing the load
         // addresses would keep 19 64-bit addresses live across the collision)
         int64_t j;
@@ -883,10 +882,10 @@ int bpersistent(lbm_batch* b, int nsteps) {
             T* f1 = (T*)b->f[1];
             int64_t ns = b->ns, ntiles = b->ntiles;
             int slot0 = b->cur, n = nsteps;
-            M sp = (M)b->sp, sm = (M)b->sm;
+            auto rates = lbm::make_rates<M>(b->sp, b->sm);
             long long limit = kBarrierLimit;
             void* args[] = {&f0, &f1, &ns, &slot0, &n, &ntiles, &b->d_vox, &b->d_grid, &b->d_tile_member,
-                            &b->d_members, &sp, &sm, &b->d_partials, &b->d_counters, &b->d_bar, &limit};
+                            &b->d_members, &rates, &b->d_partials, &b->d_counters, &b->d_bar, &limit};
             return cudaLaunchCooperativeKernel((const void*)lbm::k_batch_persistent<S, MINB>, dim3(grid),
                                                dim3(lbm::kTile), args, 0, b->stream);
         };
@@ -916,7 +915,7 @@ int bstep_once(lbm_batch* b, cudaStream_t st) {
         auto launch = [&](auto kernel) {
             kernel<<<(unsigned)b->ntiles, lbm::kTile, 0, st>>>(
                 (const T*)b->f[b->cur], (T*)b->f[b->cur ^ 1], b->ns, b->cur, b->d_vox, b->d_grid,
-                b->d_tile_member, b->d_members, (M)b->sp, (M)b->sm, b->d_partials, b->d_counters);
+                b->d_tile_member, b->d_members, lbm::make_rates<M>(b->sp, b->sm), b->d_partials, b->d_counters);
         };
         // every element offset of a buffer fits in 32 bits; GB300_LBM_BATCH_ADDR64 forces the 64-bit form (tests)
         const bool off32 = 19 * (uint64_t)b->ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_BATCH_ADDR64");
@@ -945,11 +944,11 @@ int bstep_aa(lbm_batch* b, cudaStream_t st, bool odd) {
             // OFF32 when every element offset fits in 32 bits
             if (19 * (uint64_t)b->ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_BATCH_ADDR64"))
                 lbm::k_batch_aa<S, ODD, MINB, true><<<(unsigned)b->ntiles, lbm::kTile, 0, st>>>(
-                    F, b->cur, b->d_vox, b->d_grid, b->d_tile_member, b->d_members, (M)b->sp, (M)b->sm,
+                    F, b->cur, b->d_vox, b->d_grid, b->d_tile_member, b->d_members, lbm::make_rates<M>(b->sp, b->sm),
                     b->d_partials, b->d_counters);
             else
                 lbm::k_batch_aa<S, ODD, MINB><<<(unsigned)b->ntiles, lbm::kTile, 0, st>>>(
-                    F, b->cur, b->d_vox, b->d_grid, b->d_tile_member, b->d_members, (M)b->sp, (M)b->sm,
+                    F, b->cur, b->d_vox, b->d_grid, b->d_tile_member, b->d_members, lbm::make_rates<M>(b->sp, b->sm),
                     b->d_partials, b->d_counters);
         };
         const bool capped = cfg_capped(b->config);

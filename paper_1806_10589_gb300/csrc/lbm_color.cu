@@ -195,7 +195,7 @@ constexpr int color_min_blocks() {
 template <class T, bool OFF32 = false>
 __global__ void __launch_bounds__(kCB, color_min_blocks<T>())
 k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, const ColorParams* __restrict__ prm,
-             T sp, T sm, T alpha, T beta, T phi_s) {
+             Rates<T> rates, T alpha, T beta, T phi_s) {
     const int64_t i64 = (int64_t)blockIdx.x * kCB + threadIdx.x;
     if constexpr (LBM_COLOR_PREFETCH > 0) {
         // threads 0..18: momentum rows, 19..25: A rows, 26..32: B rows (rows of ns
@@ -247,7 +247,8 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
     const T a = alpha * cmag;
     const T dm1 = a, dm9 = T(0.5) * a * (T(2) * nx * nx - ny * ny - nz * nz), dm11 = T(0.5) * a * (ny * ny - nz * nz);
     const T dm13 = T(0.5) * a * nx * ny, dm14 = T(0.5) * a * ny * nz, dm15 = T(0.5) * a * nx * nz;
-    collide(d, sp, sm);
+    collide(d, rates);
+    const T sp = rates.sp;
     // an opaque copy of i for the stores (sharing the load addresses would keep
     // them live across the collision)
     int j;
@@ -486,10 +487,9 @@ int cstep_once(lbm_color* c) {
         }
         if (19 * (uint64_t)c->L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_COLOR_ADDR64"))
             lbm::k_color_step<T, true><<<nb, lbm::kCB, 0, c->stream>>>(
-                R, (const T*)c->phi, c->L, c->d_prm, (T)c->sp, (T)c->sm, (T)c->alpha, (T)c->beta, (T)c->phi_s);
+                R, (const T*)c->phi, c->L, c->d_prm, lbm::make_rates<T>(c->sp, c->sm), (T)c->alpha, (T)c->beta, (T)c->phi_s);
         else
-            lbm::k_color_step<T><<<nb, lbm::kCB, 0, c->stream>>>(R, (const T*)c->phi, c->L, c->d_prm, (T)c->sp,
-                                                                 (T)c->sm, (T)c->alpha, (T)c->beta, (T)c->phi_s);
+            lbm::k_color_step<T><<<nb, lbm::kCB, 0, c->stream>>>(R, (const T*)c->phi, c->L, c->d_prm, lbm::make_rates<T>(c->sp, c->sm), (T)c->alpha, (T)c->beta, (T)c->phi_s);
         return cudaGetLastError();
     });
     COLOR_CUDA(c, e);

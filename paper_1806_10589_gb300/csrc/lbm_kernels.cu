@@ -361,7 +361,7 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 // 19 ns < 2^32 elements), as in the gather-scatter AA step.
 template <class S, bool OFF32 = false>
 __global__ void __launch_bounds__(kBlock, step_min_blocks<S>())
-k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, typename S::M sp, typename S::M sm,
+k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates,
        BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
     using M = typename S::M;
     __shared__ double sh[32];
@@ -403,7 +403,7 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, typename S::M sp
             const M uz = outlet_known(d) - M(bc->drho_out);
             close_outlet(d, uz);
         }
-        collide(d, sp, sm);
+        collide(d, rates);
         store_step<S>(d, P, i, pol_f, r_own, seed);
         if (i64 < L.a_01) {
             if constexpr (contrib_reload<S>()) part = next_inlet_part_stored<S>(P, L, p, i, r_own);
@@ -563,7 +563,7 @@ __device__ __forceinline__ uint64_t aa_index_policy() {
 // 8 % (FP16-dev) shorter.
 template <class S, bool ODD, bool OFF32 = false>
 __global__ void __launch_bounds__(kBlock, aa_min_blocks<S, ODD>())
-k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, typename S::M sp, typename S::M sm,
+k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename S::M> rates,
           BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
     using M = typename S::M;
     __shared__ double sh[32];
@@ -642,7 +642,7 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, typename S::M s
         } else if (i64 >= L.n - L.a_out) {
             close_outlet(d, outlet_known(d) - M(bc->drho_out));
         }
-        collide(d, sp, sm);
+        collide(d, rates);
         // an opaque copy of i for the stores: sharing the load addresses would keep
         // 19 64-bit addresses live across the collision
         int j;
@@ -919,8 +919,7 @@ __device__ __forceinline__ void read_vals(typename S::M* d, const unsigned char*
 
 template <class S, int NT>
 __global__ void __launch_bounds__(NT)
-k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, typename S::M sp,
-             typename S::M sm, BcState* bc, double* __restrict__ partials,
+k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates, BcState* bc, double* __restrict__ partials,
              unsigned* __restrict__ counter) {
     using M = typename S::M;
     constexpr int SB = AsyncSlot<S>::kBytes;
@@ -981,7 +980,7 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, typename S
                 const M uz = outlet_known(d) - M(bc->drho_out);
                 close_outlet(d, uz);
             }
-            collide(d, sp, sm);
+            collide(d, rates);
             encode_node<S>(d, seed, i, [&](auto) { return r_own; }, [&](auto qc, typename S::T v) {
                 constexpr int Q = decltype(qc)::value;
                 P.out[Q][i] = v;
@@ -1284,10 +1283,10 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
         }
         // GB300_LBM_STEP_ADDR64 forces the 64-bit form (tests)
         if (19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64"))
-            k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, (M)r.sp, (M)r.sm, bc,
+            k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc,
                                                                          partials, counter);
         else
-            k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, (M)r.sp, (M)r.sm, bc, partials,
+            k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials,
                                                                    counter);
         return cudaGetLastError();
     });
@@ -1304,7 +1303,7 @@ cudaError_t launch_async_t(const void* fin, void* fout, int slot, const DevLatti
         P.out[q] = (T*)fout + (int64_t)q * L.ns;
     }
     const size_t smem = async_smem_bytes<NT>(AsyncSlot<S>::kBytes);
-    k_step_async<S, NT><<<grid, NT, smem, st>>>(P, slot, L, (M)r.sp, (M)r.sm, bc, partials, counter);
+    k_step_async<S, NT><<<grid, NT, smem, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials, counter);
     return cudaGetLastError();
 }
 
@@ -1412,12 +1411,12 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
             const bool off32 = 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_AA_ADDR64");
             if (odd && off32)
                 k_step_aa<S, true, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(
-                    F, slot, L, (M)r.sp, (M)r.sm, bc, partials, counter);
+                    F, slot, L, make_rates<M>(r.sp, r.sm), bc, partials, counter);
             else if (odd)
-                k_step_aa<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(F, slot, L, (M)r.sp, (M)r.sm, bc,
+                k_step_aa<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(F, slot, L, make_rates<M>(r.sp, r.sm), bc,
                                                                                 partials, counter);
             else
-                k_step_aa<S, false><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(F, slot, L, (M)r.sp, (M)r.sm, bc,
+                k_step_aa<S, false><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(F, slot, L, make_rates<M>(r.sp, r.sm), bc,
                                                                                  partials, counter);
             return cudaGetLastError();
         }
