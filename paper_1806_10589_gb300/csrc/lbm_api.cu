@@ -52,6 +52,8 @@ struct lbm_ctx {
     int aa_phase = 0;
     uint32_t* d_vox = nullptr;
     int* d_grid = nullptr;
+    uint2* d_win = nullptr;
+    uint32_t* d_nodew = nullptr;
     lbm::BcState h_bc{};
     lbm::BcState* d_bc = nullptr;
     double* d_red_partials = nullptr;   // inlet reductions (prime and fused), per-block partials
@@ -232,6 +234,8 @@ void release(lbm_ctx* c) {
         if (p) cudaFree(p);
     cudaFree(c->d_vox);
     cudaFree(c->d_grid);
+    cudaFree(c->d_win);
+    cudaFree(c->d_nodew);
     cudaFree(c->d_bc);
     cudaFree(c->d_red_partials);
     cudaFree(c->d_red_counter);
@@ -351,6 +355,17 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
         c->L.sz_magic = (uint64_t)(two64 / szq + (two64 % szq != 0 ? 1 : 0));
     }
 
+    // row windows, where a window index fits the node's word
+    const int64_t nwin = (int64_t)lbm::windows_per_row(nx) * py * pz;
+    const bool windows = nwin < (int64_t)1 << 27;
+    if (windows) {
+        c->L.wy = lbm::windows_per_row(nx);
+        c->L.wz = c->L.wy * (int)py;
+        const unsigned __int128 two64 = (unsigned __int128)1 << 64;
+        const unsigned __int128 wzq = (unsigned __int128)(uint64_t)c->L.wz;
+        c->L.wz_magic = (uint64_t)(two64 / wzq + (two64 % wzq != 0 ? 1 : 0));
+    }
+
     // ---- device memory
     int rc = LBM_OK;
     const size_t fbytes = (size_t)19 * (size_t)c->L.ns * (size_t)lbm::elem_size(precision);
@@ -360,6 +375,8 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
     if ((rc = dev_alloc(c, &c->f[0], fbytes)) || (rc = dev_alloc(c, &c->f[1], fbytes)) ||
         (rc = dev_alloc(c, &c->d_vox, vox.size() * sizeof(uint32_t))) ||
         (rc = dev_alloc(c, &c->d_grid, grid.size() * sizeof(int))) ||
+        (windows && (rc = dev_alloc(c, &c->d_win, (size_t)nwin * sizeof(uint2)))) ||
+        (windows && (rc = dev_alloc(c, &c->d_nodew, (size_t)c->L.ns * sizeof(uint32_t)))) ||
         (rc = dev_alloc(c, &c->d_bc, sizeof(lbm::BcState))) ||
         (rc = dev_alloc(c, &c->d_red_partials, (size_t)nb_red * sizeof(double))) ||
         (rc = dev_alloc(c, &c->d_red_counter, sizeof(unsigned))) ||
@@ -374,9 +391,14 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
     }
     c->L.vox = c->d_vox;
     c->L.grid = c->d_grid;
+    c->L.win = c->d_win;
+    c->L.nodew = c->d_nodew;
     cudaError_t e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_vox, vox.data(), vox.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_grid, grid.data(), grid.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && windows) e = cudaMemset(c->d_nodew, 0, (size_t)c->L.ns * sizeof(uint32_t));
+    if (e == cudaSuccess && windows)
+        e = lbm::launch_build_windows(c->d_grid, c->d_vox, 0u, n, nx, ny, nz, 0u, c->d_win, c->d_nodew, 0);
     if (e == cudaSuccess) e = cudaMemset(c->d_red_counter, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(c->d_step_counter, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(c->d_mon_counter, 0, sizeof(unsigned));

@@ -156,7 +156,7 @@ __device__ __forceinline__ double next_inlet_part_b(const typename S::M* d, cons
     double s = 0.0;
     auto val = [&](auto qc) -> double {
         constexpr int Q = decltype(qc)::value;
-        return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i, Q)), r_own);
+        return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i)), r_own);
     };
     auto dest_is_pore = [&](auto qc) -> bool {
         constexpr int Q = decltype(qc)::value;
@@ -442,7 +442,7 @@ k_batch_aa(const Rows<typename S::T> F, int slot, const uint32_t* __restrict__ v
         int64_t j;
         asm volatile("mov.b64 %0, %1;" : "=l"(j) : "l"(i));
         if constexpr (kStage) {
-            F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i, 0));
+            F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i));
             // the destination of Q is the gather source of opp(Q): row Q for a pore
             // there, row opp(Q) (bounce-back) otherwise
             const uint32_t ns32 = (uint32_t)(F.row[1] - F.row[0]);
@@ -454,11 +454,11 @@ k_batch_aa(const Rows<typename S::T> F, int slot, const uint32_t* __restrict__ v
                     const bool pore = (Q & 1) ? off < (uint32_t)(Q + 1) * ns32 : off >= (uint32_t)Q * ns32;
                     r = pore ? r_own + M(cz(Q)) * g : r_own;
                 }
-                F.row[0][off] = S::template enc_sr<Q>(d[Q], r, sr_key<S>(seed, i, Q));
+                F.row[0][off] = S::template enc_sr<Q>(d[Q], r, sr_key<S>(seed, i));
             });
         } else if constexpr (ODD) {
             const int64_t ps = __ldg(vox + j);
-            F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i, 0));
+            F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i));
             if constexpr (OFF32) {
                 // one store per value at row 0 plus a 32-bit offset, destination row and plane selected
                 const uint32_t ns32 = (uint32_t)(F.row[1] - F.row[0]);
@@ -467,13 +467,13 @@ k_batch_aa(const Rows<typename S::T> F, int slot, const uint32_t* __restrict__ v
                     const int dst = __ldg(grid + ps + m.goff[opp(Q)]);  // x + xi_Q is the pull source of opp(Q)
                     const bool pore = dst >= 0;
                     F.row[0][pore ? (uint32_t)Q * ns32 + (uint32_t)dst : (uint32_t)opp(Q) * ns32 + (uint32_t)j] =
-                        S::template enc_sr<Q>(d[Q], pore ? r_own + M(cz(Q)) * g : r_own, sr_key<S>(seed, i, Q));
+                        S::template enc_sr<Q>(d[Q], pore ? r_own + M(cz(Q)) * g : r_own, sr_key<S>(seed, i));
                 });
             } else if constexpr (S::kRef && !LBM_BATCH16_PAIR_SCATTER) {
                 for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
                     constexpr int Q = decltype(qc)::value + 1;
                     const int dst = __ldg(grid + ps + m.goff[opp(Q)]);  // x + xi_Q is the pull source of opp(Q)
-                    const uint32_t key = sr_key<S>(seed, i, Q);
+                    const uint32_t key = sr_key<S>(seed, i);
                     if (dst >= 0) F.row[Q][dst] = S::template enc_sr<Q>(d[Q], r_own + M(cz(Q)) * g, key);
                     else F.row[opp(Q)][j] = S::template enc_sr<Q>(d[Q], r_own, key);
                 });
@@ -485,7 +485,7 @@ k_batch_aa(const Rows<typename S::T> F, int slot, const uint32_t* __restrict__ v
                     const int dq1 = __ldg(grid + ps + m.goff[Q]);      // and x - xi_Q that of Q
                     const uint32_t h = S::template enc_sr2<Q>(d[Q], dq >= 0 ? r_own + M(cz(Q)) * g : r_own, d[Q + 1],
                                                               dq1 >= 0 ? r_own - M(cz(Q)) * g : r_own,
-                                                              sr_key<S>(seed, i, Q), sr_key<S>(seed, i, Q + 1));
+                                                              sr_key<S>(seed, i));
                     if (dq >= 0) F.row[Q][dq] = S::half_of(h, true);
                     else F.row[Q + 1][j] = S::half_of(h, true);
                     if (dq1 >= 0) F.row[Q + 1][dq1] = S::half_of(h, false);
@@ -516,7 +516,7 @@ k_batch_aa(const Rows<typename S::T> F, int slot, const uint32_t* __restrict__ v
             auto val = [&](auto qc) -> double {
                 constexpr int Q = decltype(qc)::value;
                 const M rq = (ODD && cz(Q) < 0) ? r_own - g : r_own;
-                return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], rq, sr_key<S>(seed, i, Q)), rq);
+                return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], rq, sr_key<S>(seed, i)), rq);
             };
             auto dest_is_pore = [&](auto qc) -> bool {
                 constexpr int Q = decltype(qc)::value;

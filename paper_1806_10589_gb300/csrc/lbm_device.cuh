@@ -72,28 +72,15 @@ constexpr int ZOUT = -2;
 // depends on its own input only.  enc_sr2 rounds both values of an opposite
 // pair (q odd, q + 1) with one instruction.
 //
-// LBM_SR_MODE chooses the random numbers of a node's 19 values:
-//   2 (default): one random number per node for all 19 values;
-//   1: one per opposite pair, its two values on disjoint bit fields;
-//   0: one per direction (h + q * phi) * C, its top bits, as the conversion-
-//      free encode (add the bits, truncate) used before; gives identical states.
-// Each value is rounded without bias in every mode; what differs is how the
-// errors of a node's values are correlated.  With one number per node, an
-// opposite pair's errors are positively correlated (a large number rounds both
-// up), so they partly cancel in the momentum sum_q xi_q d_q.  Measured on a
-// 128^3 pack, 5000 steps from the FP64 steady state, L2 / max velocity error
-// against FP64: FP16-dev 3.7e-4 / 1.6e-3 (mode 2), 5.7e-4 / 7.2e-3 (mode 1),
-// 3.8e-4 / 2.9e-3 (mode 0); BF16-dev 3.0e-3 / 2.7e-2, 4.7e-3 / 5.9e-2,
-// 3.1e-3 / 2.6e-2; permeability within 6e-5 in all.  Mode 2 also needs no
-// per-value key arithmetic (FP16-dev AA step 0.1617 ms against 0.1660 and 0.1761).
-#ifndef LBM_SR_MODE
-#define LBM_SR_MODE 2
-#endif
-constexpr bool kSrSameField = LBM_SR_MODE == 2;
+// All 19 values of a node draw the same random number.  Each value is rounded
+// without bias; the errors of an opposite pair are then positively correlated (a
+// large number rounds both up), so they partly cancel in the momentum
+// sum_q xi_q d_q.  Measured on a 128^3 pack, 5000 steps from the FP64 steady
+// state, L2 / max velocity error against FP64: FP16-dev 3.7e-4 / 1.6e-3; with
+// independent numbers for the two values of a pair 5.7e-4 / 7.2e-3, with one per
+// direction 3.8e-4 / 2.9e-3; BF16-dev 3.0e-3 / 2.7e-2, 4.7e-3 / 5.9e-2, 3.1e-3 /
+// 2.6e-2; permeability within 6e-5 in all.
 constexpr float DEV_SCALE = 1024.0f;
-// Half of the packed stochastic conversion that direction q uses.
-__host__ __device__ constexpr bool sr_upper(int q) { return q == 0 || (q & 1); }
-
 // 32-bit integer hash: the "lowbias32" finaliser published by C. Wellons
 // (xor-shift / multiply rounds).
 __host__ __device__ __forceinline__ uint32_t sr_hash(uint32_t x) {
@@ -145,17 +132,12 @@ struct StoreF16 {
         return __ushort_as_half((unsigned short)(upper ? d >> 16 : d & 0xFFFFu));
     }
     template <int Q> __device__ static float scaled(M v, M r) { return fmaf(v, float(1024.0 / wq(Q)), -1024.0f * r); }
-    // rbits of the upper / lower half from a key (13-bit fields at bits 16 and 0)
-    __device__ static uint32_t bits_hi(uint32_t u) { return LBM_SR_MODE == 0 ? u >> 3 : u; }
-    __device__ static uint32_t bits_lo(uint32_t u) { return LBM_SR_MODE == 0 ? u >> 19 : u; }
     template <int Q> __device__ static T enc_sr(M v, M r, uint32_t u) {
-        constexpr bool up = sr_upper(Q) && !kSrSameField;
-        return half_of(up ? cvt_rs(scaled<Q>(v, r), 0.0f, bits_hi(u)) : cvt_rs(0.0f, scaled<Q>(v, r), bits_lo(u)), up);
+        return half_of(cvt_rs(0.0f, scaled<Q>(v, r), u), false);
     }
-    template <int Q> __device__ static uint32_t enc_sr2(M v, M r, M v1, M r1, uint32_t u, uint32_t u1) {
+    template <int Q> __device__ static uint32_t enc_sr2(M v, M r, M v1, M r1, uint32_t u) {
         static_assert(Q & 1, "a pair starts at an odd direction");
-        return cvt_rs(scaled<Q>(v, r), scaled<Q + 1>(v1, r1),
-                      LBM_SR_MODE == 0 ? ((bits_hi(u) & 0xFFFF0000u) | bits_lo(u1)) : u);
+        return cvt_rs(scaled<Q>(v, r), scaled<Q + 1>(v1, r1), u);
     }
 };
 struct StoreBF16 {
@@ -177,39 +159,23 @@ struct StoreBF16 {
         return __ushort_as_bfloat16((unsigned short)(upper ? d >> 16 : d & 0xFFFFu));
     }
     template <int Q> __device__ static float scaled(M v, M r) { return fmaf(v, float(1024.0 / wq(Q)), -1024.0f * r); }
-    // rbits of the upper / lower half from a key (16-bit fields at bits 16 and 0)
-    __device__ static uint32_t bits_hi(uint32_t u) { return u; }
-    __device__ static uint32_t bits_lo(uint32_t u) { return LBM_SR_MODE == 0 ? u >> 16 : u; }
     template <int Q> __device__ static T enc_sr(M v, M r, uint32_t u) {
-        constexpr bool up = sr_upper(Q) && !kSrSameField;
-        return half_of(up ? cvt_rs(scaled<Q>(v, r), 0.0f, bits_hi(u)) : cvt_rs(0.0f, scaled<Q>(v, r), bits_lo(u)), up);
+        return half_of(cvt_rs(0.0f, scaled<Q>(v, r), u), false);
     }
-    template <int Q> __device__ static uint32_t enc_sr2(M v, M r, M v1, M r1, uint32_t u, uint32_t u1) {
+    template <int Q> __device__ static uint32_t enc_sr2(M v, M r, M v1, M r1, uint32_t u) {
         static_assert(Q & 1, "a pair starts at an odd direction");
-        return cvt_rs(scaled<Q>(v, r), scaled<Q + 1>(v1, r1),
-                      LBM_SR_MODE == 0 ? ((u & 0xFFFF0000u) | bits_lo(u1)) : u);
+        return cvt_rs(scaled<Q>(v, r), scaled<Q + 1>(v1, r1), u);
     }
 };
 
-// Random bits of the stochastic rounding of value (node i, direction q) in the
-// step with seed `seed` (no work for the formats that store exactly): one hash
-// per node (the same call for every q, computed once).  Mode 2 places its upper
-// 16 bits in both halves of the rbits word, so either half of a conversion
-// draws the same number; modes 0 and 1 add a Weyl step per direction or pair
-// and mix it by one multiply.
+// Random bits of the stochastic rounding of node i in the step with seed `seed`
+// (no work for the formats that store exactly): the upper 16 bits of one hash in
+// both halves of the rbits word, so either half of a conversion draws the same
+// number.
 template <class S>
-__device__ __forceinline__ uint32_t sr_key(uint32_t seed, int64_t i, int q) {
-    if constexpr (S::kRef) {
-        const uint32_t h = sr_hash(seed ^ (uint32_t)i);
-        if constexpr (LBM_SR_MODE == 2) {
-            (void)q;
-            return __byte_perm(h, 0u, 0x3232u);
-        } else {
-            return (h + (uint32_t)(LBM_SR_MODE == 1 ? (q + 1) >> 1 : q) * 0x9E3779B9U) * 0x2C1B3C6DU;
-        }
-    } else {
-        return 0u;
-    }
+__device__ __forceinline__ uint32_t sr_key(uint32_t seed, int64_t i) {
+    if constexpr (S::kRef) return __byte_perm(sr_hash(seed ^ (uint32_t)i), 0u, 0x3232u);
+    else return 0u;
 }
 
 // Encodes the 19 values d of a node and hands each to put(Q, value), Q an
@@ -220,9 +186,9 @@ template <class S, int Q, class Ref, class Put>
 __device__ __forceinline__ void encode_pair_(const typename S::M* d, uint32_t seed, int64_t i, Ref& ref, Put& put) {
     using C0 = std::integral_constant<int, Q>;
     using C1 = std::integral_constant<int, Q + 1>;
-    const uint32_t u = sr_key<S>(seed, i, Q);
+    const uint32_t u = sr_key<S>(seed, i);
     if constexpr (S::kRef) {
-        const uint32_t h = S::template enc_sr2<Q>(d[Q], ref(C0{}), d[Q + 1], ref(C1{}), u, sr_key<S>(seed, i, Q + 1));
+        const uint32_t h = S::template enc_sr2<Q>(d[Q], ref(C0{}), d[Q + 1], ref(C1{}), u);
         put(C0{}, S::half_of(h, true));
         put(C1{}, S::half_of(h, false));
     } else {
@@ -234,7 +200,7 @@ template <class S, class Ref, class Put, int... P>
 __device__ __forceinline__ void encode_node_(const typename S::M* d, uint32_t seed, int64_t i, Ref& ref, Put& put,
                                              std::integer_sequence<int, P...>) {
     using C0 = std::integral_constant<int, 0>;
-    put(C0{}, S::template enc_sr<0>(d[0], ref(C0{}), sr_key<S>(seed, i, 0)));
+    put(C0{}, S::template enc_sr<0>(d[0], ref(C0{}), sr_key<S>(seed, i)));
     (encode_pair_<S, 2 * P + 1>(d, seed, i, ref, put), ...);
 }
 template <class S, class Ref, class Put>
@@ -279,6 +245,59 @@ __device__ __forceinline__ M ref_at(const BcState* bc, int z) {
 template <class M>
 __device__ __forceinline__ M ref_slope(const BcState* bc) {
     return M(bc->ref_g[bc->ref_cur]);
+}
+
+// ------------------------------------------------------ row windows ---
+// Neighbour ids without an id grid.  Pores are numbered along x inside a row, so
+// the id of a pore is the number of the row's first pore plus the pores before
+// it.  Each padded row (z, y) is cut into windows of 30 voxels; a window holds a
+// 32-bit pore mask -- bit k is the voxel at padded x = 30 w + k, so that both
+// neighbours of its 30 voxels (bits 1..30) lie in the same word -- and the id of
+// the first pore at or after bit 0.  A node's word is (window << 5) | bit.  The
+// 18 neighbours of a node lie in 9 rows: one 8-byte load and one population
+// count per row give the ids of its three dx taps (the eight rows other than the
+// node's own; there the ids are i - 1 and i + 1), where the id grid took one
+// load per neighbour.  The windows of the 256^3 pack take 4.8 MB (the id grid
+// 68 MB) and the lanes of a warp mostly share them, so these loads hit L1.
+// Measured, 100 steps, id grid -> windows: FP32 AA pattern on the 256^3 pack 16.97
+// -> 16.19 ms, BF16-dev two-buffer on a 157x149x171 pack 4.08 -> 3.90 ms, bitwise
+// equal states.  The id grid stays for boxes of 2^27 windows or more (and for the
+// inlet sums and conversions).
+constexpr int kWinVoxels = 30;
+// Direction with velocity (x, y, z), -1 if there is none.
+__host__ __device__ constexpr int dir_of(int x, int y, int z) {
+    for (int q = 0; q < 19; ++q)
+        if (cx(q) == x && cy(q) == y && cz(q) == z) return q;
+    return -1;
+}
+// The taps of one row (dy, dz): f(Q, pore, id) for every direction Q whose pull
+// source x - xi_Q lies in that row.
+template <int DY, int DZ, class F>
+__device__ __forceinline__ void row_links(uint2 v, uint32_t b, uint32_t low, uint32_t i, F& f) {
+    constexpr int QM = dir_of(1, -DY, -DZ), Q0 = dir_of(0, -DY, -DZ), QP = dir_of(-1, -DY, -DZ);
+    const uint32_t t = v.x >> (b - 1u);  // bits 0, 1, 2: x - 1, x, x + 1
+    const uint32_t c = (DY == 0 && DZ == 0) ? i : v.y + (uint32_t)__popc(v.x & low);
+    if constexpr (QM > 0) f(std::integral_constant<int, QM>{}, (t & 1u) != 0u, c - 1u);
+    if constexpr (Q0 > 0) f(std::integral_constant<int, Q0>{}, (t & 2u) != 0u, c);
+    if constexpr (QP > 0)
+        f(std::integral_constant<int, QP>{}, (t & 4u) != 0u, (DY == 0 && DZ == 0) ? c + 1u : c + ((t >> 1) & 1u));
+}
+// All 18 links of node i with word `word`; wy, wz: window strides of y and z.
+template <class F>
+__device__ __forceinline__ void for_links(const uint2* __restrict__ win, uint32_t word, int wy, int wz, uint32_t i, F&& f) {
+    const uint32_t b = word & 31u, low = (1u << b) - 1u;
+    const uint2* w = win + (word >> 5);
+    const uint2 v00 = __ldg(w), vm0 = __ldg(w - wy), vp0 = __ldg(w + wy), v0m = __ldg(w - wz), v0p = __ldg(w + wz);
+    const uint2 vmm = __ldg(w - wy - wz), vpm = __ldg(w + wy - wz), vmp = __ldg(w - wy + wz), vpp = __ldg(w + wy + wz);
+    row_links<0, 0>(v00, b, low, i, f);
+    row_links<-1, 0>(vm0, b, low, i, f);
+    row_links<1, 0>(vp0, b, low, i, f);
+    row_links<0, -1>(v0m, b, low, i, f);
+    row_links<0, 1>(v0p, b, low, i, f);
+    row_links<-1, -1>(vmm, b, low, i, f);
+    row_links<1, -1>(vpm, b, low, i, f);
+    row_links<-1, 1>(vmp, b, low, i, f);
+    row_links<1, 1>(vpp, b, low, i, f);
 }
 
 // ------------------------------------------------------- cache hints ---

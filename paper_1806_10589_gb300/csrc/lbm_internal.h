@@ -22,7 +22,20 @@ struct DevLattice {
     const int* grid;      // [(nz+2)(ny+2)(nx+2)] padded id grid
     int goff[19];         // padded-grid offset of the pull source x - xi_q, per q
     uint64_t sz_magic;    // ceil(2^64 / sz): plane of a padded voxel index
+    // Row windows (lbm_device.cuh), null when a window index needs more than 27 bits.
+    const uint2* win;         // [(nz+2)(ny+2) wy] pore mask and first id of 30 voxels of a padded row
+    const uint32_t* nodew;    // [n] (window << 5) | bit of each pore node
+    int wy, wz;               // window strides of y and z
+    uint64_t wz_magic;        // ceil(2^64 / wz): plane of a window index
 };
+
+inline int windows_per_row(int nx) { return (nx + 29) / 30; }
+// Fills the row windows of one padded box from its id grid (grid: first entry of
+// the box), and the words of its nodes from their padded voxel indices (counted
+// from the box's first entry plus `vox0`); `w0` is the index of the box's first
+// window.  The window index has to fit 27 bits.
+cudaError_t launch_build_windows(const int* grid, const uint32_t* vox, uint32_t vox0, int64_t n, int nx, int ny,
+                                 int nz, uint32_t w0, uint2* win, uint32_t* nodew, cudaStream_t st);
 
 struct Relax {
     double sp, sm;  // s+ and s- of the two-relaxation-time form

@@ -54,6 +54,12 @@ __device__ __forceinline__ typename S::M own_ref(const BcState* bc, const DevLat
     else return M(0);
 }
 template <class S>
+__device__ __forceinline__ typename S::M own_ref_word(const BcState* bc, const DevLattice& L, uint32_t word) {
+    using M = typename S::M;
+    if constexpr (S::kRef) return ref_at<M>(bc, plane_of((uint64_t)(word >> 5), L.wz_magic));
+    else return M(0);
+}
+template <class S>
 __device__ __forceinline__ typename S::M own_slope(const BcState* bc) {
     using M = typename S::M;
     if constexpr (S::kRef) return ref_slope<M>(bc);
@@ -120,7 +126,7 @@ __device__ __forceinline__ void st_stream(T* a, T v, uint64_t pol) {
 // Pull all 19 values of node i (padded voxel p): a pore source gives its own
 // value, a solid or outside source the node's opposite value (halfway
 // bounce-back; the z-outside ones are replaced by the closure).
-template <class S, bool OFF32 = false>
+template <class S>
 __device__ __forceinline__ void pull_step(typename S::M* d, const StepPtrs<typename S::T>& P,
                                           const DevLattice& L, uint32_t p, int i, uint64_t pol_f,
                                           uint64_t pol_idx, typename S::M r_own, typename S::M g) {
@@ -132,16 +138,28 @@ __device__ __forceinline__ void pull_step(typename S::M* d, const StepPtrs<typen
         } else {
             // padded voxel indices fit in 32 bits (checked at creation)
             const int id = ld_index(L.grid + (uint32_t)(p + (uint32_t)L.goff[Q]), pol_idx);
-            const typename S::T* a;
-            if constexpr (OFF32)  // row 0 plus one 32-bit element offset (rows are ns apart)
-                a = P.in[0] + (id >= 0 ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)id
-                                       : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)i);
-            else
-                a = id >= 0 ? P.in[Q] + id : P.in[opp(Q)] + i;
+            const typename S::T* a = id >= 0 ? P.in[Q] + id : P.in[opp(Q)] + i;
             // a pulled value was written on plane z - xi_z (reference r_own - g xi_z)
             const M r = (cz(Q) != 0 && id >= 0) ? r_own - M(cz(Q)) * g : r_own;
             d[Q] = S::template dec<Q>(ld_stream(a, pol_f), r);
         }
+    });
+}
+
+// The same from the row windows: every source is row 0 plus one 32-bit element
+// offset (rows are ns apart, buffers of fewer than 2^32 elements).
+template <class S>
+__device__ __forceinline__ void pull_step_win(typename S::M* d, const StepPtrs<typename S::T>& P, const DevLattice& L,
+                                              uint32_t word, int i, uint64_t pol_f, typename S::M r_own,
+                                              typename S::M g) {
+    using M = typename S::M;
+    d[0] = S::template dec<0>(ld_stream(P.in[0] + i, pol_f), r_own);
+    for_links(L.win, word, L.wy, L.wz, (uint32_t)i, [&](auto qc, bool pore, uint32_t id) {
+        constexpr int Q = decltype(qc)::value;
+        const uint32_t off = pore ? (uint32_t)Q * (uint32_t)L.ns + id : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)i;
+        // a pulled value was written on plane z - xi_z (reference r_own - g xi_z)
+        const M r = (cz(Q) != 0 && pore) ? r_own - M(cz(Q)) * g : r_own;
+        d[Q] = S::template dec<Q>(ld_stream(P.in[0] + off, pol_f), r);
     });
 }
 
@@ -330,7 +348,7 @@ __device__ __forceinline__ double next_inlet_part(const typename S::M* d, const 
                                                   int64_t p, int i, typename S::M r_own, uint32_t seed) {
     return inlet_contribution<S>(L, (uint32_t)p, i, [&](auto qc) -> double {
         constexpr int Q = decltype(qc)::value;
-        return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i, Q)), r_own);
+        return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i)), r_own);
     });
 }
 
@@ -357,9 +375,9 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 #define LBM_STEP_PREFETCH 224
 #endif
 
-// OFF32: pulls addressed as row 0 plus a 32-bit element offset (buffers of
-// 19 ns < 2^32 elements), as in the gather-scatter AA step.
-template <class S, bool OFF32 = false>
+// WIN: pulls from the row windows, addressed as row 0 plus a 32-bit element
+// offset (buffers of 19 ns < 2^32 elements), as in the gather-scatter AA step.
+template <class S, bool WIN = false>
 __global__ void __launch_bounds__(kBlock, step_min_blocks<S>())
 k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates,
        BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
@@ -376,7 +394,7 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
         const int64_t s = ((int64_t)blockIdx.x + LBM_STEP_PREFETCH) * kBlock;
         const int t = (int)threadIdx.x;
         if (t < 19) l2_prefetch_range(P.in[0] + (int64_t)t * L.ns, s, kBlock, L.ns);
-        else if (t == 19) l2_prefetch_range(L.vox, s, kBlock, L.n & ~(int64_t)3);
+        else if (t == 19) l2_prefetch_range(WIN ? L.nodew : L.vox, s, kBlock, L.n & ~(int64_t)3);
     }
     if (i64 < L.n) {
 #if LBM_L2_HINTS >= 2
@@ -389,11 +407,12 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
 #else
         const uint64_t pol_idx = 0;
 #endif
-        const uint32_t p = ld_index(L.vox + i, pol_idx);
-        const M r_own = own_ref<S>(bc, L, p), g = own_slope<S>(bc);
+        const uint32_t p = ld_index((WIN ? L.nodew : L.vox) + i, pol_idx);  // node word or padded voxel
+        const M r_own = WIN ? own_ref_word<S>(bc, L, p) : own_ref<S>(bc, L, p), g = own_slope<S>(bc);
         const uint32_t seed = step_seed<S>(bc, slot);
         M d[19];
-        pull_step<S, OFF32>(d, P, L, p, i, pol_f, pol_idx, r_own, g);
+        if constexpr (WIN) pull_step_win<S>(d, P, L, p, i, pol_f, r_own, g);
+        else pull_step<S>(d, P, L, p, i, pol_f, pol_idx, r_own, g);
         if (i < L.a_in) {
             // Section 2: after streaming, before collision.  u_z from Eq. (inlet)
             // with the density of Eq. (potential); then the Appendix B closure.
@@ -406,8 +425,9 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
         collide(d, rates);
         store_step<S>(d, P, i, pol_f, r_own, seed);
         if (i64 < L.a_01) {
-            if constexpr (contrib_reload<S>()) part = next_inlet_part_stored<S>(P, L, p, i, r_own);
-            else part = next_inlet_part<S>(d, L, p, i, r_own, seed);
+            const uint32_t pv = WIN ? __ldg(L.vox + i) : p;
+            if constexpr (contrib_reload<S>()) part = next_inlet_part_stored<S>(P, L, pv, i, r_own);
+            else part = next_inlet_part<S>(d, L, pv, i, r_own, seed);
         }
     }
     // blocks that hold plane z = 0 or z = 1 nodes (block-uniform branch)
@@ -452,20 +472,6 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
 // faces are kept like bounced ones; the closures overwrite them.  The next
 // step's inlet density is formed exactly as in k_step: the landing rule of a
 // post-collision value does not depend on where it is stored.
-// Where the gather-scatter step keeps its 18 neighbour ids across the
-// collision (LBM_AA_IDS): 0 = registers (spills at the 64-register cap),
-// 1 = loads them again from the id grid, 2 = shared memory (18 KB per block;
-// with LBM_AA_SMEM_OFF the gather offsets instead of the ids).  Measured best:
-// 2 for every format (LBM_AA16_IDS for the 16-bit ones); with ids instead of
-// offsets staged, 1 and 2 were equal in FP32.
-#ifndef LBM_AA_IDS
-#define LBM_AA_IDS 2
-#endif
-#ifndef LBM_AA16_IDS
-#define LBM_AA16_IDS 2
-#endif
-
-
 // Row pointers of the single buffer as kernel parameters (constant bank), as
 // for k_step: no registers spent on 19 row addresses.
 template <class T>
@@ -512,13 +518,6 @@ struct AAPtrs {
 #ifndef LBM_AA16_PREFETCH
 #define LBM_AA16_PREFETCH 224
 #endif
-// LBM_AA16_PAIR_SCATTER: 1 = the 16-bit gather-scatter step rounds each
-// opposite pair with one conversion before its two stores, 0 = one conversion
-// per value next to its store.  Measured on the 256^3 pack: 0 is 2.9 % (FP16)
-// and 2.8 % (BF16) faster in that launch (the node-local launch rounds pairs).
-#ifndef LBM_AA16_PAIR_SCATTER
-#define LBM_AA16_PAIR_SCATTER 0
-#endif
 template <class S, bool ODD>
 constexpr int aa_min_blocks() {
     if constexpr (sizeof(typename S::M) == 8) return 1;
@@ -542,36 +541,23 @@ __device__ __forceinline__ uint64_t aa_index_policy() {
 #endif
 }
 
-// LBM_AA_SMEM_OFF: 1 = with ids staged in shared memory (LBM_AA16_IDS /
-// LBM_AA_IDS 2) and 32-bit offsets, the gather stores each direction's element
-// offset instead of its id.  The scatter destination of q is the gather source
-// of opp(q) -- F[q][x + xi_q] for a pore there, else the bounce-back slot
-// F[opp q][x], both read by the gather of opp(q) -- so the scatter reads its
-// offset as it is and needs no id test or offset arithmetic; 0 = ids staged.
-// Measured on the 256^3 pack (same-call A/B, bitwise equal states): the
-// gather-scatter launch 0.2006 -> 0.1825 ms (FP16-dev), 0.2024 -> 0.1840 ms
-// (BF16-dev), and with the FP32 ids staged as well (LBM_AA_IDS 2; staged ids
-// alone gave 0.2007 ms) 0.2013 -> 0.1972 ms.
-#ifndef LBM_AA_SMEM_OFF
-#define LBM_AA_SMEM_OFF 1
-#endif
-
-// OFF32 (gather-scatter launch, buffers of 19 ns < 2^32 elements): every
-// neighbour address is row 0 plus one 32-bit element offset, the source or
-// destination row chosen by a 32-bit select, instead of a select between two
-// 64-bit row pointers.  Measured on the 256^3 pack: the launch 6.5 % (FP32) and
-// 8 % (FP16-dev) shorter.
-template <class S, bool ODD, bool OFF32 = false>
+// WIN (gather-scatter launch, buffers of 19 ns < 2^32 elements): neighbours from
+// the row windows, every neighbour address row 0 plus one 32-bit element offset,
+// and each direction's gather offset staged in shared memory.  The scatter
+// destination of q is the gather source of opp(q) -- F[q][x + xi_q] for a pore
+// there, else the bounce-back slot F[opp q][x], both read by the gather of
+// opp(q) -- so the scatter reads its offset as it is and needs no id test or
+// offset arithmetic (the launch on the 256^3 pack, ids staged -> offsets staged:
+// 0.2006 -> 0.1825 ms FP16-dev, 0.2013 -> 0.1972 ms FP32).  Otherwise the ids of
+// the id grid are staged and the rows addressed by 64-bit pointers.
+template <class S, bool ODD, bool WIN = false>
 __global__ void __launch_bounds__(kBlock, aa_min_blocks<S, ODD>())
 k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename S::M> rates,
           BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
     using M = typename S::M;
     __shared__ double sh[32];
     __shared__ bool last;
-    constexpr int kIds = S::kRef ? LBM_AA16_IDS : LBM_AA_IDS;
-    // staged per direction: the gather's element offset (kOffs) or the pore id
-    constexpr bool kOffs = OFF32 && kIds == 2 && LBM_AA_SMEM_OFF;
-    __shared__ int sid[(ODD && kIds == 2) ? 18 : 1][kBlock];
+    __shared__ int sid[ODD ? 18 : 1][kBlock];  // gather offset (WIN) or pore id per direction
     const int64_t i64 = (int64_t)blockIdx.x * kBlock + threadIdx.x;
     const int i = (int)i64;
     double part = 0.0;
@@ -579,22 +565,33 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
     if constexpr (ODD && kAhead > 0) {
         // threads 0..18: row q of the buffer (rows are F.row[0] + q ns, as
         // launched; 128-element padding keeps every range 16-byte aligned for
-        // 2-byte values too); thread 19: the voxel list, cut to a multiple of 4 entries
+        // 2-byte values too); thread 19: the node list, cut to a multiple of 4 entries
         const int64_t s = ((int64_t)blockIdx.x + kAhead) * kBlock;
         const int t = (int)threadIdx.x;
         if (t < 19) l2_prefetch_range(F.row[0] + (int64_t)t * L.ns, s, kBlock, L.ns);
-        else if (t == 19) l2_prefetch_range(L.vox, s, kBlock, L.n & ~(int64_t)3);
+        else if (t == 19) l2_prefetch_range(WIN ? L.nodew : L.vox, s, kBlock, L.n & ~(int64_t)3);
     }
     if (i64 < L.n) {
         M d[19];
-        int nb[19];  // odd step: pore id of x - xi_q (the pull source of q), or a negative marker
         // 16-bit formats: every stored value is encoded with the reference of the
         // plane of the node that holds it (the even step writes its own slots; the
         // odd step encodes a scattered value with its destination's plane), so a
         // value read from the neighbour x - xi_q decodes with r(z - xi_z).
         M r_own = M(0), g = M(0);
         const uint32_t seed = step_seed<S>(bc, slot);
-        if constexpr (ODD) {
+        if constexpr (ODD && WIN) {
+            const uint32_t word = ld_aa_index(L.nodew + i, aa_index_policy());
+            r_own = own_ref_word<S>(bc, L, word);
+            g = own_slope<S>(bc);
+            d[0] = S::template dec<0>(F.row[0][i], r_own);
+            for_links(L.win, word, L.wy, L.wz, (uint32_t)i, [&](auto qc, bool pore, uint32_t id) {
+                constexpr int Q = decltype(qc)::value;
+                const uint32_t off =
+                    pore ? (uint32_t)opp(Q) * (uint32_t)L.ns + id : (uint32_t)Q * (uint32_t)L.ns + (uint32_t)i;
+                sid[Q - 1][threadIdx.x] = (int)off;
+                d[Q] = S::template dec<Q>(F.row[0][off], (S::kRef && pore) ? r_own - M(cz(Q)) * g : r_own);
+            });
+        } else if constexpr (ODD) {
             const uint64_t pol_idx = aa_index_policy();
             const uint32_t p = ld_aa_index(L.vox + i, pol_idx);
             r_own = own_ref<S>(bc, L, p);
@@ -602,35 +599,14 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
             d[0] = S::template dec<0>(F.row[0][i], r_own);
             for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
                 constexpr int Q = decltype(qc)::value + 1;
-                nb[Q] = ld_aa_index(L.grid + (uint32_t)(p + (uint32_t)L.goff[Q]), pol_idx);
-                if constexpr (kIds == 2 && !kOffs) sid[Q - 1][threadIdx.x] = nb[Q];
-                if constexpr (S::kRef) {
-                    // 16-bit (instruction-bound): one load and one decode, the
-                    // source slot and its plane selected
-                    const bool pore = nb[Q] >= 0;
-                    const typename S::T* src;
-                    if constexpr (OFF32) {  // one 32-bit element offset from row 0 (the rows are ns apart)
-                        const uint32_t off = pore ? (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)nb[Q]
-                                                  : (uint32_t)Q * (uint32_t)L.ns + (uint32_t)i;
-                        if constexpr (kOffs) sid[Q - 1][threadIdx.x] = (int)off;
-                        src = F.row[0] + off;
-                    } else {
-                        src = pore ? F.row[opp(Q)] + nb[Q] : F.row[Q] + i;
-                    }
-                    d[Q] = S::template dec<Q>(*src, pore ? r_own - M(cz(Q)) * g : r_own);
-                } else {
-                    if constexpr (OFF32) {
-                        const uint32_t off = nb[Q] >= 0 ? (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)nb[Q]
-                                                        : (uint32_t)Q * (uint32_t)L.ns + (uint32_t)i;
-                        if constexpr (kOffs) sid[Q - 1][threadIdx.x] = (int)off;
-                        d[Q] = F.row[0][off];
-                    } else {
-                        d[Q] = nb[Q] >= 0 ? F.row[opp(Q)][nb[Q]] : F.row[Q][i];
-                    }
-                }
+                const int id = ld_aa_index(L.grid + (uint32_t)(p + (uint32_t)L.goff[Q]), pol_idx);
+                sid[Q - 1][threadIdx.x] = id;
+                d[Q] = id >= 0 ? S::template dec<Q>(F.row[opp(Q)][id], r_own - M(cz(Q)) * g)
+                               : S::template dec<Q>(F.row[Q][i], r_own);
             });
         } else {
-            if constexpr (S::kRef) r_own = own_ref<S>(bc, L, __ldg(L.vox + i));
+            if constexpr (S::kRef)
+                r_own = L.nodew ? own_ref_word<S>(bc, L, __ldg(L.nodew + i)) : own_ref<S>(bc, L, __ldg(L.vox + i));
             for_q(AllQ{}, [&](auto qc) {
                 constexpr int Q = decltype(qc)::value;
                 d[Q] = S::template dec<Q>(F.row[Q][i], r_own);
@@ -647,76 +623,29 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
         // 19 64-bit addresses live across the collision
         int j;
         asm volatile("mov.b32 %0, %1;" : "=r"(j) : "r"(i));
-        if constexpr (ODD) {
-            // kIds == 1: fresh policy and voxel index, nothing of the gather stays live
-            const uint64_t pol_s = kIds == 1 ? aa_index_policy() : 0;
-            const uint32_t ps = kIds == 1 ? ld_aa_index(L.vox + j, pol_s) : 0u;
-            F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i, 0));
-            // x + xi_Q is the pull source of opp(Q)
-            auto dest = [&](auto qc) -> int {
-                constexpr int Q = decltype(qc)::value;
-                if constexpr (kIds == 1) return ld_aa_index(L.grid + (uint32_t)(ps + (uint32_t)L.goff[opp(Q)]), pol_s);
-                else if constexpr (kIds == 2) return sid[opp(Q) - 1][threadIdx.x];
-                else return nb[opp(Q)];
-            };
-            if constexpr (kOffs) {
-                // the destination of Q is the gather source of opp(Q), its offset
-                // staged by this thread; a pore destination lies in row Q, a
-                // bounce-back one in row opp(Q)
-                for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
-                    constexpr int Q = decltype(qc)::value + 1;
-                    const uint32_t off = (uint32_t)sid[opp(Q) - 1][threadIdx.x];
-                    if constexpr (S::kRef) {
-                        M r = r_own;
-                        if constexpr (cz(Q) != 0) {
-                            const bool pore = (Q & 1) ? off < (uint32_t)(Q + 1) * (uint32_t)L.ns
-                                                      : off >= (uint32_t)Q * (uint32_t)L.ns;
-                            r = pore ? r_own + M(cz(Q)) * g : r_own;
-                        }
-                        F.row[0][off] = S::template enc_sr<Q>(d[Q], r, sr_key<S>(seed, i, Q));
-                    } else {
-                        F.row[0][off] = d[Q];
-                    }
-                });
-            } else if constexpr (S::kRef && !LBM_AA16_PAIR_SCATTER) {
-                for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
-                    constexpr int Q = decltype(qc)::value + 1;
-                    const int dst = dest(qc_t<Q>{});
-                    const bool pore = dst >= 0;
-                    typename S::T* out;
-                    if constexpr (OFF32)
-                        out = F.row[0] + (pore ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)dst
-                                               : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)j);
-                    else
-                        out = pore ? F.row[Q] + dst : F.row[opp(Q)] + j;
-                    *out = S::template enc_sr<Q>(d[Q], pore ? r_own + M(cz(Q)) * g : r_own, sr_key<S>(seed, i, Q));
-                });
-            } else if constexpr (S::kRef) {
-                // 16-bit: per opposite pair one stochastic conversion; per value one
-                // store, destination slot and plane selected
-                for_q(std::make_integer_sequence<int, 9>{}, [&](auto pc) {
-                    constexpr int Q = 2 * decltype(pc)::value + 1;
-                    const int dq = dest(qc_t<Q>{});
-                    const int dq1 = dest(qc_t<Q + 1>{});
-                    const uint32_t h = S::template enc_sr2<Q>(d[Q], dq >= 0 ? r_own + M(cz(Q)) * g : r_own, d[Q + 1],
-                                                              dq1 >= 0 ? r_own - M(cz(Q)) * g : r_own,
-                                                              sr_key<S>(seed, i, Q), sr_key<S>(seed, i, Q + 1));
-                    *(dq >= 0 ? F.row[Q] + dq : F.row[Q + 1] + j) = S::half_of(h, true);
-                    *(dq1 >= 0 ? F.row[Q + 1] + dq1 : F.row[Q] + j) = S::half_of(h, false);
-                });
-            } else {  // FP32/FP64 store d directly; the branch form measured faster there
-                for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
-                    constexpr int Q = decltype(qc)::value + 1;
-                    const int dst = dest(qc_t<Q>{});
-                    if constexpr (OFF32) {
-                        F.row[0][dst >= 0 ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)dst
-                                          : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)j] = d[Q];
-                    } else {
-                        if (dst >= 0) F.row[Q][dst] = d[Q];
-                        else F.row[opp(Q)][j] = d[Q];
-                    }
-                });
-            }
+        if constexpr (ODD && WIN) {
+            F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i));
+            // a pore destination lies in row Q, a bounce-back one in row opp(Q)
+            for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
+                constexpr int Q = decltype(qc)::value + 1;
+                const uint32_t off = (uint32_t)sid[opp(Q) - 1][threadIdx.x];
+                M r = r_own;
+                if constexpr (S::kRef && cz(Q) != 0) {
+                    const bool pore = (Q & 1) ? off < (uint32_t)(Q + 1) * (uint32_t)L.ns
+                                              : off >= (uint32_t)Q * (uint32_t)L.ns;
+                    r = pore ? r_own + M(cz(Q)) * g : r_own;
+                }
+                F.row[0][off] = S::template enc_sr<Q>(d[Q], r, sr_key<S>(seed, i));
+            });
+        } else if constexpr (ODD) {
+            F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i));
+            for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
+                constexpr int Q = decltype(qc)::value + 1;
+                const int dst = sid[opp(Q) - 1][threadIdx.x];  // x + xi_Q is the pull source of opp(Q)
+                const uint32_t key = sr_key<S>(seed, i);
+                if (dst >= 0) F.row[Q][dst] = S::template enc_sr<Q>(d[Q], r_own + M(cz(Q)) * g, key);
+                else F.row[opp(Q)][j] = S::template enc_sr<Q>(d[Q], r_own, key);
+            });
         } else {
             encode_node<S>(d, seed, i, [&](auto) { return r_own; }, [&](auto qc, typename S::T v) {
                 constexpr int Q = decltype(qc)::value;
@@ -729,7 +658,7 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
             part = inlet_contribution<S>(L, L.vox[i], i, [&](auto qc) -> double {
                 constexpr int Q = decltype(qc)::value;
                 const M rq = (ODD && cz(Q) < 0) ? r_own - g : r_own;
-                return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], rq, sr_key<S>(seed, i, Q)), rq);
+                return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], rq, sr_key<S>(seed, i)), rq);
             });
         }
     }
@@ -1240,6 +1169,30 @@ __global__ void k_decode(const typename S::T* __restrict__ f, DevLattice L, cons
     });
 }
 
+// Row windows (lbm_device.cuh) of one padded box from its id grid, one thread per window.
+__global__ void k_windows(const int* __restrict__ grid, int sy, int rows, int nw, uint2* __restrict__ win) {
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= (int64_t)rows * nw) return;
+    const int64_t row = k / nw;
+    const int x0 = 30 * (int)(k - row * nw);
+    uint32_t bits = 0, first = 0;
+    for (int b = 31; b >= 0; --b) {  // a bit past the padded row stays 0
+        const int id = x0 + b < sy ? grid[row * sy + x0 + b] : SOLID;
+        if (id >= 0) {
+            bits |= 1u << b;
+            first = (uint32_t)id;
+        }
+    }
+    win[k] = make_uint2(bits, first);
+}
+__global__ void k_node_words(const uint32_t* __restrict__ vox, uint32_t vox0, int64_t n, int sy, int nw, uint32_t w0,
+                             uint32_t* __restrict__ nodew) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint32_t p = vox[i] - vox0, row = p / (uint32_t)sy, x = p - row * (uint32_t)sy, w = (x - 1u) / 30u;
+    nodew[i] = (w0 + row * (uint32_t)nw + w) << 5 | (x - 30u * w);
+}
+
 inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 template <class F>
@@ -1254,6 +1207,14 @@ cudaError_t dispatch(int prec, F&& f) {
 }
 
 }  // namespace
+
+cudaError_t launch_build_windows(const int* grid, const uint32_t* vox, uint32_t vox0, int64_t n, int nx, int ny,
+                                 int nz, uint32_t w0, uint2* win, uint32_t* nodew, cudaStream_t st) {
+    const int nw = windows_per_row(nx), rows = (ny + 2) * (nz + 2);
+    k_windows<<<blocks_for((int64_t)rows * nw, 256), 256, 0, st>>>(grid, nx + 2, rows, nw, win + w0);
+    if (n > 0) k_node_words<<<blocks_for(n, 256), 256, 0, st>>>(vox, vox0, n, nx + 2, nw, w0, nodew);
+    return cudaGetLastError();
+}
 
 int elem_size(int prec) { return prec == 0 ? 8 : prec == 1 ? 4 : 2; }
 int inlet_reduce_blocks(const DevLattice& L) { return (int)blocks_for(L.a_in, kReduceBlock); }
@@ -1281,8 +1242,8 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
             P.in[q] = (const T*)fin + (int64_t)q * L.ns;
             P.out[q] = (T*)fout + (int64_t)q * L.ns;
         }
-        // GB300_LBM_STEP_ADDR64 forces the 64-bit form (tests)
-        if (19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64"))
+        // GB300_LBM_STEP_ADDR64 forces the id-grid form with 64-bit addresses (tests)
+        if (L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64"))
             k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc,
                                                                          partials, counter);
         else
@@ -1406,10 +1367,10 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
         {
             AAPtrs<typename S::T> F;
             for (int q = 0; q < 19; ++q) F.row[q] = (typename S::T*)f + (int64_t)q * L.ns;
-            // every element offset of the buffer fits in 32 bits; the environment
-            // variable GB300_LBM_AA_ADDR64 forces the 64-bit form (for tests)
-            const bool off32 = 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_AA_ADDR64");
-            if (odd && off32)
+            // row windows, and every element offset of the buffer in 32 bits; the
+            // environment variable GB300_LBM_AA_ADDR64 forces the id-grid form (for tests)
+            const bool win = L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_AA_ADDR64");
+            if (odd && win)
                 k_step_aa<S, true, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(
                     F, slot, L, make_rates<M>(r.sp, r.sm), bc, partials, counter);
             else if (odd)
