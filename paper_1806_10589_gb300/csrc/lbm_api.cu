@@ -396,9 +396,8 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
     cudaError_t e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_vox, vox.data(), vox.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_grid, grid.data(), grid.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && windows) e = cudaMemset(c->d_nodew, 0, (size_t)c->L.ns * sizeof(uint32_t));
     if (e == cudaSuccess && windows)
-        e = lbm::launch_build_windows(c->d_grid, c->d_vox, 0u, n, nx, ny, nz, 0u, c->d_win, c->d_nodew, 0);
+        e = lbm::launch_build_windows(c->d_grid, c->d_vox, 0u, n, c->L.ns, nx, ny, nz, 0u, c->d_win, c->d_nodew, 0);
     if (e == cudaSuccess) e = cudaMemset(c->d_red_counter, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(c->d_step_counter, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(c->d_mon_counter, 0, sizeof(unsigned));

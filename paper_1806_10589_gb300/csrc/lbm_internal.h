@@ -31,11 +31,12 @@ struct DevLattice {
 
 inline int windows_per_row(int nx) { return (nx + 29) / 30; }
 // Fills the row windows of one padded box from its id grid (grid: first entry of
-// the box), and the words of its nodes from their padded voxel indices (counted
-// from the box's first entry plus `vox0`); `w0` is the index of the box's first
-// window.  The window index has to fit 27 bits.
-cudaError_t launch_build_windows(const int* grid, const uint32_t* vox, uint32_t vox0, int64_t n, int nx, int ny,
-                                 int nz, uint32_t w0, uint2* win, uint32_t* nodew, cudaStream_t st);
+// the box), and the words of its n nodes from their padded voxel indices (which
+// count from vox0); `w0` is the index of the box's first window, `win` the start
+// of all windows.  The n_pad - n slots after the nodes get a valid word too.
+// The window index has to fit 27 bits.
+cudaError_t launch_build_windows(const int* grid, const uint32_t* vox, uint32_t vox0, int64_t n, int64_t n_pad,
+                                 int nx, int ny, int nz, uint32_t w0, uint2* win, uint32_t* nodew, cudaStream_t st);
 
 struct Relax {
     double sp, sm;  // s+ and s- of the two-relaxation-time form

@@ -20,6 +20,7 @@
 
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
+#include "lbm_pair.cuh"
 
 namespace lbm {
 
@@ -480,16 +481,14 @@ struct AAPtrs {
 };
 
 // Resident blocks per SM the two AA kernels are compiled for (register caps).
-// The FP32 gather-scatter step measured best at 5 (48 registers): with the
-// gather offsets staged in shared memory it compiles there without spills, and
-// its launch took 0.1897 ms against 0.1970 ms at 4 (64 registers).  (With the
-// ids reloaded for the scatter, 4 was best with the L2 prefetch, 5 with spills
-// without it.)
+// On the 256^3 pack the FP32 gather-scatter step measured best at 5 (48 registers):
+// 171 us against 180 at 4 and 186 at 6; the node-local one at 5: 143.8 us against
+// 145.2 at 6 and 160.6 at 7.
 #ifndef LBM_AA_MIN_BLOCKS
 #define LBM_AA_MIN_BLOCKS 5
 #endif
 #ifndef LBM_AA_EVEN_MIN_BLOCKS
-#define LBM_AA_EVEN_MIN_BLOCKS 6
+#define LBM_AA_EVEN_MIN_BLOCKS 5
 #endif
 // LBM_AA_ID_HINT: 1 = the id grid is read with the L2 evict-last policy, 0 = plain.
 #ifndef LBM_AA_ID_HINT
@@ -628,7 +627,7 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
             // a pore destination lies in row Q, a bounce-back one in row opp(Q)
             for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
                 constexpr int Q = decltype(qc)::value + 1;
-                const uint32_t off = (uint32_t)sid[opp(Q) - 1][threadIdx.x];
+                const uint32_t off = *(volatile uint32_t*)&sid[opp(Q) - 1][threadIdx.x];
                 M r = r_own;
                 if constexpr (S::kRef && cz(Q) != 0) {
                     const bool pore = (Q & 1) ? off < (uint32_t)(Q + 1) * (uint32_t)L.ns
@@ -683,6 +682,286 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
             }
         }
     }
+}
+
+// ------------------------------------------- two nodes per thread (16-bit) ---
+// The 16-bit steps of k_step and k_step_aa with the slots i and i + 1 (i even) on
+// one thread: 128 threads per 256-node tile.  See lbm_pair.cuh for why.  A row
+// ends in padding (rows are multiples of 128 elements, and their node words name
+// an interior window), so the slot i + 1 of an odd last node exists; what is
+// written there is never read by another node.
+// Resident blocks per SM (register caps), measured on those packs: two-buffer step
+// 33.6, 33.1 and 34.0 us at 5, 6 and 7; gather-scatter 149, 144 and 148 us at 4, 5
+// and 6; node-local 77.6, 76.9 and 98 us at 6, 7 and 8, with the L2 prefetch 448
+// tiles ahead (86 us without, 79 at 224).  The staged offsets are read back through
+// a volatile pointer: otherwise the compiler keeps all 36 in registers (200 bytes
+// of spills, 195 us).
+constexpr int kPair = kBlock / 2;  // threads per tile
+#ifndef LBM_PAIR_STEP_BLOCKS
+#define LBM_PAIR_STEP_BLOCKS 6
+#endif
+#ifndef LBM_PAIR_ODD_BLOCKS
+#define LBM_PAIR_ODD_BLOCKS 5
+#endif
+#ifndef LBM_PAIR_EVEN_BLOCKS
+#define LBM_PAIR_EVEN_BLOCKS 7
+#endif
+#ifndef LBM_PAIR_EVEN_PREFETCH
+#define LBM_PAIR_EVEN_PREFETCH 448
+#endif
+
+// Inlet and outlet closures of the nodes i0 < i1 of a thread (both planes are rare).
+__device__ __forceinline__ void close_nodes(F2* d, int64_t i0, int64_t i1, const DevLattice& L, const BcState* bc,
+                                            int slot) {
+    if (i0 < L.a_in || i1 >= L.n - L.a_out) {
+        float a[2][19];
+#pragma unroll
+        for (int q = 0; q < 19; ++q) split(d[q], a[0][q], a[1][q]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int64_t i = k ? i1 : i0;
+            if (i < L.a_in) {
+                const float drin = bc->inlet_mode ? float(bc->drho_in_fixed) : float(bc->drho_in[slot]);
+                close_inlet(a[k], drin - inlet_known(a[k]));
+            } else if (i >= L.n - L.a_out) {
+                close_outlet(a[k], outlet_known(a[k]) - float(bc->drho_out));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 19; ++q) d[q] = f2(a[0][q], a[1][q]);
+    }
+}
+
+// Their part of the next inlet sum (see inlet_contribution); ref(k, Q): the
+// reference density that direction Q's value of node k is stored with.
+template <class S, class Ref>
+__device__ __forceinline__ double inlet_part_nodes(const F2* d, int64_t i0, int64_t i1, const DevLattice& L,
+                                                   uint32_t seed, Ref&& ref) {
+    double s = 0.0;
+    if (i0 >= L.a_01) return s;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int64_t i = k ? i1 : i0;
+        if (i < L.a_01) {
+            const uint32_t u = sr_key<S>(seed, i);
+            s += inlet_contribution<S>(L, L.vox[i], (int)i, [&](auto qc) -> double {
+                constexpr int Q = decltype(qc)::value;
+                float v[2];
+                split(d[Q], v[0], v[1]);
+                const float r = ref(k, qc);
+                return (double)S::template dec<Q>(S::template enc_sr<Q>(v[k], r, u), r);
+            });
+        }
+    }
+    return s;
+}
+
+// End of a step: the tile's part of the next inlet sum, the last tile writes the
+// next density (and the next rounding seed).
+template <class S, int NT>
+__device__ __forceinline__ void finish_inlet(double part, const DevLattice& L, BcState* bc, int slot,
+                                             double* __restrict__ partials, unsigned* __restrict__ counter, double* sh,
+                                             bool* last) {
+    const unsigned nb = (unsigned)((L.a_01 + kBlock - 1) / kBlock);
+    const double b = block_sum<NT>(part, sh);
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = b;
+        __threadfence();
+        *last = atomicAdd(counter, 1u) == nb - 1;
+    }
+    __syncthreads();
+    if (*last) {
+        __threadfence();
+        double s = 0.0;
+        for (unsigned j = threadIdx.x; j < nb; j += NT) s += __ldcg(partials + j);
+        s = block_sum<NT>(s, sh);
+        if (threadIdx.x == 0) {
+            bc->drho_in[slot ^ 1] = (bc->Q + s) / (double)L.a_in;
+            if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
+            *counter = 0u;
+        }
+    }
+}
+
+template <class S>
+__global__ void __launch_bounds__(kPair, LBM_PAIR_STEP_BLOCKS)
+k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float> rates, BcState* bc,
+            double* __restrict__ partials, unsigned* __restrict__ counter) {
+    using T = typename S::T;
+    __shared__ double sh[32];
+    __shared__ bool last;
+    {
+        const int64_t s = ((int64_t)blockIdx.x + LBM_STEP_PREFETCH) * kBlock;
+        const int t = (int)threadIdx.x;
+        if (t < 19) l2_prefetch_range(P.in[0] + (int64_t)t * L.ns, s, kBlock, L.ns);
+        else if (t == 19) l2_prefetch_range(L.nodew, s, kBlock, L.n & ~(int64_t)3);
+    }
+    const int64_t i64 = (int64_t)blockIdx.x * kBlock + 2 * threadIdx.x;
+    double part = 0.0;
+    if (i64 < L.n) {
+        const uint32_t i = (uint32_t)i64, ns = (uint32_t)L.ns;
+        const uint2 w = __ldg(reinterpret_cast<const uint2*>(L.nodew + i));
+        const float g = own_slope<S>(bc);
+        const float r0 = own_ref_word<S>(bc, L, w.x), r1 = own_ref_word<S>(bc, L, w.y);
+        const uint32_t seed = step_seed<S>(bc, slot);
+        F2 d[19];
+        {
+            float v[2][19];
+            split(dec2<S, 0>(widen2<S>(__ldg(reinterpret_cast<const uint32_t*>(P.in[0] + i))),
+                             f2(float(wq(0)) * r0, float(wq(0)) * r1)), v[0][0], v[1][0]);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float r = k ? r1 : r0;
+                const uint32_t ik = i + k;
+                for_links(L.win, k ? w.y : w.x, L.wy, L.wz, ik, [&](auto qc, bool pore, uint32_t id) {
+                    constexpr int Q = decltype(qc)::value;
+                    const uint32_t off = pore ? (uint32_t)Q * ns + id : (uint32_t)opp(Q) * ns + ik;
+                    v[k][Q] = S::template dec<Q>(__ldg(P.in[0] + off), (cz(Q) != 0 && pore) ? r - float(cz(Q)) * g : r);
+                });
+            }
+#pragma unroll
+            for (int q = 0; q < 19; ++q) d[q] = f2(v[0][q], v[1][q]);
+        }
+        close_nodes(d, i64, i64 + 1, L, bc, slot);
+        collide2<true>(d, rates.sp, rates.sm);
+        const F2 nr = f2(-1024.0f * r0, -1024.0f * r1);
+        const uint32_t u = sr_key2(seed, i, i + 1u);
+        for_q(AllQ{}, [&](auto qc) {
+            constexpr int Q = decltype(qc)::value;
+            *reinterpret_cast<uint32_t*>(P.out[Q] + i) = enc_sr2<S, Q>(d[Q], nr, u);
+        });
+        part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
+    }
+    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair>(part, L, bc, slot, partials, counter, sh, &last);
+}
+
+// Gather-scatter launch: thread t of a warp owns the nodes 64 w + t and
+// 64 w + 32 + t, so that a warp's 2-byte gathers and scatters of one node each
+// cover consecutive slots (with neighbouring nodes on a thread every store leaves
+// half of each sector to the next one: L2 throughput 65 % and the launch slower
+// than one node per thread).
+template <class S>
+__global__ void __launch_bounds__(kPair, LBM_PAIR_ODD_BLOCKS)
+k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float> rates, BcState* bc,
+              double* __restrict__ partials, unsigned* __restrict__ counter) {
+    __shared__ double sh[32];
+    __shared__ bool last;
+    // gather offsets: the scatter destination of q is the gather source of opp(q)
+    __shared__ uint32_t soff[2][18][kPair];
+    {
+        const int64_t s = ((int64_t)blockIdx.x + LBM_AA16_PREFETCH) * kBlock;
+        const int t = (int)threadIdx.x;
+        if (t < 19) l2_prefetch_range(f + (int64_t)t * L.ns, s, kBlock, L.ns);
+        else if (t == 19) l2_prefetch_range(L.nodew, s, kBlock, L.n & ~(int64_t)3);
+    }
+    const int64_t i64 = (int64_t)blockIdx.x * kBlock + 2 * (threadIdx.x & ~31u) + (threadIdx.x & 31u);
+    double part = 0.0;
+    if (i64 < L.n) {
+        const uint32_t ns = (uint32_t)L.ns;
+        const uint32_t i = (uint32_t)i64;
+        // an absent second node repeats the first one's reads and writes nothing
+        const bool two = i64 + 32 < L.n;
+        const uint32_t i1 = two ? i + 32u : i;
+        const uint32_t w0 = __ldg(L.nodew + i), w1 = __ldg(L.nodew + i1);
+        const float g = own_slope<S>(bc);
+        const float r0 = own_ref_word<S>(bc, L, w0), r1 = own_ref_word<S>(bc, L, w1);
+        const uint32_t seed = step_seed<S>(bc, slot);
+        F2 d[19];
+        {
+            float v[2][19];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float r = k ? r1 : r0;
+                const uint32_t ik = k ? i1 : i;
+                v[k][0] = S::template dec<0>(f[ik], r);
+                for_links(L.win, k ? w1 : w0, L.wy, L.wz, ik, [&](auto qc, bool pore, uint32_t id) {
+                    constexpr int Q = decltype(qc)::value;
+                    const uint32_t o = pore ? (uint32_t)opp(Q) * ns + id : (uint32_t)Q * ns + ik;
+                    soff[k][Q - 1][threadIdx.x] = o;
+                    v[k][Q] = S::template dec<Q>(f[o], (cz(Q) != 0 && pore) ? r - float(cz(Q)) * g : r);
+                });
+            }
+#pragma unroll
+            for (int q = 0; q < 19; ++q) d[q] = f2(v[0][q], v[1][q]);
+        }
+        close_nodes(d, i64, i64 + 32, L, bc, slot);
+        collide2<false>(d, rates.sp, rates.sm);
+        const float m0 = -1024.0f * r0, m1 = -1024.0f * r1;
+        const uint32_t u = sr_key2(seed, i, i + 32u);
+        {
+            const uint32_t h = enc_sr2<S, 0>(d[0], f2(m0, m1), u);
+            f[i] = S::half_of(h, false);
+            if (two) f[i1] = S::half_of(h, true);
+        }
+        // a value for a pore on another plane is encoded with that plane's reference
+        const float up0 = -1024.0f * (r0 + g), up1 = -1024.0f * (r1 + g);
+        const float dn0 = -1024.0f * (r0 - g), dn1 = -1024.0f * (r1 - g);
+        for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
+            constexpr int Q = decltype(qc)::value + 1;
+            const uint32_t o0 = *(volatile uint32_t*)&soff[0][opp(Q) - 1][threadIdx.x];
+            const uint32_t o1 = *(volatile uint32_t*)&soff[1][opp(Q) - 1][threadIdx.x];
+            F2 n = f2(m0, m1);
+            if constexpr (cz(Q) != 0) {
+                // a pore destination lies in row Q, a bounce-back one in row opp(Q)
+                const bool p0 = (Q & 1) ? o0 < (uint32_t)(Q + 1) * ns : o0 >= (uint32_t)Q * ns;
+                const bool p1 = (Q & 1) ? o1 < (uint32_t)(Q + 1) * ns : o1 >= (uint32_t)Q * ns;
+                n = f2(p0 ? (cz(Q) > 0 ? up0 : dn0) : m0, p1 ? (cz(Q) > 0 ? up1 : dn1) : m1);
+            }
+            const uint32_t h = enc_sr2<S, Q>(d[Q], n, u);
+            f[o0] = S::half_of(h, false);
+            if (two) f[o1] = S::half_of(h, true);
+        });
+        part = inlet_part_nodes<S>(d, i64, i64 + 32, L, seed, [&](int k, auto qc) {
+            const float r = k ? r1 : r0;
+            return cz(decltype(qc)::value) < 0 ? r - g : r;
+        });
+    }
+    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair>(part, L, bc, slot, partials, counter, sh, &last);
+}
+
+// Node-local launch: neighbouring nodes on a thread, one 4-byte load and store per row.
+template <class S>
+__global__ void __launch_bounds__(kPair, LBM_PAIR_EVEN_BLOCKS)
+k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<float> rates, BcState* bc,
+               double* __restrict__ partials, unsigned* __restrict__ counter) {
+    __shared__ double sh[32];
+    __shared__ bool last;
+    if constexpr (LBM_PAIR_EVEN_PREFETCH > 0) {
+        const int64_t s = ((int64_t)blockIdx.x + LBM_PAIR_EVEN_PREFETCH) * kBlock;
+        const int t = (int)threadIdx.x;
+        if (t < 19) l2_prefetch_range(F.row[0] + (int64_t)t * L.ns, s, kBlock, L.ns);
+        else if (t == 19) l2_prefetch_range(L.nodew, s, kBlock, L.n & ~(int64_t)3);
+    }
+    const int64_t i64 = (int64_t)blockIdx.x * kBlock + 2 * threadIdx.x;
+    double part = 0.0;
+    if (i64 < L.n) {
+        const uint32_t i = (uint32_t)i64;
+        uint32_t raw[19];
+        for_q(AllQ{}, [&](auto qc) {
+            constexpr int Q = decltype(qc)::value;
+            raw[Q] = *reinterpret_cast<const uint32_t*>(F.row[Q] + i);
+        });
+        const uint2 w = __ldg(reinterpret_cast<const uint2*>(L.nodew + i));
+        const float r0 = own_ref_word<S>(bc, L, w.x), r1 = own_ref_word<S>(bc, L, w.y);
+        const uint32_t seed = step_seed<S>(bc, slot);
+        F2 d[19];
+        for_q(AllQ{}, [&](auto qc) {
+            constexpr int Q = decltype(qc)::value;
+            d[Q] = dec2<S, Q>(widen2<S>(raw[Q]), f2(float(wq(Q)) * r0, float(wq(Q)) * r1));
+        });
+        close_nodes(d, i64, i64 + 1, L, bc, slot);
+        collide2<false>(d, rates.sp, rates.sm);
+        const F2 nr = f2(-1024.0f * r0, -1024.0f * r1);
+        const uint32_t u = sr_key2(seed, i, i + 1u);
+        uint32_t j;  // an opaque copy: the store addresses must not stay live from the loads
+        asm volatile("mov.b32 %0, %1;" : "=r"(j) : "r"(i));
+        for_q(AllQ{}, [&](auto qc) {
+            constexpr int Q = decltype(qc)::value;
+            *reinterpret_cast<uint32_t*>(F.row[opp(Q)] + j) = enc_sr2<S, Q>(d[Q], nr, u);
+        });
+        part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
+    }
+    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair>(part, L, bc, slot, partials, counter, sh, &last);
 }
 
 // Pull layout <-> layout S: swap F[q][x] and F[opp q][x] at every node.
@@ -1185,12 +1464,17 @@ __global__ void k_windows(const int* __restrict__ grid, int sy, int rows, int nw
     }
     win[k] = make_uint2(bits, first);
 }
-__global__ void k_node_words(const uint32_t* __restrict__ vox, uint32_t vox0, int64_t n, int sy, int nw, uint32_t w0,
-                             uint32_t* __restrict__ nodew) {
+// Words of n nodes; those of the padding slots up to n_pad name an interior window.
+__global__ void k_node_words(const uint32_t* __restrict__ vox, uint32_t vox0, int64_t n, int64_t n_pad, int sy, int nw,
+                             uint32_t w0, uint32_t w_pad, uint32_t* __restrict__ nodew) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t p = vox[i] - vox0, row = p / (uint32_t)sy, x = p - row * (uint32_t)sy, w = (x - 1u) / 30u;
-    nodew[i] = (w0 + row * (uint32_t)nw + w) << 5 | (x - 30u * w);
+    if (i >= n_pad) return;
+    uint32_t word = w_pad << 5 | 1u;
+    if (i < n) {
+        const uint32_t p = vox[i] - vox0, row = p / (uint32_t)sy, x = p - row * (uint32_t)sy, w = (x - 1u) / 30u;
+        word = (w0 + row * (uint32_t)nw + w) << 5 | (x - 30u * w);
+    }
+    nodew[i] = word;
 }
 
 inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -1208,11 +1492,12 @@ cudaError_t dispatch(int prec, F&& f) {
 
 }  // namespace
 
-cudaError_t launch_build_windows(const int* grid, const uint32_t* vox, uint32_t vox0, int64_t n, int nx, int ny,
-                                 int nz, uint32_t w0, uint2* win, uint32_t* nodew, cudaStream_t st) {
+cudaError_t launch_build_windows(const int* grid, const uint32_t* vox, uint32_t vox0, int64_t n, int64_t n_pad,
+                                 int nx, int ny, int nz, uint32_t w0, uint2* win, uint32_t* nodew, cudaStream_t st) {
     const int nw = windows_per_row(nx), rows = (ny + 2) * (nz + 2);
     k_windows<<<blocks_for((int64_t)rows * nw, 256), 256, 0, st>>>(grid, nx + 2, rows, nw, win + w0);
-    if (n > 0) k_node_words<<<blocks_for(n, 256), 256, 0, st>>>(vox, vox0, n, nx + 2, nw, w0, nodew);
+    const uint32_t w_pad = w0 + (uint32_t)nw * (uint32_t)(ny + 3);  // row y = 0 of plane z = 0
+    k_node_words<<<blocks_for(n_pad, 256), 256, 0, st>>>(vox, vox0, n, n_pad, nx + 2, nw, w0, w_pad, nodew);
     return cudaGetLastError();
 }
 
@@ -1244,9 +1529,14 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
         }
         // GB300_LBM_STEP_ADDR64 forces the id-grid form with 64-bit addresses (tests)
         if (L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64"))
-            k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc,
-                                                                         partials, counter);
-        else
+        {
+            if constexpr (S::kRef)
+                k_step_pair<S><<<blocks_for(L.n, kBlock), kPair, 0, st>>>(P, slot, L, make_rates<float>(r.sp, r.sm), bc,
+                                                                          partials, counter);
+            else
+                k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc,
+                                                                             partials, counter);
+        } else
             k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials,
                                                                    counter);
         return cudaGetLastError();
@@ -1370,15 +1660,22 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
             // row windows, and every element offset of the buffer in 32 bits; the
             // environment variable GB300_LBM_AA_ADDR64 forces the id-grid form (for tests)
             const bool win = L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_AA_ADDR64");
-            if (odd && win)
-                k_step_aa<S, true, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(
-                    F, slot, L, make_rates<M>(r.sp, r.sm), bc, partials, counter);
-            else if (odd)
-                k_step_aa<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(F, slot, L, make_rates<M>(r.sp, r.sm), bc,
-                                                                                partials, counter);
-            else
-                k_step_aa<S, false><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(F, slot, L, make_rates<M>(r.sp, r.sm), bc,
-                                                                                 partials, counter);
+            const unsigned nb = blocks_for(L.n, kBlock);
+            const auto rates = make_rates<M>(r.sp, r.sm);
+            if constexpr (S::kRef) {
+                if (win) {
+                    if (odd)
+                        k_aa_odd_pair<S><<<nb, kPair, 0, st>>>((typename S::T*)f, slot, L, rates, bc, partials, counter);
+                    else
+                        k_aa_even_pair<S><<<nb, kPair, 0, st>>>(F, slot, L, rates, bc, partials, counter);
+                    return cudaGetLastError();
+                }
+            } else if (odd && win) {
+                k_step_aa<S, true, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials, counter);
+                return cudaGetLastError();
+            }
+            if (odd) k_step_aa<S, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials, counter);
+            else k_step_aa<S, false><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials, counter);
             return cudaGetLastError();
         }
     });

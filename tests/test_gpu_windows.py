@@ -2,6 +2,8 @@
 
 Both forms read the same values into the same arithmetic, so the states are
 bitwise equal.  Widths around multiples of 30 put runs across window borders.
+The 16-bit formats also compare two nodes per thread (windows) with one (id
+grid): odd node counts, one to several 256-node tiles.
 """
 import numpy as np
 import pytest
