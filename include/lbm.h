@@ -263,7 +263,9 @@ int lbm_batch_time_step(lbm_batch* b, int n, float* ms);
  *     graph, with in-place layout swaps around each call.  Both buffers stay
  *     allocated.
  *   *_CAPPED: the same launch compiled for 5 resident 256-thread blocks per SM
- *     (48 registers) instead of 4 (64 registers).  There is no cap for FP64.
+ *     (48 registers) instead of 4 (64 registers).  There is no cap for FP64.  The
+ *     16-bit per-step launches advance two nodes per thread: 6 resident 128-thread
+ *     blocks (80 registers) instead of 5 (96 registers).
  * lbm_batch_set_config selects a configuration.  lbm_batch_autotune measures
  * them for you.  For every configuration it runs trial_steps steps untimed, then
  * trial_steps timed steps, restoring the state after each run.  The restore uses

@@ -30,6 +30,7 @@
 #include "../../include/lbm.h"
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
+#include "lbm_pair.cuh"
 
 namespace lbm {
 namespace {
@@ -49,6 +50,9 @@ struct Member {
     uint64_t sz_magic;  // ceil(2^64 / ((nx+2)(ny+2)))
     int nz;
     int goff[19];       // padded-grid offsets of the pull sources
+    uint32_t w0;        // first row window of the member (lbm_device.cuh)
+    int wy, wz;         // window strides of y and z
+    uint64_t wz_magic;  // ceil(2^64 / wz)
     double Q;           // prescribed inlet flux
     double drho_out;    // outlet density - 1
     double drho_in[2];  // inlet density - 1 for the step reading buffer c
@@ -83,7 +87,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     __syncthreads();
     double r = 0.0;
     if (wid == 0) {
-        r = lane < kTile / 32 ? sh[lane] : 0.0;
+        r = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
         r = warp_sum(r);
     }
     __syncthreads();
@@ -95,6 +99,17 @@ __device__ __forceinline__ typename S::M member_ref(const Member& m, int64_t p_g
     using M = typename S::M;
     if constexpr (S::kRef) {
         const int z = plane_of((uint64_t)(p_global - m.grid_base), m.sz_magic);
+        const int c = m.ref_cur;
+        return M(m.ref_r0[c]) + M(m.ref_g[c]) * M(z);
+    } else {
+        return M(0);
+    }
+}
+template <class S>
+__device__ __forceinline__ typename S::M member_ref_word(const Member& m, uint32_t word) {
+    using M = typename S::M;
+    if constexpr (S::kRef) {
+        const int z = plane_of((uint64_t)((word >> 5) - m.w0), m.wz_magic);
         const int c = m.ref_cur;
         return M(m.ref_r0[c]) + M(m.ref_g[c]) * M(z);
     } else {
@@ -125,11 +140,7 @@ __device__ __forceinline__ T ld_state(const T* p) {
     }
 }
 
-// OFF32 (per-step launches, ensembles of 19 ns < 2^32 elements): the source is
-// fin plus one 32-bit element offset, its row chosen by a 32-bit select, rather
-// than one of two 64-bit addresses.  Measured on the 64-pack FP16-dev ensemble:
-// the step 0.981 against 1.141 ms (48-register cap), and no spills at that cap.
-template <class S, int Q, bool COH = false, bool OFF32 = false>
+template <class S, int Q, bool COH = false>
 __device__ __forceinline__ typename S::M pull_b(const typename S::T* fin, int64_t ns,
                                                 const int* __restrict__ grid, const Member& m,
                                                 int64_t p, int64_t i, typename S::M r_own,
@@ -137,15 +148,8 @@ __device__ __forceinline__ typename S::M pull_b(const typename S::T* fin, int64_
     using M = typename S::M;
     if (Q == 0) return S::template dec<0>(ld_state<COH>(fin + i), r_own);
     const int id = __ldg(grid + p + m.goff[Q]);
-    if constexpr (OFF32) {
-        const bool pore = id >= 0;
-        const uint32_t off =
-            pore ? (uint32_t)Q * (uint32_t)ns + (uint32_t)id : (uint32_t)opp(Q) * (uint32_t)ns + (uint32_t)i;
-        return S::template dec<Q>(ld_state<COH>(fin + off), pore ? r_own - M(cz(Q)) * g : r_own);
-    } else {
-        if (id >= 0) return S::template dec<Q>(ld_state<COH>(fin + (int64_t)Q * ns + id), r_own - M(cz(Q)) * g);
-        return S::template dec<Q>(ld_state<COH>(fin + (int64_t)opp(Q) * ns + i), r_own);
-    }
+    if (id >= 0) return S::template dec<Q>(ld_state<COH>(fin + (int64_t)Q * ns + id), r_own - M(cz(Q)) * g);
+    return S::template dec<Q>(ld_state<COH>(fin + (int64_t)opp(Q) * ns + i), r_own);
 }
 
 // Same contribution rule as the single-lattice step (see lbm_kernels.cu).
@@ -189,7 +193,7 @@ __device__ __forceinline__ void member_reduce(double part, int64_t tile, int64_t
     if (last) {
         __threadfence();
         double s = 0.0;
-        for (int64_t j = threadIdx.x; j < ntm; j += kTile) s += __ldcg(partials + tile0 + j);
+        for (int64_t j = threadIdx.x; j < ntm; j += blockDim.x) s += __ldcg(partials + tile0 + j);
         s = block_sum(s, sh);
         if (threadIdx.x == 0) {
             finish(s);
@@ -198,30 +202,62 @@ __device__ __forceinline__ void member_reduce(double part, int64_t tile, int64_t
     }
 }
 
+// Where a member finds its neighbours: the padded voxel list and id grid, or the
+// row windows and node words (per-step launches of ensembles of 19 ns < 2^32
+// elements: every source is then fin plus one 32-bit element offset).
+struct Links {
+    const uint32_t* vox;
+    const int* grid;
+    const uint2* win;
+    const uint32_t* nodew;
+};
+
+// End of a tile: its part of the member's next inlet density (the member's last
+// tile finishes).
+template <class S, bool COH>
+__device__ __forceinline__ void batch_finish(double part, int slot, int64_t tile, int mi, Member* members,
+                                             double* partials, unsigned* counters, double* sh) {
+    const Member& m = members[mi];
+    const int64_t tile0 = m.base / kTile, nt01 = (m.a_01 + kTile - 1) / kTile;
+    if (tile - tile0 < nt01)
+        member_reduce(part, tile, tile0, nt01, partials, counters + mi, sh, [&](double s) {
+            members[mi].drho_in[slot ^ 1] = (m.Q + s) / (double)m.a_in;
+            if constexpr (S::kRef) members[mi].sr_seed[slot ^ 1] = sr_next(ld_state<COH>(&m.sr_seed[slot]));
+        });
+}
+
 // One 256-node tile of one step: the single-lattice step with the member's own
-// boundary scalars, and the member's next inlet density (last tile finishes).
-template <class S, bool COH, bool OFF32 = false>
+// boundary scalars, and the member's next inlet density.
+template <class S, bool COH, bool WIN = false>
 __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typename S::T* fout, int64_t ns, int slot,
-                                                int64_t tile, const uint32_t* __restrict__ vox,
-                                                const int* __restrict__ grid, const int* __restrict__ tile_member,
-                                                Member* members, Rates<typename S::M> rates,
-                                                double* partials, unsigned* counters, double* sh) {
+                                                int64_t tile, const Links& K, const int* __restrict__ tile_member,
+                                                Member* members, const Rates<typename S::M>& rates, double* partials,
+                                                unsigned* counters, double* sh) {
     using M = typename S::M;
     const int mi = tile_member[tile];
     const Member& m = members[mi];
-    const int64_t tile0 = m.base / kTile;
     const int64_t i = tile * kTile + threadIdx.x;
     const int64_t il = i - m.base;
     double part = 0.0;
     if (il < m.n) {
-        const int64_t p = vox[i];
-        const M r_own = member_ref<S>(m, p), g = member_slope<S>(m);
+        const uint32_t p = WIN ? __ldg(K.nodew + i) : K.vox[i];  // node word or padded voxel
+        const M r_own = WIN ? member_ref_word<S>(m, p) : member_ref<S>(m, p), g = member_slope<S>(m);
         const uint32_t seed = S::kRef ? ld_state<COH>(&m.sr_seed[slot]) : 0u;
         M d[19];
-        for_q(AllQ{}, [&](auto qc) {
-            constexpr int Q = decltype(qc)::value;
-            d[Q] = pull_b<S, Q, COH, OFF32>(fin, ns, grid, m, p, i, r_own, g);
-        });
+        if constexpr (WIN) {
+            d[0] = S::template dec<0>(fin[i], r_own);
+            for_links(K.win, p, m.wy, m.wz, (uint32_t)i, [&](auto qc, bool pore, uint32_t id) {
+                constexpr int Q = decltype(qc)::value;
+                const uint32_t off =
+                    pore ? (uint32_t)Q * (uint32_t)ns + id : (uint32_t)opp(Q) * (uint32_t)ns + (uint32_t)i;
+                d[Q] = S::template dec<Q>(fin[off], (cz(Q) != 0 && pore) ? r_own - M(cz(Q)) * g : r_own);
+            });
+        } else {
+            for_q(AllQ{}, [&](auto qc) {
+                constexpr int Q = decltype(qc)::value;
+                d[Q] = pull_b<S, Q, COH>(fin, ns, K.grid, m, p, i, r_own, g);
+            });
+        }
         if (il < m.a_in) {
             close_inlet(d, M(ld_state<COH>(&m.drho_in[slot])) - inlet_known(d));
         } else if (il >= m.n - m.a_out) {
@@ -232,14 +268,9 @@ __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typena
             constexpr int Q = decltype(qc)::value;
             fout[(int64_t)Q * ns + i] = v;
         });
-        if (il < m.a_01) part = next_inlet_part_b<S>(d, grid, m, p, il, r_own, seed, i);
+        if (il < m.a_01) part = next_inlet_part_b<S>(d, K.grid, m, K.vox[i], il, r_own, seed, i);
     }
-    const int64_t nt01 = (m.a_01 + kTile - 1) / kTile;
-    if (tile - tile0 < nt01)
-        member_reduce(part, tile, tile0, nt01, partials, counters + mi, sh, [&](double s) {
-            members[mi].drho_in[slot ^ 1] = (m.Q + s) / (double)m.a_in;
-            if constexpr (S::kRef) members[mi].sr_seed[slot ^ 1] = sr_next(ld_state<COH>(&m.sr_seed[slot]));
-        });
+    batch_finish<S, COH>(part, slot, tile, mi, members, partials, counters, sh);
 }
 
 // LBM_BATCH_PREFETCH: the per-step and gather-scatter AA kernels ask L2 for the
@@ -271,16 +302,80 @@ constexpr int batch_min_blocks() {
 }
 
 // One step, one tile per block.
-template <class S, int MINB, bool OFF32 = false>
+template <class S, int MINB, bool WIN = false>
 __global__ void __launch_bounds__(kTile, batch_min_blocks<S, MINB>())
-k_batch_step(const typename S::T* __restrict__ fin, typename S::T* __restrict__ fout, int64_t ns, int slot,
-             const uint32_t* __restrict__ vox, const int* __restrict__ grid, const int* __restrict__ tile_member,
-             Member* members, Rates<typename S::M> rates, double* __restrict__ partials,
-             unsigned* __restrict__ counters) {
+k_batch_step(const typename S::T* __restrict__ fin, typename S::T* __restrict__ fout, int64_t ns, int slot, Links K,
+             const int* __restrict__ tile_member, Member* members, Rates<typename S::M> rates,
+             double* __restrict__ partials, unsigned* __restrict__ counters) {
     __shared__ double sh[32];
-    batch_prefetch(fin, ns, vox);
-    batch_tile_step<S, false, OFF32>(fin, fout, ns, slot, blockIdx.x, vox, grid, tile_member, members, rates,
-                                     partials, counters, sh);
+    batch_prefetch(fin, ns, WIN ? K.nodew : K.vox);
+    batch_tile_step<S, false, WIN>(fin, fout, ns, slot, blockIdx.x, K, tile_member, members, rates, partials,
+                                   counters, sh);
+}
+
+// The 16-bit step with the slots i and i + 1 (i even) on one thread, 128 threads
+// per tile (lbm_pair.cuh).  A member's slots are padded to whole tiles, so an odd
+// last node has a slot after it that no other node reads.  Measured on six
+// FP16-dev packs with edges 64..160 (3.1 M pores), row windows and two nodes per
+// thread against the id grid and one: 79.9 -> 63.8 us per step.
+template <class S, int MINB>
+__global__ void __launch_bounds__(kTile / 2, MINB)
+k_batch_pair(const typename S::T* __restrict__ fin, typename S::T* __restrict__ fout, int64_t ns, int slot, Links K,
+             const int* __restrict__ tile_member, Member* members, Rates<float> rates,
+             double* __restrict__ partials, unsigned* __restrict__ counters) {
+    __shared__ double sh[32];
+    batch_prefetch(fin, ns, K.nodew);
+    const int64_t tile = blockIdx.x;
+    const int mi = tile_member[tile];
+    const Member& m = members[mi];
+    const int64_t i64 = tile * kTile + 2 * threadIdx.x, il = i64 - m.base;
+    double part = 0.0;
+    if (il < m.n) {
+        const uint32_t i = (uint32_t)i64, ns32 = (uint32_t)ns;
+        const uint2 w = __ldg(reinterpret_cast<const uint2*>(K.nodew + i));
+        const float g = member_slope<S>(m);
+        const float r0 = member_ref_word<S>(m, w.x), r1 = member_ref_word<S>(m, w.y);
+        const uint32_t seed = m.sr_seed[slot];
+        float v[2][19];
+        split(dec2<S, 0>(widen2<S>(__ldg(reinterpret_cast<const uint32_t*>(fin + i))),
+                         f2(float(wq(0)) * r0, float(wq(0)) * r1)), v[0][0], v[1][0]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float r = k ? r1 : r0;
+            const uint32_t ik = i + k;
+            for_links(K.win, k ? w.y : w.x, m.wy, m.wz, ik, [&](auto qc, bool pore, uint32_t id) {
+                constexpr int Q = decltype(qc)::value;
+                const uint32_t off = pore ? (uint32_t)Q * ns32 + id : (uint32_t)opp(Q) * ns32 + ik;
+                v[k][Q] = S::template dec<Q>(__ldg(fin + off), (cz(Q) != 0 && pore) ? r - float(cz(Q)) * g : r);
+            });
+        }
+        if (il < m.a_in || il + 1 >= m.n - m.a_out) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (il + k < m.a_in) close_inlet(v[k], float(m.drho_in[slot]) - inlet_known(v[k]));
+                else if (il + k >= m.n - m.a_out) close_outlet(v[k], outlet_known(v[k]) - float(m.drho_out));
+            }
+        }
+        F2 d[19];
+#pragma unroll
+        for (int q = 0; q < 19; ++q) d[q] = f2(v[0][q], v[1][q]);
+        collide2<true>(d, rates.sp, rates.sm);
+        const F2 nr = f2(-1024.0f * r0, -1024.0f * r1);
+        const uint32_t u = sr_key2(seed, i, i + 1u);
+        for_q(AllQ{}, [&](auto qc) {
+            constexpr int Q = decltype(qc)::value;
+            *reinterpret_cast<uint32_t*>(fout + (int64_t)Q * ns + i) = enc_sr2<S, Q>(d[Q], nr, u);
+        });
+        if (il < m.a_01) {
+#pragma unroll
+            for (int q = 0; q < 19; ++q) split(d[q], v[0][q], v[1][q]);
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (il + k < m.a_01)
+                    part += next_inlet_part_b<S>(v[k], K.grid, m, K.vox[i64 + k], il + k, k ? r1 : r0, seed, i64 + k);
+        }
+    }
+    batch_finish<S, false>(part, slot, tile, mi, members, partials, counters, sh);
 }
 
 // Grid barrier of the persistent launch.  Thread 0 of every block arrives on a
@@ -331,8 +426,7 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier* bar, unsigned nblocks,
 // slot0 ^ (s & 1).
 template <class S, int MINB>
 __global__ void __launch_bounds__(kTile, batch_min_blocks<S, MINB>())
-k_batch_persistent(typename S::T* f0, typename S::T* f1, int64_t ns, int slot0, int nsteps, int64_t ntiles,
-                   const uint32_t* __restrict__ vox, const int* __restrict__ grid,
+k_batch_persistent(typename S::T* f0, typename S::T* f1, int64_t ns, int slot0, int nsteps, int64_t ntiles, Links K,
                    const int* __restrict__ tile_member, Member* members, Rates<typename S::M> rates,
                    double* partials, unsigned* counters, GridBarrier* bar, long long limit) {
     __shared__ double sh[32];
@@ -343,8 +437,7 @@ k_batch_persistent(typename S::T* f0, typename S::T* f1, int64_t ns, int slot0, 
         const typename S::T* fin = slot ? f1 : f0;
         typename S::T* fout = slot ? f0 : f1;
         for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-            batch_tile_step<S, true>(fin, fout, ns, slot, tile, vox, grid, tile_member, members, rates, partials,
-                                     counters, sh);
+            batch_tile_step<S, true>(fin, fout, ns, slot, tile, K, tile_member, members, rates, partials, counters, sh);
         if (!grid_barrier(bar, gridDim.x, gen, limit)) return;
     }
 }
@@ -772,6 +865,8 @@ struct lbm_batch {
     int cur = 0;
     uint32_t* d_vox = nullptr;
     int* d_grid = nullptr;
+    uint2* d_win = nullptr;        // row windows and node words (null: an index needs more than 27 bits)
+    uint32_t* d_nodew = nullptr;
     int* d_tile_member = nullptr;
     lbm::Member* d_members = nullptr;
     double* d_partials = nullptr;
@@ -830,6 +925,8 @@ void brelease(lbm_batch* b) {
         if (p) cudaFree(p);
     cudaFree(b->d_vox);
     cudaFree(b->d_grid);
+    cudaFree(b->d_win);
+    cudaFree(b->d_nodew);
     cudaFree(b->d_tile_member);
     cudaFree(b->d_members);
     cudaFree(b->d_partials);
@@ -839,6 +936,8 @@ void brelease(lbm_batch* b) {
     cudaFree(b->d_bar);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
 }
+
+lbm::Links blinks(const lbm_batch* b) { return lbm::Links{b->d_vox, b->d_grid, b->d_win, b->d_nodew}; }
 
 // Register cap of a configuration: 4 or 5 resident 256-thread blocks per SM
 // (64 or 48 registers).
@@ -884,7 +983,8 @@ int bpersistent(lbm_batch* b, int nsteps) {
             int slot0 = b->cur, n = nsteps;
             auto rates = lbm::make_rates<M>(b->sp, b->sm);
             long long limit = kBarrierLimit;
-            void* args[] = {&f0, &f1, &ns, &slot0, &n, &ntiles, &b->d_vox, &b->d_grid, &b->d_tile_member,
+            lbm::Links K = blinks(b);
+            void* args[] = {&f0, &f1, &ns, &slot0, &n, &ntiles, &K, &b->d_tile_member,
                             &b->d_members, &rates, &b->d_partials, &b->d_counters, &b->d_bar, &limit};
             return cudaLaunchCooperativeKernel((const void*)lbm::k_batch_persistent<S, MINB>, dim3(grid),
                                                dim3(lbm::kTile), args, 0, b->stream);
@@ -912,17 +1012,24 @@ int bstep_once(lbm_batch* b, cudaStream_t st) {
         using S = decltype(s);
         using T = typename S::T;
         using M = typename S::M;
-        auto launch = [&](auto kernel) {
-            kernel<<<(unsigned)b->ntiles, lbm::kTile, 0, st>>>(
-                (const T*)b->f[b->cur], (T*)b->f[b->cur ^ 1], b->ns, b->cur, b->d_vox, b->d_grid,
-                b->d_tile_member, b->d_members, lbm::make_rates<M>(b->sp, b->sm), b->d_partials, b->d_counters);
+        auto launch = [&](auto kernel, int threads) {
+            kernel<<<(unsigned)b->ntiles, threads, 0, st>>>((const T*)b->f[b->cur], (T*)b->f[b->cur ^ 1], b->ns, b->cur,
+                                                            blinks(b), b->d_tile_member, b->d_members,
+                                                            lbm::make_rates<M>(b->sp, b->sm), b->d_partials,
+                                                            b->d_counters);
         };
-        // every element offset of a buffer fits in 32 bits; GB300_LBM_BATCH_ADDR64 forces the 64-bit form (tests)
-        const bool off32 = 19 * (uint64_t)b->ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_BATCH_ADDR64");
-        if (cfg_capped(b->config))
-            off32 ? launch(lbm::k_batch_step<S, 5, true>) : launch(lbm::k_batch_step<S, 5>);
-        else
-            off32 ? launch(lbm::k_batch_step<S, 4, true>) : launch(lbm::k_batch_step<S, 4>);
+        // row windows, and every element offset of a buffer in 32 bits;
+        // GB300_LBM_BATCH_ADDR64 forces the id-grid form (tests)
+        const bool win = b->d_win && 19 * (uint64_t)b->ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_BATCH_ADDR64");
+        const bool capped = cfg_capped(b->config);
+        if (win) {
+            if constexpr (S::kRef)
+                capped ? launch(lbm::k_batch_pair<S, 6>, lbm::kTile / 2) : launch(lbm::k_batch_pair<S, 5>, lbm::kTile / 2);
+            else
+                capped ? launch(lbm::k_batch_step<S, 5, true>, lbm::kTile) : launch(lbm::k_batch_step<S, 4, true>, lbm::kTile);
+        } else {
+            capped ? launch(lbm::k_batch_step<S, 5>, lbm::kTile) : launch(lbm::k_batch_step<S, 4>, lbm::kTile);
+        }
         return cudaGetLastError();
     });
     BATCH_CUDA(b, e);
@@ -1075,7 +1182,7 @@ int lbm_batch_create(int n_members, const uint8_t* const* masks, const int* dims
     std::vector<int> grid;
     std::vector<uint32_t> vox;
     std::vector<int> tile_member;
-    int64_t base = 0, gbase = 0;
+    int64_t base = 0, gbase = 0, wbase = 0;
     for (int mi = 0; mi < n_members; ++mi) {
         const int nx = dims[3 * mi], ny = dims[3 * mi + 1], nz = dims[3 * mi + 2];
         const uint8_t* mask = masks[mi];
@@ -1130,6 +1237,12 @@ int lbm_batch_create(int n_members, const uint8_t* const* masks, const int* dims
         const unsigned __int128 two64 = (unsigned __int128)1 << 64;
         const unsigned __int128 szq = (unsigned __int128)(uint64_t)(px * py);
         m.sz_magic = (uint64_t)(two64 / szq + (two64 % szq != 0 ? 1 : 0));
+        m.w0 = (uint32_t)wbase;
+        m.wy = lbm::windows_per_row(nx);
+        m.wz = m.wy * (int)py;
+        const unsigned __int128 wzq = (unsigned __int128)(uint64_t)m.wz;
+        m.wz_magic = (uint64_t)(two64 / wzq + (two64 % wzq != 0 ? 1 : 0));
+        wbase += (int64_t)m.wz * pz;
         b->h_members[(size_t)mi] = m;
         const int64_t nt = (n + lbm::kTile - 1) / lbm::kTile;
         for (int64_t t = 0; t < nt; ++t) tile_member.push_back(mi);
@@ -1153,6 +1266,11 @@ int lbm_batch_create(int n_members, const uint8_t* const* masks, const int* dims
     A(&b->f[1], fbytes);
     A(&b->d_vox, vox.size() * 4);
     A(&b->d_grid, grid.size() * 4);
+    const bool windows = wbase < (int64_t)1 << 27;
+    if (windows) {
+        A(&b->d_win, (size_t)wbase * sizeof(uint2));
+        A(&b->d_nodew, (size_t)base * sizeof(uint32_t));
+    }
     A(&b->d_tile_member, tile_member.size() * 4);
     A(&b->d_members, (size_t)n_members * sizeof(lbm::Member));
     A(&b->d_partials, (size_t)b->ntiles * sizeof(double));
@@ -1163,6 +1281,12 @@ int lbm_batch_create(int n_members, const uint8_t* const* masks, const int* dims
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_vox, vox.data(), vox.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_grid, grid.data(), grid.size() * 4, cudaMemcpyHostToDevice);
+    for (int mi = 0; mi < n_members && windows && e == cudaSuccess; ++mi) {
+        const lbm::Member& m = b->h_members[(size_t)mi];
+        e = lbm::launch_build_windows(b->d_grid + m.grid_base, b->d_vox + m.base, (uint32_t)m.grid_base, m.n,
+                                      (m.n + lbm::kTile - 1) / lbm::kTile * lbm::kTile, dims[3 * mi], dims[3 * mi + 1],
+                                      dims[3 * mi + 2], m.w0, b->d_win, b->d_nodew + m.base, 0);
+    }
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_tile_member, tile_member.data(), tile_member.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
