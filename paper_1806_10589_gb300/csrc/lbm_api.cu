@@ -369,8 +369,8 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
     // ---- device memory
     int rc = LBM_OK;
     const size_t fbytes = (size_t)19 * (size_t)c->L.ns * (size_t)lbm::elem_size(precision);
-    // per-tile partials of the inlet reductions (tiles of >= 128 nodes)
-    const int nb_red = std::max(lbm::inlet_reduce_blocks(c->L), (int)((a_01 + 127) / 128));
+    // partial sums of the inlet reductions: one per 32 nodes of whole 256-node tiles
+    const int nb_red = std::max(lbm::inlet_reduce_blocks(c->L), (int)((a_01 + 255) / 256 * 8));
     const int nb_mon = lbm::monitor_blocks(c->L);
     if ((rc = dev_alloc(c, &c->f[0], fbytes)) || (rc = dev_alloc(c, &c->f[1], fbytes)) ||
         (rc = dev_alloc(c, &c->d_vox, vox.size() * sizeof(uint32_t))) ||

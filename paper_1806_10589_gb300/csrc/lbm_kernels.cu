@@ -324,32 +324,60 @@ k_inlet_reduce(const typename S::T* __restrict__ fin, int slot, DevLattice L, Bc
 //   z = 1:  twice each xi_z = -1 value whose destination on z = 0 is a pore.
 // `val(Q)` returns the stored value of direction Q exactly as the next step
 // will decode it.
+//   FP32 values are added without error in three FP32 words (two chained two-sums,
+// Knuth's) and reach FP64 once per node: a conversion and an FP64 addition per
+// value, at two FP64 operations per clock and SM, made the inlet tiles the tail of
+// every step of a small lattice (61x67x72, 112 k nodes: 9.1 -> 8.0 us per step).
+struct SumF32 {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    __device__ __forceinline__ static void two_sum(float& s, float x, float& err) {
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+        s = t;
+    }
+    __device__ __forceinline__ void add(float x) {
+        float e, f;
+        two_sum(hi, x, e);
+        two_sum(mid, e, f);
+        lo = __fadd_rn(lo, f);
+    }
+    // an infinite or NaN sum has no error terms
+    __device__ __forceinline__ double value() const {
+        return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
+    }
+};
+struct SumF64 {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ double value() const { return s; }
+};
 template <class S, class V>
 __device__ __forceinline__ double inlet_contribution(const DevLattice& L, uint32_t p, int i, V&& val) {
-    double s = 0.0;
+    using M = typename S::M;
+    std::conditional_t<sizeof(M) == 8, SumF64, SumF32> s;
     auto dest_is_pore = [&](auto qc) -> bool {
         constexpr int Q = decltype(qc)::value;  // destination i + xi_Q = pull source of opp(Q)
         return __ldg(L.grid + (uint32_t)(p + (uint32_t)L.goff[opp(Q)])) >= 0;
     };
     if (i < L.a_in) {
         for_q(std::integer_sequence<int, 0, 1, 2, 3, 4, 7, 8, 9, 10>{},
-              [&](auto qc) { s += val(qc); });
+              [&](auto qc) { s.add(val(qc)); });
         for_q(std::integer_sequence<int, 5, 11, 14, 15, 18>{},
-              [&](auto qc) { if (!dest_is_pore(qc)) s += 2.0 * val(qc); });
+              [&](auto qc) { if (!dest_is_pore(qc)) s.add(M(2) * val(qc)); });
     } else {
         for_q(std::integer_sequence<int, 6, 12, 13, 16, 17>{},
-              [&](auto qc) { if (dest_is_pore(qc)) s += 2.0 * val(qc); });
+              [&](auto qc) { if (dest_is_pore(qc)) s.add(M(2) * val(qc)); });
     }
-    return s;
+    return s.value();
 }
 
 // From values still in registers (the pipelined kernel).
 template <class S>
 __device__ __forceinline__ double next_inlet_part(const typename S::M* d, const DevLattice& L,
                                                   int64_t p, int i, typename S::M r_own, uint32_t seed) {
-    return inlet_contribution<S>(L, (uint32_t)p, i, [&](auto qc) -> double {
+    return inlet_contribution<S>(L, (uint32_t)p, i, [&](auto qc) {
         constexpr int Q = decltype(qc)::value;
-        return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i)), r_own);
+        return S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i)), r_own);
     });
 }
 
@@ -359,10 +387,10 @@ __device__ __forceinline__ double next_inlet_part(const typename S::M* d, const 
 template <class S>
 __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename S::T>& P, const DevLattice& L,
                                                          uint32_t p, int i, typename S::M r_own) {
-    return inlet_contribution<S>(L, p, i, [&](auto qc) -> double {
+    return inlet_contribution<S>(L, (uint32_t)p, i, [&](auto qc) {
         constexpr int Q = decltype(qc)::value;
         const typename S::T v = *(volatile const typename S::T*)(P.out[Q] + i);
-        return (double)S::template dec<Q>(v, r_own);
+        return S::template dec<Q>(v, r_own);
     });
 }
 
@@ -376,19 +404,65 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 #define LBM_STEP_PREFETCH 224
 #endif
 
+// End of a step, called by the blocks whose tile (number `tile`, of NT / 32 warps
+// of GROUP nodes each) holds plane z = 0 or z = 1 nodes: every warp stores its part
+// of the next inlet sum; the last tile adds the parts and writes the next density
+// (and the next rounding seed).  The parts are added in an order that does not
+// depend on NT -- part j on virtual lane j mod 256, then the trees of 8 virtual
+// warps, then one of the 8 sums -- so the block size does not change the result.
+template <class S, int NT, int GROUP = 32>
+__device__ __forceinline__ void finish_inlet(double part, int64_t tile, const DevLattice& L, BcState* bc, int slot,
+                                             double* __restrict__ partials, unsigned* __restrict__ counter, double* sh,
+                                             bool* last) {
+    constexpr int W = NT / 32;
+    const unsigned tiles = (unsigned)((L.a_01 + W * GROUP - 1) / (W * GROUP));
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const double v = warp_sum(part);
+    if (lane == 0) {
+        partials[tile * W + wid] = v;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        *last = atomicAdd(counter, 1u) == tiles - 1;
+    }
+    __syncthreads();
+    if (*last) {
+        __threadfence();
+        for (int vw = wid; vw < 8; vw += W) {
+            double s = 0.0;
+            for (unsigned j = vw * 32 + lane; j < tiles * W; j += 256) s += __ldcg(partials + j);
+            s = warp_sum(s);
+            if (lane == 0) sh[vw] = s;
+        }
+        __syncthreads();
+        if (wid == 0) {
+            const double s = warp_sum(lane < 8 ? sh[lane] : 0.0);
+            if (lane == 0) {
+                bc->drho_in[slot ^ 1] = (bc->Q + s) / (double)L.a_in;
+                if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
+                *counter = 0u;
+            }
+        }
+        __syncthreads();
+    }
+}
+
 // WIN: pulls from the row windows, addressed as row 0 plus a 32-bit element
-// offset (buffers of 19 ns < 2^32 elements), as in the gather-scatter AA step.
-template <class S, bool WIN = false>
-__global__ void __launch_bounds__(kBlock, step_min_blocks<S>())
+// offset (buffers of 19 ns < 2^32 elements), as in the gather-scatter AA step.  NT
+// nodes per block.
+template <class S, bool WIN = false, int NT = kBlock>
+__global__ void __launch_bounds__(NT, step_min_blocks<S>())
 k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates,
        BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
     using M = typename S::M;
     __shared__ double sh[32];
     __shared__ bool last;
-    const int64_t i64 = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+    const int64_t i64 = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int i = (int)i64;
     double part = 0.0;
-    if constexpr (LBM_STEP_PREFETCH > 0) {
+    if constexpr (LBM_STEP_PREFETCH > 0 && NT == kBlock) {
         // threads 0..18: input row q (rows are P.in[0] + q ns; the 128-element
         // padding keeps every range 16-byte aligned); thread 19: the voxel list,
         // cut to a multiple of 4 entries
@@ -431,28 +505,7 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
             else part = next_inlet_part<S>(d, L, pv, i, r_own, seed);
         }
     }
-    // blocks that hold plane z = 0 or z = 1 nodes (block-uniform branch)
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) {
-        const unsigned nb = (unsigned)((L.a_01 + kBlock - 1) / kBlock);
-        const double b = block_sum<kBlock>(part, sh);
-        if (threadIdx.x == 0) {
-            partials[blockIdx.x] = b;
-            __threadfence();
-            last = atomicAdd(counter, 1u) == nb - 1;
-        }
-        __syncthreads();
-        if (last) {
-            __threadfence();
-            double s = 0.0;
-            for (unsigned j = threadIdx.x; j < nb; j += kBlock) s += __ldcg(partials + j);
-            s = block_sum<kBlock>(s, sh);
-            if (threadIdx.x == 0) {
-                bc->drho_in[slot ^ 1] = (bc->Q + s) / (double)L.a_in;
-                if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
-                *counter = 0u;
-            }
-        }
-    }
+    if ((int64_t)blockIdx.x * NT < L.a_01) finish_inlet<S, NT>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
 }
 
 // ------------------------------------------------------ AA-pattern step ---
@@ -549,19 +602,19 @@ __device__ __forceinline__ uint64_t aa_index_policy() {
 // offset arithmetic (the launch on the 256^3 pack, ids staged -> offsets staged:
 // 0.2006 -> 0.1825 ms FP16-dev, 0.2013 -> 0.1972 ms FP32).  Otherwise the ids of
 // the id grid are staged and the rows addressed by 64-bit pointers.
-template <class S, bool ODD, bool WIN = false>
-__global__ void __launch_bounds__(kBlock, aa_min_blocks<S, ODD>())
+template <class S, bool ODD, bool WIN = false, int NT = kBlock>
+__global__ void __launch_bounds__(NT, aa_min_blocks<S, ODD>())
 k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename S::M> rates,
           BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
     using M = typename S::M;
     __shared__ double sh[32];
     __shared__ bool last;
-    __shared__ int sid[ODD ? 18 : 1][kBlock];  // gather offset (WIN) or pore id per direction
-    const int64_t i64 = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+    __shared__ int sid[ODD ? 18 : 1][NT];  // gather offset (WIN) or pore id per direction
+    const int64_t i64 = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int i = (int)i64;
     double part = 0.0;
     constexpr int kAhead = S::kRef ? LBM_AA16_PREFETCH : LBM_AA_PREFETCH;
-    if constexpr (ODD && kAhead > 0) {
+    if constexpr (ODD && kAhead > 0 && NT == kBlock) {
         // threads 0..18: row q of the buffer (rows are F.row[0] + q ns, as
         // launched; 128-element padding keeps every range 16-byte aligned for
         // 2-byte values too); thread 19: the node list, cut to a multiple of 4 entries
@@ -654,34 +707,14 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
         if (i64 < L.a_01) {
             // the counted values land on plane 0: from plane 1 (xi_z = -1, stored
             // with plane 0's reference in the odd step) or staying on plane 0
-            part = inlet_contribution<S>(L, L.vox[i], i, [&](auto qc) -> double {
+            part = inlet_contribution<S>(L, L.vox[i], i, [&](auto qc) {
                 constexpr int Q = decltype(qc)::value;
                 const M rq = (ODD && cz(Q) < 0) ? r_own - g : r_own;
-                return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], rq, sr_key<S>(seed, i)), rq);
+                return S::template dec<Q>(S::template enc_sr<Q>(d[Q], rq, sr_key<S>(seed, i)), rq);
             });
         }
     }
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) {
-        const unsigned nbk = (unsigned)((L.a_01 + kBlock - 1) / kBlock);
-        const double b = block_sum<kBlock>(part, sh);
-        if (threadIdx.x == 0) {
-            partials[blockIdx.x] = b;
-            __threadfence();
-            last = atomicAdd(counter, 1u) == nbk - 1;
-        }
-        __syncthreads();
-        if (last) {
-            __threadfence();
-            double s = 0.0;
-            for (unsigned j = threadIdx.x; j < nbk; j += kBlock) s += __ldcg(partials + j);
-            s = block_sum<kBlock>(s, sh);
-            if (threadIdx.x == 0) {
-                bc->drho_in[slot ^ 1] = (bc->Q + s) / (double)L.a_in;
-                if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
-                *counter = 0u;
-            }
-        }
-    }
+    if ((int64_t)blockIdx.x * NT < L.a_01) finish_inlet<S, NT>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
 }
 
 // ------------------------------------------- two nodes per thread (16-bit) ---
@@ -744,43 +777,16 @@ __device__ __forceinline__ double inlet_part_nodes(const F2* d, int64_t i0, int6
         const int64_t i = k ? i1 : i0;
         if (i < L.a_01) {
             const uint32_t u = sr_key<S>(seed, i);
-            s += inlet_contribution<S>(L, L.vox[i], (int)i, [&](auto qc) -> double {
+            s += inlet_contribution<S>(L, L.vox[i], (int)i, [&](auto qc) {
                 constexpr int Q = decltype(qc)::value;
                 float v[2];
                 split(d[Q], v[0], v[1]);
                 const float r = ref(k, qc);
-                return (double)S::template dec<Q>(S::template enc_sr<Q>(v[k], r, u), r);
+                return S::template dec<Q>(S::template enc_sr<Q>(v[k], r, u), r);
             });
         }
     }
     return s;
-}
-
-// End of a step: the tile's part of the next inlet sum, the last tile writes the
-// next density (and the next rounding seed).
-template <class S, int NT>
-__device__ __forceinline__ void finish_inlet(double part, const DevLattice& L, BcState* bc, int slot,
-                                             double* __restrict__ partials, unsigned* __restrict__ counter, double* sh,
-                                             bool* last) {
-    const unsigned nb = (unsigned)((L.a_01 + kBlock - 1) / kBlock);
-    const double b = block_sum<NT>(part, sh);
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = b;
-        __threadfence();
-        *last = atomicAdd(counter, 1u) == nb - 1;
-    }
-    __syncthreads();
-    if (*last) {
-        __threadfence();
-        double s = 0.0;
-        for (unsigned j = threadIdx.x; j < nb; j += NT) s += __ldcg(partials + j);
-        s = block_sum<NT>(s, sh);
-        if (threadIdx.x == 0) {
-            bc->drho_in[slot ^ 1] = (bc->Q + s) / (double)L.a_in;
-            if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
-            *counter = 0u;
-        }
-    }
 }
 
 template <class S>
@@ -832,7 +838,7 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
         });
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair>(part, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair, 64>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
 }
 
 // Gather-scatter launch: thread t of a warp owns the nodes 64 w + t and
@@ -916,7 +922,7 @@ k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float
             return cz(decltype(qc)::value) < 0 ? r - g : r;
         });
     }
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair>(part, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair, 64>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
 }
 
 // Node-local launch: neighbouring nodes on a thread, one 4-byte load and store per row.
@@ -961,7 +967,7 @@ k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<floa
         });
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair>(part, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair, 64>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
 }
 
 // Pull layout <-> layout S: swap F[q][x] and F[opp q][x] at every node.
@@ -1195,26 +1201,8 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<type
             });
             if (i64 < L.a_01) part = next_inlet_part<S>(d, L, p_cur, i, r_own, seed);
         }
-        if (t < nt01) {  // tile holds plane z = 0 / z = 1 nodes (block-uniform)
-            const double b = block_sum<NT>(part, sh);
-            if (threadIdx.x == 0) {
-                partials[t] = b;
-                __threadfence();
-                last = atomicAdd(counter, 1u) == (unsigned)nt01 - 1;
-            }
-            __syncthreads();
-            if (last) {
-                __threadfence();
-                double s = 0.0;
-                for (int64_t j = threadIdx.x; j < nt01; j += NT) s += __ldcg(partials + j);
-                s = block_sum<NT>(s, sh);
-                if (threadIdx.x == 0) {
-                    bc->drho_in[slot ^ 1] = (bc->Q + s) / (double)L.a_in;
-                    if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
-                    *counter = 0u;
-                }
-            }
-        }
+        if (t < nt01)  // tile holds plane z = 0 / z = 1 nodes (block-uniform)
+            finish_inlet<S, NT>(part, t, L, bc, slot, partials, counter, sh, &last);
         hi_cur = hi_next;
         nb_cur = nb_next;
         p_cur = p_next;
@@ -1477,6 +1465,13 @@ __global__ void k_node_words(const uint32_t* __restrict__ vox, uint32_t vox0, in
     nodew[i] = word;
 }
 
+// FP64 lattices of at most one wave of 256-node blocks (152 SMs, one such block
+// resident) run in small blocks, so that every SM's FP64 units get an even share:
+// 16x16x64 duct, 12,544 nodes, 100 steps 2.05 -> 1.64 ms.  FP32 (61x67x72 pack,
+// 112 k nodes) measured slower: 1.01 ms in blocks of 256, 1.02 in 128, 1.17 in 64.
+constexpr int64_t kSmallNodes = 152 * 256;
+constexpr int kSmallBlock = 32;
+
 inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 template <class F>
@@ -1533,6 +1528,9 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
             if constexpr (S::kRef)
                 k_step_pair<S><<<blocks_for(L.n, kBlock), kPair, 0, st>>>(P, slot, L, make_rates<float>(r.sp, r.sm), bc,
                                                                           partials, counter);
+            else if (sizeof(M) == 8 && L.n < kSmallNodes)
+                k_step<S, true, kSmallBlock><<<blocks_for(L.n, kSmallBlock), kSmallBlock, 0, st>>>(
+                    P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials, counter);
             else
                 k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc,
                                                                              partials, counter);
@@ -1670,6 +1668,15 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
                         k_aa_even_pair<S><<<nb, kPair, 0, st>>>(F, slot, L, rates, bc, partials, counter);
                     return cudaGetLastError();
                 }
+            } else if (win && sizeof(M) == 8 && L.n < kSmallNodes) {
+                const unsigned nbs = blocks_for(L.n, kSmallBlock);
+                if (odd)
+                    k_step_aa<S, true, true, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials,
+                                                                                       counter);
+                else
+                    k_step_aa<S, false, false, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc,
+                                                                                         partials, counter);
+                return cudaGetLastError();
             } else if (odd && win) {
                 k_step_aa<S, true, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials, counter);
                 return cudaGetLastError();
