@@ -46,6 +46,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lbm.h"
@@ -666,6 +667,233 @@ k_wgrad(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensor
     }
 }
 
+// ---------------------------------------- weight gradient marching in z ---
+// The weight gradient of the narrow layers (CIN, COUT in {32, 64}).  What bounds
+// k_wgrad there is again the L2 -> shared memory stream: it loads every shifted
+// activation window apart (280 KB per 128 rows, 11.6 TB/s over the chip).  Here a
+// CTA marches along z over a patch of a plane with the activation planes it needs
+// resident, and
+//   D[(dy, ci) x (dx, co)] += sum_r' act[r' + off(dz, dy)][ci] g[r' - dx][co]
+// takes the three dx taps as three column blocks: the output-gradient operand
+// started one row apart (MN blocks whose distance is one row), so one product of
+// N = 3 COUT does the work of three.  The dy taps are MN blocks of the activation
+// operand one padded row line apart: with 32 channels dy = -1, 0, 1 and one unused
+// block, with 64 channels two of them (dy = -1, 0 and dy = 1 with an unused one).
+// A group of 128 (dy, ci) lanes takes 3 COUT accumulator columns; blockIdx.y picks
+// the groups of a CTA (at most 512 columns).  The row sum of a patch ends with the
+// interior lines, rounded up to 16 rows of zeros.
+//   The tensor core truncates as it adds, so the error of a sum grows with the
+// products added in one accumulator.  An accumulator is therefore drained (added
+// to the CTA's partial sums in FP32) before it has taken more than a split of
+// k_wgrad would, or 64 products of 16 rows: on 64 -> 64 channels, 4 x 44x52x36
+// voxels, the error against 64 bits is 1.5e-6 of the gradient, 1.6e-6 with k_wgrad
+// (6.2e-6 with one drain per CTA).
+template <int CIN, int COUT>
+struct WmCfg {
+    static constexpr int GDY = CIN == 32 ? 1 : 2;             // groups per dz
+    static constexpr int N = 3 * COUT;
+    static constexpr int GPC = COUT == 32 ? 3 : GDY;          // groups of a CTA
+    static constexpr int SETS = 3 * GDY / GPC;
+    static constexpr int ND = GPC == 3 * GDY ? 3 : (GPC + GDY - 1) / GDY;  // activation planes of a step
+    static constexpr uint32_t AROW = CIN * 2, GROW = COUT * 2;
+    static constexpr uint32_t ASWZ = CIN == 64 ? 2u : 4u, GSWZ = COUT == 64 ? 2u : 4u;
+    static constexpr size_t SMEM_MAX = 227 * 1024;
+};
+struct WmArgs {
+    int T;                  // 128-row tiles of a patch
+    int na, ng;             // activation and output-gradient plane buffers
+    int seg, abox, anbox, nseg, abytes;   // as in MarchArgs, rows without the dx halo
+    int gbox, gnbox, gbytes;
+    int patches;
+    int limit;              // 16-row products an accumulator takes before it is drained
+};
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(kThreads, 1)
+k_wgrad_march(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mG, WgArgs w, WmArgs a) {
+    using K = WmCfg<CIN, COUT>;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    unsigned char* sA = base;
+    unsigned char* sG = sA + (size_t)a.na * a.abytes;
+    uint64_t* afull = (uint64_t*)(sG + (size_t)a.ng * a.gbytes);
+    uint64_t* aempty = afull + 8;
+    uint64_t* gfull = aempty + 8;
+    uint64_t* gempty = gfull + 4;
+    uint64_t* accb = gempty + 4;
+    uint64_t* drained = accb + 1;
+    uint32_t* tslot = (uint32_t*)(drained + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g0 = blockIdx.y * K::GPC;                        // first group
+    const int dz0 = g0 / K::GDY, dz1 = (g0 + K::GPC - 1) / K::GDY;  // dz + 1 of the first and last group
+    const int nd = dz1 - dz0 + 1;
+    const int Z = w.g.Z, xp = w.g.xp();
+    const int64_t plane = w.g.plane();
+    const int64_t items = (int64_t)w.g.B * a.patches * Z;
+    const int64_t i0 = items * blockIdx.x / gridDim.x, i1 = items * (blockIdx.x + 1) / gridDim.x;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < a.na; ++s) {
+            tc::mbar_init(&afull[s], 1);
+            tc::mbar_init(&aempty[s], 1);
+        }
+        for (int s = 0; s < a.ng; ++s) {
+            tc::mbar_init(&gfull[s], 1);
+            tc::mbar_init(&gempty[s], 1);
+        }
+        tc::mbar_init(accb, 1);
+        tc::mbar_init(drained, 4);
+        tc::mbar_init_fence();
+    }
+    if (warp == 1) tc::tmem_alloc(tslot, 512);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tslot;
+    // 16-row products of a step on the patch of item i
+    auto steps_of = [&](int64_t i) -> int {
+        const int64_t p0 = xp + (i / Z % a.patches) * a.T * kRows;
+        return (int)((min((int64_t)a.T * kRows, (int64_t)(w.g.Y + 1) * xp - p0) + 15) / 16);
+    };
+    if (warp == 0) {
+        if (lane == 0) {
+            const uint32_t ab = (uint32_t)(a.nseg * a.anbox * a.abox) * K::AROW;
+            const uint32_t gb = (uint32_t)(a.gnbox * a.gbox) * K::GROW;
+            uint32_t ca = 0, cg = 0;
+            bool ok = true;
+            for (int64_t i = i0; i < i1 && ok;) {
+                const int64_t col = i / Z;
+                const int zs = (int)(i - col * Z), ze = (int)min((int64_t)Z - 1, zs + (i1 - i) - 1);
+                const int64_t b = col / a.patches, p0 = xp + (col - b * a.patches) * a.T * kRows;
+                const int64_t sample = b * w.g.per_sample();
+                for (int z = zs; z <= ze && ok; ++z, ++cg) {
+                    // activation planes z + dz of this step that are not resident yet
+                    for (int d = z == zs ? dz0 : dz1; d <= dz1; ++d, ++ca) {
+                        const uint32_t s = ca % a.na, use = ca / a.na;
+                        if (use > 0 && !tc::mbar_wait(&aempty[s], (use - 1) & 1, w.err)) {
+                            ok = false;
+                            break;
+                        }
+                        tc::mbar_expect_tx(&afull[s], ab);
+                        const int64_t r = sample + (int64_t)(z + d) * plane + p0 - xp;  // padded plane z + 1 + (d - 1)
+                        unsigned char* dst = sA + (size_t)s * a.abytes;
+                        for (int g = 0; g < a.nseg; ++g)
+                            for (int k = 0; k < a.anbox; ++k)
+                                tc::tma_load_2d(dst + (size_t)(g * a.anbox + k) * a.abox * K::AROW, &mA, &afull[s], 0,
+                                                (int)(r + (int64_t)g * xp + k * a.abox));
+                    }
+                    const uint32_t s = cg % a.ng, use = cg / a.ng;
+                    if (!ok || (use > 0 && !tc::mbar_wait(&gempty[s], (use - 1) & 1, w.err))) {
+                        ok = false;
+                        break;
+                    }
+                    tc::mbar_expect_tx(&gfull[s], gb);
+                    const int64_t r = sample + (int64_t)(z + 1) * plane + p0 - 1;
+                    for (int k = 0; k < a.gnbox; ++k)
+                        tc::tma_load_2d(sG + (size_t)s * a.gbytes + (size_t)k * a.gbox * K::GROW, &mG, &gfull[s], 0,
+                                        (int)(r + k * a.gbox));
+                }
+                i += ze - zs + 1;
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = tc::idesc_bf16(kRows, K::N, true, true);
+            uint32_t ca = 0, cg = 0;  // ca: the oldest resident activation plane
+            bool ok = true, first = true;
+            int taken = 0;            // products in the accumulators
+            uint32_t drains = 0;
+            for (int64_t i = i0; i < i1 && ok;) {
+                const int64_t col = i / Z;
+                const int zs = (int)(i - col * Z), ze = (int)min((int64_t)Z - 1, zs + (i1 - i) - 1);
+                const int nk = steps_of(i);
+                for (int z = zs; z <= ze; ++z, ++cg) {
+                    if (taken > 0 && taken + nk > a.limit) {
+                        tc::mma_commit(accb);
+                        if (!(ok = tc::mbar_wait(drained, drains & 1, w.err))) break;
+                        tc::fence_after_sync();
+                        ++drains;
+                        taken = 0;
+                        first = true;
+                    }
+                    taken += nk;
+                    for (int d = z == zs ? 0 : nd - 1; d < nd && ok; ++d)
+                        ok = tc::mbar_wait(&afull[(ca + d) % a.na], ((ca + d) / a.na) & 1, w.err);
+                    if (!ok || !(ok = tc::mbar_wait(&gfull[cg % a.ng], (cg / a.ng) & 1, w.err))) break;
+                    tc::fence_after_sync();
+                    const uint32_t gp = tc::su32(sG + (size_t)(cg % a.ng) * a.gbytes);
+                    uint32_t ap[K::GPC];
+#pragma unroll
+                    for (int j = 0; j < K::GPC; ++j) {
+                        const int d = (g0 + j) / K::GDY - dz0, dy = (g0 + j) % K::GDY * 2;  // first dy block
+                        ap[j] = tc::su32(sA + (size_t)((ca + d) % a.na) * a.abytes) + (uint32_t)(dy * a.seg) * K::AROW;
+                    }
+                    for (int k = 0; k < nk; ++k) {
+                        const uint64_t gd = tc::smem_desc(gp + (uint32_t)k * 16 * K::GROW, K::GROW, 8 * K::GROW, K::GSWZ);
+#pragma unroll
+                        for (int j = 0; j < K::GPC; ++j)
+                            tc::mma_bf16(tmem + j * K::N,
+                                         tc::smem_desc(ap[j] + (uint32_t)k * 16 * K::AROW, (uint32_t)a.seg * K::AROW,
+                                                       8 * K::AROW, K::ASWZ),
+                                         gd, idesc, !(first && k == 0));
+                    }
+                    first = false;
+                    tc::mma_commit(&gempty[cg % a.ng]);
+                    const int done = z == ze ? nd : 1;
+                    for (int d = 0; d < done; ++d, ++ca) tc::mma_commit(&aempty[ca % a.na]);
+                }
+                i += ze - zs + 1;
+            }
+            tc::mma_commit(accb);
+        }
+    } else {
+        const int q = warp & 3;
+        const int64_t nw = (int64_t)w.cout_real * 27 * w.cin_real;
+        int64_t i = i0;
+        bool ok = i1 > i0;
+        for (uint32_t drain = 0; i < i1 && ok; ++drain) {
+            int taken = 0;
+            do taken += steps_of(i++);
+            while (i < i1 && taken + steps_of(i) <= a.limit);
+            ok = tc::mbar_wait(accb, drain & 1, w.err);
+            tc::fence_after_sync();
+#pragma unroll 1
+            for (int j = 0; j < K::GPC; ++j) {
+                const int m = q * 32 + lane, blk = m / CIN, ci = m % CIN;
+                const int dz = (g0 + j) / K::GDY, dy = (g0 + j) % K::GDY * 2 + blk;  // both + 1
+                const bool valid = ok && dy < 3 && ci < w.cin_real;
+#pragma unroll 1
+                for (int c0 = 0; c0 < K::N; c0 += 32) {
+                    float v[32];
+                    tc::tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + j * K::N + c0, v);
+                    if (!valid) continue;
+                    const int tap = dz * 9 + dy * 3 + 2 - c0 / COUT;  // column block bi is dx = 1 - bi
+#pragma unroll
+                    for (int k = 0; k < 32; ++k) {
+                        const int co = c0 % COUT + k;
+                        if (co >= w.cout_real) continue;
+                        const int64_t o = ((int64_t)co * 27 + tap) * w.cin_real + ci;
+                        // this thread alone writes its partial sums: the additions (no
+                        // result asked for, nothing waited for) keep their order
+                        float* part = w.part + (int64_t)blockIdx.x * nw + o;
+                        if (!w.part) atomicAdd(w.gw + o, v[k]);
+                        else if (drain) atomicAdd(part, v[k]);
+                        else *part = v[k];
+                    }
+                }
+            }
+            tc::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(drained);
+        }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 1) {
+        tc::fence_after_sync();
+        tc::tmem_dealloc(tmem, 512);
+    }
+}
+
 // ------------------------------------------------- elementwise kernels ---
 // Zeros on the border row lines and planes of a padded tensor of C channels, one
 // warp per row line.
@@ -838,14 +1066,30 @@ __global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, 
     }
 }
 
-// gw[w] += sum over k of part[k][w], k in order (the deterministic finish of
-// the weight- and bias-gradient kernels)
-__global__ void k_split_sum(const float* __restrict__ part, int64_t splits, int64_t nw, float* __restrict__ gw) {
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nw; w += (int64_t)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int64_t k = 0; k < splits; ++k) s += part[k * nw + w];
+// gw[w] += sum over k of part[k][w] in a fixed order (the deterministic finish of
+// the weight- and bias-gradient kernels): 8 threads per w each add every eighth
+// split, then the eight sums are added in order.  One thread per w left the card
+// waiting on its chain of loads (19 us a layer on average, 16 MB read).
+__global__ void __launch_bounds__(256)
+k_split_sum(const float* __restrict__ part, int64_t splits, int64_t nw, float* __restrict__ gw) {
+    __shared__ float sh[8][32];
+    const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
+    const int64_t w = (int64_t)blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (w < nw) {
+#pragma unroll 4
+        for (int64_t k = sub; k < splits; k += 8) s += part[k * nw + w];
+    }
+    sh[sub][lane] = s;
+    __syncthreads();
+    if (sub == 0 && w < nw) {
+        for (int u = 1; u < 8; ++u) s += sh[u][lane];
         gw[w] += s;
     }
+}
+inline cudaError_t split_sum(const float* part, int64_t splits, int64_t nw, float* gw, cudaStream_t st) {
+    k_split_sum<<<(unsigned)((nw + 31) / 32), 256, 0, st>>>(part, splits, nw, gw);
+    return cudaGetLastError();
 }
 
 // gb[c] += sum over rows of G[row][c], c < creal; block of 256 threads, C / 8 channel groups.
@@ -1021,6 +1265,65 @@ cudaError_t march_t(const bf16* in, const bf16* wt, int cout, const ConvEpi& epi
     return cudaGetLastError();
 }
 
+// Patch of a marching weight gradient: the largest T for which the resident
+// planes and one more of each kind fit (more tiles: fewer halo rows).  The zero
+// rows after a patch (up to 16) have to end before the next plane's interior:
+// padded lines of 8 rows or more.
+template <int CIN, int COUT>
+bool wm_plan(const PGeo& g, int n_sm, WmArgs* out, size_t* smem) {
+    using K = WmCfg<CIN, COUT>;
+    if (g.xp() < 8) return false;
+    const int64_t lines = (int64_t)g.Y * g.xp();
+    for (int T = 4; T >= 1; --T) {
+        if (T > 1 && (T - 1) * kRows >= lines) continue;
+        for (int nseg = 1; nseg <= 3; nseg += 2) {
+            const int rows = nseg == 1 ? T * kRows + 2 * g.xp() : T * kRows;
+            WmArgs a{};
+            a.T = T;
+            a.nseg = nseg;
+            a.anbox = (rows + 255) / 256;
+            a.abox = ((rows + a.anbox - 1) / a.anbox + 7) / 8 * 8;
+            a.seg = nseg == 1 ? g.xp() : a.anbox * a.abox;
+            a.abytes = (int)(((size_t)nseg * a.anbox * a.abox * K::AROW + 1023) / 1024 * 1024);
+            const int grows = T * kRows + 2;
+            a.gnbox = (grows + 255) / 256;
+            a.gbox = ((grows + a.gnbox - 1) / a.gnbox + 7) / 8 * 8;
+            a.gbytes = (int)(((size_t)a.gnbox * a.gbox * K::GROW + 1023) / 1024 * 1024);
+            a.na = K::ND + 1;
+            a.ng = 2;
+            a.patches = (int)((lines + T * kRows - 1) / (T * kRows));
+            // the unused block of the activation operand reads up to one segment past
+            // its plane: into the buffers after it, and at the end into this slack
+            const size_t used = (size_t)a.na * a.abytes + (size_t)a.ng * a.gbytes + 256;
+            const size_t over = (size_t)a.seg * K::AROW;
+            const size_t slack = over > (size_t)a.ng * a.gbytes ? over - (size_t)a.ng * a.gbytes : 0;
+            const size_t total = 1024 + used + slack;
+            if (total > K::SMEM_MAX) continue;
+            a.limit = (int)std::max<int64_t>(64, g.rows() / wgrad_splits(CIN, COUT, g.rows(), n_sm) / 16);
+            *out = a;
+            *smem = total;
+            return true;
+        }
+    }
+    return false;
+}
+template <int CIN, int COUT>
+int64_t wm_splits(const PGeo& g, const WmArgs& a, int n_sm) {
+    return std::min<int64_t>(std::max(1, n_sm / WmCfg<CIN, COUT>::SETS), (int64_t)g.B * a.patches * g.Z);
+}
+template <int CIN, int COUT>
+cudaError_t wm_t(const bf16* act, const bf16* gout, const WgArgs& w, const WmArgs& a, size_t smem, int64_t splits,
+                 cudaStream_t st) {
+    using K = WmCfg<CIN, COUT>;
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad_march<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    CUtensorMap ma, mg;
+    if (e == cudaSuccess) e = make_map(&ma, act, CIN, w.g.rows(), CIN, a.abox);
+    if (e == cudaSuccess) e = make_map(&mg, gout, COUT, w.g.rows(), COUT, a.gbox);
+    if (e != cudaSuccess) return e;
+    k_wgrad_march<CIN, COUT><<<dim3((unsigned)splits, K::SETS), kThreads, smem, st>>>(ma, mg, w, a);
+    return cudaGetLastError();
+}
+
 template <int CIN, int COUT>
 cudaError_t wgrad_t(const bf16* act, const bf16* gout, const WgArgs& a0, cudaStream_t st, int n_sm) {
     using K = WgCfg<CIN, COUT>;
@@ -1037,7 +1340,6 @@ cudaError_t wgrad_t(const bf16* act, const bf16* gout, const WgArgs& a0, cudaStr
     const int64_t nw = (int64_t)a.cout_real * 27 * a.cin_real;
     if (a.part && (int64_t)splits * nw > a.part_cap) return cudaErrorInvalidValue;
     k_wgrad<CIN, COUT><<<dim3(splits, (unsigned)gsets), kThreads, K::SMEM, st>>>(ma, mg, a);
-    if (a.part) k_split_sum<<<gs_blocks(nw), 256, 0, st>>>(a.part, splits, nw, a.gw);
     return cudaGetLastError();
 }
 
@@ -1086,8 +1388,53 @@ cudaError_t conv(int cin, int cout, const bf16* in, const bf16* w, const bf16* w
         default: return cudaErrorInvalidValue;
     }
 }
-cudaError_t wgrad(int cin, int cout, const bf16* act, const bf16* gout, const WgArgs& a, cudaStream_t st, int n_sm) {
+// f(cin, cout as integral constants) for the pairs whose weight gradient can march.
+template <class F>
+bool wm_pair(int cin, int cout, F&& f) {
+    using C32 = std::integral_constant<int, 32>;
+    using C64 = std::integral_constant<int, 64>;
+    if (cin == 32 && cout == 32) return f(C32{}, C32{});
+    if (cin == 32 && cout == 64) return f(C32{}, C64{});
+    if (cin == 64 && cout == 32) return f(C64{}, C32{});
+    if (cin == 64 && cout == 64) return f(C64{}, C64{});
+    return false;
+}
+// Row splits (partial sums) of a layer's weight gradient.
+int64_t weight_splits(int cin, int cout, const PGeo& g, int n_sm) {
+    int64_t n = 0;
+    if (wm_pair(cin, cout, [&](auto ci, auto co) {
+            constexpr int CI = decltype(ci)::value, CO = decltype(co)::value;
+            WmArgs a{};
+            size_t smem;
+            if (!wm_plan<CI, CO>(g, n_sm, &a, &smem)) return false;
+            n = wm_splits<CI, CO>(g, a, n_sm);
+            return true;
+        }))
+        return n;
+    return wgrad_splits(cin, cout, g.rows(), n_sm);
+}
+cudaError_t wgrad_old(int cin, int cout, const bf16* act, const bf16* gout, const WgArgs& a, cudaStream_t st, int n_sm) {
     WS_DISPATCH(wgrad_t, cin, cout, act, gout, a, st, n_sm)
+}
+cudaError_t wgrad(int cin, int cout, const bf16* act, const bf16* gout, const WgArgs& a, cudaStream_t st, int n_sm) {
+    cudaError_t e = cudaSuccess;
+    int64_t splits = 0;
+    const bool marched = wm_pair(cin, cout, [&](auto ci, auto co) {
+        constexpr int CI = decltype(ci)::value, CO = decltype(co)::value;
+        WmArgs m{};
+        size_t smem;
+        if (!wm_plan<CI, CO>(a.g, n_sm, &m, &smem)) return false;
+        splits = wm_splits<CI, CO>(a.g, m, n_sm);
+        const int64_t nw = (int64_t)a.cout_real * 27 * a.cin_real;
+        e = a.part && splits * nw > a.part_cap ? cudaErrorInvalidValue : wm_t<CI, CO>(act, gout, a, m, smem, splits, st);
+        return true;
+    });
+    if (!marched) {
+        splits = wgrad_splits(cin, cout, a.g.rows(), n_sm);
+        e = wgrad_old(cin, cout, act, gout, a, st, n_sm);
+    }
+    if (e != cudaSuccess || !a.part) return e;
+    return split_sum(a.part, splits, (int64_t)a.cout_real * 27 * a.cin_real, a.gw, st);
 }
 
 bool chan_ok(int c) { return c == 32 || c == 64 || c == 128 || c == 256; }
@@ -1280,7 +1627,7 @@ int bwd_weight(lbm_wsnet* n, int k, const bf16* act, const bf16* gout, int l) {
     const unsigned nb = (unsigned)std::min<int64_t>(std::max<int64_t>(1, rows / 512), 152 * 4);
     // partial sums per row split, added in a fixed order: the gradients (and so
     // the training) do not depend on the order in which CTAs finish
-    const int64_t need = std::max<int64_t>(wsn::wgrad_splits(d.cin_p, d.cout_p, rows, n->n_sm) * d.cout * 27 * d.cin,
+    const int64_t need = std::max<int64_t>(wsn::weight_splits(d.cin_p, d.cout_p, a.g, n->n_sm) * d.cout * 27 * d.cin,
                                            (int64_t)nb * d.cout);
     if (need > n->part_cap) {
         WS_CUDA(n, cudaStreamSynchronize(n->stream));
@@ -1295,8 +1642,7 @@ int bwd_weight(lbm_wsnet* n, int k, const bf16* act, const bf16* gout, int l) {
     a.part_cap = n->part_cap;
     WS_CUDA(n, wsn::wgrad(d.cin_p, d.cout_p, act, gout, a, n->stream, n->n_sm));
     wsn::k_bias_grad<<<nb, 256, 0, n->stream>>>(gout, rows, d.cout_p, d.cout, n->g + d.boff, n->part);
-    wsn::k_split_sum<<<wsn::gs_blocks(d.cout), 256, 0, n->stream>>>(n->part, nb, d.cout, n->g + d.boff);
-    WS_CUDA(n, cudaGetLastError());
+    WS_CUDA(n, wsn::split_sum(n->part, nb, d.cout, n->g + d.boff, n->stream));
     return LBM_OK;
 }
 
