@@ -1164,7 +1164,67 @@ __global__ void k_adam(float* p, const float* g, float* m, float* v, int64_t n, 
     }
 }
 
+// One layer's caller weights w[co][27][ci] in the layouts of k_conv (wk) and of the
+// kernels that read whole taps (wt): as they are, or flipped in tap and transposed
+// in channel for the data gradient (op 1).
+__global__ void k_pack_layer(const bf16* __restrict__ w, int cin, int cout, int op, bf16* __restrict__ wk,
+                             bf16* __restrict__ wt) {
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= (int64_t)cout * 27 * cin) return;
+    const int ci = (int)(k % cin), t = (int)((k / cin) % 27), co = (int)(k / (27 * cin));
+    const bf16 v = w[k];
+    if (op == 0) {
+        wk[k] = v;
+        wt[((int64_t)t * cout + co) * cin + ci] = v;
+    } else {
+        wk[((int64_t)ci * 27 + (26 - t)) * cout + co] = v;
+        wt[((int64_t)(26 - t) * cin + ci) * cout + co] = v;
+    }
+}
+
 // ------------------------------------------------------- host helpers ---
+// Scratch of a single convolution call, stream-ordered from one pool per device:
+// the pool keeps at most kScratchKept bytes between calls (a cudaMalloc and a
+// cudaFree per call took 170 us, about as long as a layer), shared by all threads
+// and streams; lbm_wsnet_release_buffers gives them back.
+constexpr uint64_t kScratchKept = 16u << 20;
+constexpr int kMaxDevices = 64;
+cudaMemPool_t g_scratch[kMaxDevices] = {};
+std::mutex g_scratch_mutex;
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    cudaMemPool_t pool;
+    {
+        std::lock_guard<std::mutex> lock(g_scratch_mutex);
+        if (!g_scratch[dev]) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t made = nullptr;
+            if ((e = cudaMemPoolCreate(&made, &props)) != cudaSuccess) return e;
+            uint64_t kept = kScratchKept;
+            if ((e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &kept)) != cudaSuccess) {
+                cudaMemPoolDestroy(made);
+                return e;
+            }
+            g_scratch[dev] = made;
+        }
+        pool = g_scratch[dev];
+    }
+    return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+void scratch_trim() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    if (g_scratch[dev]) cudaMemPoolTrimTo(g_scratch[dev], 0);
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 std::once_flag g_encode_once;
 
@@ -2030,6 +2090,7 @@ int lbm_wsnet_release_buffers(lbm_wsnet* n) {
     if (rc) return rc;
     cudaStreamSynchronize(n->stream);
     free_buffers(n);
+    wsn::scratch_trim();
     cudaFree(n->part);
     n->part = nullptr;
     n->part_cap = 0;
@@ -2069,31 +2130,22 @@ int conv_call(int op, const void* in, const void* aux, const void* w, const floa
         op < 0 || op > 2 || (op == 2 && !aux) || reps < 1)
         return LBM_EINVAL;
     const PGeo g{batch, nx, ny, nz};
-    int* d_err = nullptr;
-    if (cudaMalloc(&d_err, sizeof(int)) != cudaSuccess) return LBM_ENOMEM;
-    cudaError_t e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
-    // the layouts the convolution kernel reads: forward [cout][27][cin] and
-    // [27][cout][cin]; data gradient (flipped taps) [cin][27][cout] and [27][cin][cout]
-    bf16* wb = nullptr;  // two arrays: wb and wb + n
+    // scratch: the error flag, then the layouts the convolution kernels read:
+    // forward [cout][27][cin] and [27][cout][cin]; data gradient (flipped taps)
+    // [cin][27][cout] and [27][cin][cout]
     const size_t nw = (size_t)cout * 27 * cin;
+    void* scratch = nullptr;
+    cudaError_t e = wsn::scratch_alloc(&scratch, 256 + (op < 2 ? 2 * nw * sizeof(bf16) : 0), st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
+    }
+    int* d_err = (int*)scratch;
+    bf16* wb = (bf16*)((char*)scratch + 256);  // two arrays: wb and wb + nw
+    e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
     if (e == cudaSuccess && op < 2) {
-        std::vector<uint16_t> hw(nw), hb(2 * nw);
-        e = cudaMemcpyAsync(hw.data(), w, nw * 2, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        for (int co = 0; co < cout && e == cudaSuccess; ++co)
-            for (int t = 0; t < 27; ++t)
-                for (int ci = 0; ci < cin; ++ci) {
-                    const uint16_t v = hw[((size_t)co * 27 + t) * cin + ci];
-                    if (op == 0) {
-                        hb[((size_t)co * 27 + t) * cin + ci] = v;
-                        hb[nw + ((size_t)t * cout + co) * cin + ci] = v;
-                    } else {
-                        hb[((size_t)ci * 27 + (26 - t)) * cout + co] = v;
-                        hb[nw + ((size_t)(26 - t) * cin + ci) * cout + co] = v;
-                    }
-                }
-        if (e == cudaSuccess) e = cudaMalloc(&wb, hb.size() * 2);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(wb, hb.data(), hb.size() * 2, cudaMemcpyHostToDevice, st);
+        wsn::k_pack_layer<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>((const bf16*)w, cin, cout, op, wb, wb + nw);
+        e = cudaGetLastError();
     }
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
@@ -2142,8 +2194,7 @@ int conv_call(int op, const void* in, const void* aux, const void* w, const floa
     }
     for (auto& x : ev)
         if (x) cudaEventDestroy(x);
-    cudaFree(d_err);
-    if (wb) cudaFree(wb);
+    if (cudaFreeAsync(scratch, st) != cudaSuccess && e == cudaSuccess) e = cudaErrorUnknown;
     if (e != cudaSuccess) return LBM_ECUDA;
     return h ? LBM_ETIMEOUT : LBM_OK;
 }
