@@ -228,12 +228,16 @@ __device__ __forceinline__ void batch_finish(double part, int slot, int64_t tile
 
 // One 256-node tile of one step: the single-lattice step with the member's own
 // boundary scalars, and the member's next inlet density.
-template <class S, bool COH, bool WIN = false>
+// FORM: kGrid64 the id grid with 64-bit addresses, kGrid32 the id grid and kWindows
+// the row windows, both with fin plus one 32-bit element offset per source.
+enum { kGrid64 = 0, kGrid32 = 1, kWindows = 2 };
+template <class S, bool COH, int FORM = kGrid64>
 __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typename S::T* fout, int64_t ns, int slot,
                                                 int64_t tile, const Links& K, const int* __restrict__ tile_member,
                                                 Member* members, const Rates<typename S::M>& rates, double* partials,
                                                 unsigned* counters, double* sh) {
     using M = typename S::M;
+    constexpr bool WIN = FORM == kWindows;
     const int mi = tile_member[tile];
     const Member& m = members[mi];
     const int64_t i = tile * kTile + threadIdx.x;
@@ -255,7 +259,15 @@ __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typena
         } else {
             for_q(AllQ{}, [&](auto qc) {
                 constexpr int Q = decltype(qc)::value;
-                d[Q] = pull_b<S, Q, COH>(fin, ns, K.grid, m, p, i, r_own, g);
+                if constexpr (FORM == kGrid32 && Q > 0) {
+                    const int id = __ldg(K.grid + p + m.goff[Q]);
+                    const bool pore = id >= 0;
+                    const uint32_t off = pore ? (uint32_t)Q * (uint32_t)ns + (uint32_t)id
+                                              : (uint32_t)opp(Q) * (uint32_t)ns + (uint32_t)i;
+                    d[Q] = S::template dec<Q>(fin[off], pore ? r_own - M(cz(Q)) * g : r_own);
+                } else {
+                    d[Q] = pull_b<S, Q, COH>(fin, ns, K.grid, m, p, i, r_own, g);
+                }
             });
         }
         if (il < m.a_in) {
@@ -301,15 +313,25 @@ constexpr int batch_min_blocks() {
     return sizeof(typename S::M) == 8 ? 1 : MINB;
 }
 
+// Ensembles of fewer tiles (8 a SM) fit one or two waves: their step is a chain of
+// latencies, where one node per thread and the id grid (resident in L2) are
+// shorter.  Per step, FP16-dev, id grid against windows with pairs: 83,816 pores 9.3
+// and 10.0 us, 365,138 pores 11.3 and 11.2, 707,421 pores 19.1 and 15.4; FP32 8.8
+// and 9.1, 10.5 and 10.3, 22.1 and 20.8.
+#ifndef LBM_WINDOW_TILES
+#define LBM_WINDOW_TILES (8 * 152)
+#endif
+constexpr int64_t kWindowTiles = LBM_WINDOW_TILES;
+
 // One step, one tile per block.
-template <class S, int MINB, bool WIN = false>
+template <class S, int MINB, int FORM = kGrid64>
 __global__ void __launch_bounds__(kTile, batch_min_blocks<S, MINB>())
 k_batch_step(const typename S::T* __restrict__ fin, typename S::T* __restrict__ fout, int64_t ns, int slot, Links K,
              const int* __restrict__ tile_member, Member* members, Rates<typename S::M> rates,
              double* __restrict__ partials, unsigned* __restrict__ counters) {
     __shared__ double sh[32];
-    batch_prefetch(fin, ns, WIN ? K.nodew : K.vox);
-    batch_tile_step<S, false, WIN>(fin, fout, ns, slot, blockIdx.x, K, tile_member, members, rates, partials,
+    batch_prefetch(fin, ns, FORM == kWindows ? K.nodew : K.vox);
+    batch_tile_step<S, false, FORM>(fin, fout, ns, slot, blockIdx.x, K, tile_member, members, rates, partials,
                                    counters, sh);
 }
 
@@ -1018,15 +1040,19 @@ int bstep_once(lbm_batch* b, cudaStream_t st) {
                                                             lbm::make_rates<M>(b->sp, b->sm), b->d_partials,
                                                             b->d_counters);
         };
-        // row windows, and every element offset of a buffer in 32 bits;
+        // 32-bit offsets where every element offset of a buffer fits;
         // GB300_LBM_BATCH_ADDR64 forces the id-grid form (tests)
-        const bool win = b->d_win && 19 * (uint64_t)b->ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_BATCH_ADDR64");
+        const bool off32 = 19 * (uint64_t)b->ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_BATCH_ADDR64");
         const bool capped = cfg_capped(b->config);
-        if (win) {
+        if (off32 && b->ntiles < lbm::kWindowTiles) {
+            capped ? launch(lbm::k_batch_step<S, 5, lbm::kGrid32>, lbm::kTile)
+                   : launch(lbm::k_batch_step<S, 4, lbm::kGrid32>, lbm::kTile);
+        } else if (off32 && b->d_win) {
             if constexpr (S::kRef)
                 capped ? launch(lbm::k_batch_pair<S, 6>, lbm::kTile / 2) : launch(lbm::k_batch_pair<S, 5>, lbm::kTile / 2);
             else
-                capped ? launch(lbm::k_batch_step<S, 5, true>, lbm::kTile) : launch(lbm::k_batch_step<S, 4, true>, lbm::kTile);
+                capped ? launch(lbm::k_batch_step<S, 5, lbm::kWindows>, lbm::kTile)
+                       : launch(lbm::k_batch_step<S, 4, lbm::kWindows>, lbm::kTile);
         } else {
             capped ? launch(lbm::k_batch_step<S, 5>, lbm::kTile) : launch(lbm::k_batch_step<S, 4>, lbm::kTile);
         }

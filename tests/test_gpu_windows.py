@@ -36,3 +36,29 @@ def test_windows_equal_id_grid(monkeypatch, shape, prec, variant):
     monkeypatch.setenv("GB300_LBM_STEP_ADDR64", "1")
     monkeypatch.setenv("GB300_LBM_AA_ADDR64", "1")
     np.testing.assert_array_equal(got, _state(mask, prec, variant, 5))
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16dev", "bf16dev"])
+@pytest.mark.parametrize("config", [0, 1])
+def test_large_ensemble_windows_equal_id_grid(monkeypatch, prec, config):
+    """Ensembles of 1216 tiles or more take the row windows (16-bit: two nodes per
+    thread); odd pore counts, members of one and of many windows per row."""
+    from paper_1806_10589_gb300 import Batch
+
+    masks = [random_mask(*s, 0.1, 5 + k) for k, s in enumerate([(61, 70, 75), (29, 31, 12), (90, 30, 24)])]
+
+    def run():
+        with Batch(masks, 0.8, "mrt", prec) as b:
+            b.set_config(config)
+            assert b.info()["n_tiles"] >= 1216
+            for k in range(len(masks)):
+                b.set_flux_bc(k, 0.05 * (k + 1))
+            b.step(4)
+            return [np.stack(b.fields(k)) for k in range(len(masks))], [b.get_flux(k) for k in range(len(masks))]
+
+    got = run()
+    monkeypatch.setenv("GB300_LBM_BATCH_ADDR64", "1")
+    want = run()
+    for a, b in zip(got[0], want[0]):
+        np.testing.assert_array_equal(a, b)
+    assert got[1] == want[1]
