@@ -56,9 +56,9 @@ struct lbm_ctx {
     uint32_t* d_nodew = nullptr;
     lbm::BcState h_bc{};
     lbm::BcState* d_bc = nullptr;
-    double* d_red_partials = nullptr;   // inlet reductions (prime and fused), per-block partials
-    unsigned* d_red_counter = nullptr;  // ticket of the stand-alone inlet reduction
-    unsigned* d_step_counter = nullptr; // ticket of the reduction fused into the step
+    double* d_red_partials = nullptr;   // stand-alone inlet reduction: per-block partials
+    unsigned* d_red_counter = nullptr;  // and its ticket
+    double* d_parts = nullptr;          // parts of the next step's inlet sum, two parities
     double* d_mon_partials = nullptr;
     unsigned* d_mon_counter = nullptr;
     lbm::MonitorOut* d_mon = nullptr;
@@ -136,7 +136,7 @@ int push_bc(lbm_ctx* c) {
 
 int one_step(lbm_ctx* c, cudaStream_t st) {
     LBM_CUDA(c, lbm::launch_step_cfg(c->prec, c->step_cfg, state_f(c), c->f[c->cur ^ 1], c->cur, c->L,
-                                     c->relax, c->d_bc, c->d_red_partials, c->d_step_counter, st));
+                                     c->relax, c->d_bc, c->d_parts, st));
     c->cur ^= 1;
     return LBM_OK;
 }
@@ -145,7 +145,7 @@ int one_step(lbm_ctx* c, cudaStream_t st) {
 // a node-local one when it is 1; the two alternate across lbm_step calls.
 int aa_step(lbm_ctx* c, cudaStream_t st) {
     LBM_CUDA(c, lbm::launch_aa_step(c->prec, c->f[0], c->aa_phase == 0, c->cur, c->L, c->relax, c->d_bc,
-                                    c->d_red_partials, c->d_step_counter, st));
+                                    c->d_parts, st));
     c->cur ^= 1;
     c->aa_phase ^= 1;
     return LBM_OK;
@@ -188,6 +188,7 @@ int prime_inlet(lbm_ctx* c) {
 // the re-encoded values.  Asynchronous; a no-op for FP32/FP64.
 int maybe_reencode(lbm_ctx* c) {
     if (c->prec < LBM_PREC_FP16DEV || c->since_reencode < kReencodeInterval) return LBM_OK;
+    LBM_CUDA(c, lbm::launch_inlet_finish(c->L, c->d_bc, c->cur, c->d_parts, c->stream));
     LBM_CUDA(c, lbm::launch_reencode(c->prec, state_f(c), c->L, c->d_bc, c->ref_e, c->cur, c->stream));
     c->ref_e ^= 1;
     c->since_reencode = 0;
@@ -239,7 +240,7 @@ void release(lbm_ctx* c) {
     cudaFree(c->d_bc);
     cudaFree(c->d_red_partials);
     cudaFree(c->d_red_counter);
-    cudaFree(c->d_step_counter);
+    cudaFree(c->d_parts);
     cudaFree(c->d_mon_partials);
     cudaFree(c->d_mon_counter);
     cudaFree(c->d_mon);
@@ -369,8 +370,9 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
     // ---- device memory
     int rc = LBM_OK;
     const size_t fbytes = (size_t)19 * (size_t)c->L.ns * (size_t)lbm::elem_size(precision);
-    // partial sums of the inlet reductions: one per 32 nodes of whole 256-node tiles
-    const int nb_red = std::max(lbm::inlet_reduce_blocks(c->L), (int)((a_01 + 255) / 256 * 8));
+    // parts of the inlet sum: one per 32 nodes of whole 256-node tiles
+    c->L.part_stride = (a_01 + 255) / 256 * 8;
+    const int nb_red = lbm::inlet_reduce_blocks(c->L);
     const int nb_mon = lbm::monitor_blocks(c->L);
     if ((rc = dev_alloc(c, &c->f[0], fbytes)) || (rc = dev_alloc(c, &c->f[1], fbytes)) ||
         (rc = dev_alloc(c, &c->d_vox, vox.size() * sizeof(uint32_t))) ||
@@ -380,7 +382,7 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
         (rc = dev_alloc(c, &c->d_bc, sizeof(lbm::BcState))) ||
         (rc = dev_alloc(c, &c->d_red_partials, (size_t)nb_red * sizeof(double))) ||
         (rc = dev_alloc(c, &c->d_red_counter, sizeof(unsigned))) ||
-        (rc = dev_alloc(c, &c->d_step_counter, sizeof(unsigned))) ||
+        (rc = dev_alloc(c, &c->d_parts, (size_t)2 * c->L.part_stride * sizeof(double))) ||
         (rc = dev_alloc(c, &c->d_mon_partials, (size_t)5 * nb_mon * sizeof(double))) ||
         (rc = dev_alloc(c, &c->d_mon_counter, sizeof(unsigned))) ||
         (rc = dev_alloc(c, &c->d_mon, sizeof(lbm::MonitorOut)))) {
@@ -399,7 +401,6 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
     if (e == cudaSuccess && windows)
         e = lbm::launch_build_windows(c->d_grid, c->d_vox, 0u, n, c->L.ns, nx, ny, nz, 0u, c->d_win, c->d_nodew, 0);
     if (e == cudaSuccess) e = cudaMemset(c->d_red_counter, 0, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemset(c->d_step_counter, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(c->d_mon_counter, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(c->f[0], 0, fbytes);
     if (e == cudaSuccess) e = cudaMemset(c->f[1], 0, fbytes);
@@ -552,10 +553,10 @@ int lbm_time_kernels(lbm_ctx* c, int n, float* ms_step, float* ms_inlet) {
         LBM_CUDA(c, cudaEventRecord(ev[2 * k], c->stream));
         if (c->aa) {
             LBM_CUDA(c, lbm::launch_aa_step(c->prec, c->f[0], (k & 1) == 0, c->cur, c->L, c->relax, c->d_bc,
-                                            c->d_red_partials, c->d_step_counter, c->stream));
+                                            c->d_parts, c->stream));
         } else {
             LBM_CUDA(c, lbm::launch_step_cfg(c->prec, c->step_cfg, state_f(c), c->f[c->cur ^ 1], c->cur, c->L,
-                                             c->relax, c->d_bc, c->d_red_partials, c->d_step_counter, c->stream));
+                                             c->relax, c->d_bc, c->d_parts, c->stream));
         }
         LBM_CUDA(c, cudaEventRecord(ev[2 * k + 1], c->stream));
         c->cur ^= 1;

@@ -212,7 +212,9 @@ __device__ __forceinline__ void encode_node(const typename S::M* d, uint32_t see
 // FP64 scalars of the boundary conditions, in device memory so that captured
 // graphs pick up new values.  All densities are stored as drho = rho - 1.
 // drho_in[c] is the inlet density (Eq. potential) for the step that reads
-// distribution buffer c; the step that reads buffer c produces drho_in[c ^ 1].
+// distribution buffer c.  A step leaves the parts of the next step's inlet sum
+// (parts[c] of them, c the buffer the next step reads) and the next step adds them
+// and records drho_in[c]; parts[c] = 0 means that drho_in[c] is already set.
 struct BcState {
     double Q;              // prescribed inlet flux (Eq. flux)
     double drho_in_fixed;  // inlet density when the inlet is in pressure mode
@@ -227,6 +229,7 @@ struct BcState {
     int ref_cur;
     // stochastic-rounding seed of the step reading buffer c (16-bit formats)
     uint32_t sr_seed[2];
+    int parts[2];
     int pad2_;
 };
 // The host writes only the fields before drho_in; the rest is device-owned.

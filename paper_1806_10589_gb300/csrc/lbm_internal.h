@@ -16,6 +16,7 @@ struct DevLattice {
     int64_t a_in;       // inlet pore nodes: pore indices [0, a_in)
     int64_t a_out;      // outlet pore nodes: pore indices [n - a_out, n)
     int64_t a_01;       // pore nodes on the planes z = 0 and z = 1: indices [0, a_01)
+    int64_t part_stride;  // inlet-sum parts per buffer parity (doubles)
     int nx, ny, nz;     // voxel box
     int sy, sz;         // strides of the padded id grid: (nx+2), (nx+2)(ny+2)
     const uint32_t* vox;  // [n] padded linear voxel index of each pore node
@@ -56,10 +57,12 @@ struct MonitorOut {
 // over the inlet plane; used whenever the state or Q changes outside a step.
 cudaError_t launch_inlet_reduce(int prec, const void* fin, int slot, const DevLattice& L, BcState* bc,
                                 double* partials, unsigned* counter, cudaStream_t st);
-// One full step fin (parity `slot`) -> fout; also produces drho_in[slot ^ 1].
+// One full step fin (parity `slot`) -> fout; also leaves the parts of the inlet sum
+// of the step after it in partials (two parities of L.part_stride doubles).
 cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const DevLattice& L, Relax r,
-                        BcState* bc, double* partials, unsigned* counter, cudaStream_t st);
-int step_reduce_blocks(const DevLattice& L);
+                        BcState* bc, double* partials, cudaStream_t st);
+// drho_in[slot] from the parts the last step left, if it left any.
+cudaError_t launch_inlet_finish(const DevLattice& L, BcState* bc, int slot, const double* partials, cudaStream_t st);
 
 // Step-kernel variant: 0 = one thread per node (k_step); 1 / 2 = persistent
 // cp.async-pipelined kernel (k_step_async) with 256 / 128-node tiles.
@@ -69,12 +72,12 @@ struct StepConfig {
 };
 cudaError_t configure_step(int prec, int variant, const DevLattice& L, StepConfig* cfg);
 cudaError_t launch_step_cfg(int prec, const StepConfig& cfg, const void* fin, void* fout, int slot,
-                            const DevLattice& L, Relax r, BcState* bc, double* partials, unsigned* counter,
+                            const DevLattice& L, Relax r, BcState* bc, double* partials,
                             cudaStream_t st);
 // AA pattern (single buffer): one odd (gather-scatter) or even
 // (node-local) step in place, and the layout swaps around a call.
 cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattice& L, Relax r, BcState* bc,
-                           double* partials, unsigned* counter, cudaStream_t st);
+                           double* partials, cudaStream_t st);
 cudaError_t launch_aa_swap(int prec, void* f, const DevLattice& L, cudaStream_t st);
 cudaError_t launch_aa_unstream(int prec, void* f, const DevLattice& L, const BcState* bc, cudaStream_t st);
 cudaError_t launch_monitors(int prec, const void* f, const DevLattice& L, const BcState* bc, double* partials,

@@ -7,7 +7,7 @@
 //                   forms the NEXT step's inlet density: every stored value that
 //                   the next step pulls into an inlet node's known sum (Eq.
 //                   inlet) is added, in FP64, by the node that produces it, then
-//                   a deterministic last-block finish writes drho_in[slot ^ 1].
+//                   deterministic per-warp parts that the next step adds.
 //   k_inlet_reduce  the same density by a pull over the inlet plane, for states
 //                   set from outside a step (creation, set_*, a new Q).
 //   k_step_aa       the same step on ONE buffer (AA pattern, FP64/FP32), with
@@ -309,6 +309,7 @@ k_inlet_reduce(const typename S::T* __restrict__ fin, int slot, DevLattice L, Bc
     s = block_sum<kReduceBlock>(s, sh);
     if (threadIdx.x == 0) {
         bc->drho_in[slot] = (bc->Q + s) / (double)L.a_in;
+        bc->parts[slot] = 0;
         *counter = 0u;
     }
 }
@@ -404,49 +405,69 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 #define LBM_STEP_PREFETCH 224
 #endif
 
-// End of a step, called by the blocks whose tile (number `tile`, of NT / 32 warps
-// of GROUP nodes each) holds plane z = 0 or z = 1 nodes: every warp stores its part
-// of the next inlet sum; the last tile adds the parts and writes the next density
-// (and the next rounding seed).  The parts are added in an order that does not
-// depend on NT -- part j on virtual lane j mod 256, then the trees of 8 virtual
-// warps, then one of the 8 sums -- so the block size does not change the result.
-template <class S, int NT, int GROUP = 32>
-__device__ __forceinline__ void finish_inlet(double part, int64_t tile, const DevLattice& L, BcState* bc, int slot,
-                                             double* __restrict__ partials, unsigned* __restrict__ counter, double* sh,
-                                             bool* last) {
+// The inlet sum of the next step leaves a step as parts, one per warp of the tiles
+// that hold plane z = 0 or z = 1 nodes (tile number `tile`, of NT / 32 warps), and
+// the blocks of the next step that hold inlet nodes add them while their gathers
+// are on the way.  (Adding them here, in the tile that finishes last, put a memory
+// fence, a ticket and a second round of loads at the end of every step: 8.5 us per
+// step of a 10k-node FP32 lattice against 6.7, 8.8 against 7.5 at 173k nodes, 11.0
+// against 9.1 at 365k.)
+template <class S, int NT>
+__device__ __forceinline__ void store_inlet_part(double part, int64_t tile, int64_t tiles, const DevLattice& L,
+                                                 BcState* bc, int slot, double* __restrict__ partials) {
     constexpr int W = NT / 32;
-    const unsigned tiles = (unsigned)((L.a_01 + W * GROUP - 1) / (W * GROUP));
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double v = warp_sum(part);
-    if (lane == 0) {
-        partials[tile * W + wid] = v;
-        __threadfence();
+    if ((threadIdx.x & 31) == 0) partials[(slot ^ 1) * L.part_stride + tile * W + (threadIdx.x >> 5)] = v;
+    if (tile == 0 && threadIdx.x == 0) {
+        bc->parts[slot ^ 1] = (int)(tiles * W);
+        if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
+    }
+}
+
+// Inlet density - 1 of this step, for every thread of a block that holds inlet
+// nodes; the block `first` records it.  The parts are added in an order that does
+// not depend on NT -- part j on virtual lane j mod 256, then the trees of 8 virtual
+// warps, then one of the 8 sums.
+template <class M, int NT>
+__device__ __forceinline__ M density_of_parts(const DevLattice& L, BcState* bc, int slot,
+                                              const double* __restrict__ partials, double* sh, bool first) {
+    constexpr int W = NT / 32;
+    const int n = bc->parts[slot];
+    if (n == 0) return M(bc->drho_in[slot]);
+    const double* p = partials + slot * L.part_stride;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int vw = wid; vw < 8; vw += W) {
+        double s = 0.0;
+        for (int j = vw * 32 + lane; j < n; j += 256) s += p[j];
+        s = warp_sum(s);
+        if (lane == 0) sh[vw] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        *last = atomicAdd(counter, 1u) == tiles - 1;
+    if (wid == 0) {
+        const double s = warp_sum(lane < 8 ? sh[lane] : 0.0);
+        if (lane == 0) {
+            const double drho = (bc->Q + s) / (double)L.a_in;
+            sh[8] = drho;
+            if (first) bc->drho_in[slot] = drho;
+        }
     }
     __syncthreads();
-    if (*last) {
-        __threadfence();
-        for (int vw = wid; vw < 8; vw += W) {
-            double s = 0.0;
-            for (unsigned j = vw * 32 + lane; j < tiles * W; j += 256) s += __ldcg(partials + j);
-            s = warp_sum(s);
-            if (lane == 0) sh[vw] = s;
-        }
-        __syncthreads();
-        if (wid == 0) {
-            const double s = warp_sum(lane < 8 ? sh[lane] : 0.0);
-            if (lane == 0) {
-                bc->drho_in[slot ^ 1] = (bc->Q + s) / (double)L.a_in;
-                if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
-                *counter = 0u;
-            }
-        }
-        __syncthreads();
-    }
+    return M(sh[8]);
+}
+
+template <class M, int NT>
+__device__ __forceinline__ M inlet_density(const DevLattice& L, BcState* bc, int slot, const double* __restrict__ partials,
+                                           double* sh, bool first) {
+    if (bc->inlet_mode) return M(bc->drho_in_fixed);
+    return density_of_parts<M, NT>(L, bc, slot, partials, sh, first);
+}
+
+// drho_in[slot] from its parts, for readers between steps (the 16-bit reference,
+// which takes it in pressure mode too).
+__global__ void __launch_bounds__(kReduceBlock)
+k_inlet_finish(DevLattice L, BcState* bc, int slot, const double* __restrict__ partials) {
+    __shared__ double sh[32];
+    density_of_parts<double, kReduceBlock>(L, bc, slot, partials, sh, true);
 }
 
 // WIN: pulls from the row windows, addressed as row 0 plus a 32-bit element
@@ -455,10 +476,9 @@ __device__ __forceinline__ void finish_inlet(double part, int64_t tile, const De
 template <class S, bool WIN = false, int NT = kBlock>
 __global__ void __launch_bounds__(NT, step_min_blocks<S>())
 k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates,
-       BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
+       BcState* bc, double* __restrict__ partials) {
     using M = typename S::M;
     __shared__ double sh[32];
-    __shared__ bool last;
     const int64_t i64 = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int i = (int)i64;
     double part = 0.0;
@@ -471,27 +491,33 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
         if (t < 19) l2_prefetch_range(P.in[0] + (int64_t)t * L.ns, s, kBlock, L.ns);
         else if (t == 19) l2_prefetch_range(WIN ? L.nodew : L.vox, s, kBlock, L.n & ~(int64_t)3);
     }
-    if (i64 < L.n) {
 #if LBM_L2_HINTS >= 2
-        const uint64_t pol_f = l2_policy_evict_first();
+    const uint64_t pol_f = l2_policy_evict_first();
 #else
-        const uint64_t pol_f = 0;
+    const uint64_t pol_f = 0;
 #endif
 #if LBM_L2_HINTS >= 1
-        const uint64_t pol_idx = l2_policy_evict_last();
+    const uint64_t pol_idx = l2_policy_evict_last();
 #else
-        const uint64_t pol_idx = 0;
+    const uint64_t pol_idx = 0;
 #endif
-        const uint32_t p = ld_index((WIN ? L.nodew : L.vox) + i, pol_idx);  // node word or padded voxel
-        const M r_own = WIN ? own_ref_word<S>(bc, L, p) : own_ref<S>(bc, L, p), g = own_slope<S>(bc);
-        const uint32_t seed = step_seed<S>(bc, slot);
-        M d[19];
+    uint32_t p = 0;  // node word or padded voxel
+    M r_own = M(0), drin = M(0);
+    uint32_t seed = 0;
+    M d[19];
+    if (i64 < L.n) {
+        p = ld_index((WIN ? L.nodew : L.vox) + i, pol_idx);  // node word or padded voxel
+        const M g = own_slope<S>(bc);
+        r_own = WIN ? own_ref_word<S>(bc, L, p) : own_ref<S>(bc, L, p);
+        seed = step_seed<S>(bc, slot);
         if constexpr (WIN) pull_step_win<S>(d, P, L, p, i, pol_f, r_own, g);
         else pull_step<S>(d, P, L, p, i, pol_f, pol_idx, r_own, g);
+    }
+    if ((int64_t)blockIdx.x * NT < L.a_in) drin = inlet_density<M, NT>(L, bc, slot, partials, sh, blockIdx.x == 0);
+    if (i64 < L.n) {
         if (i < L.a_in) {
             // Section 2: after streaming, before collision.  u_z from Eq. (inlet)
             // with the density of Eq. (potential); then the Appendix B closure.
-            const M drin = bc->inlet_mode ? M(bc->drho_in_fixed) : M(bc->drho_in[slot]);
             close_inlet(d, drin - inlet_known(d));
         } else if (i64 >= L.n - L.a_out) {
             const M uz = outlet_known(d) - M(bc->drho_out);
@@ -505,7 +531,8 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
             else part = next_inlet_part<S>(d, L, pv, i, r_own, seed);
         }
     }
-    if ((int64_t)blockIdx.x * NT < L.a_01) finish_inlet<S, NT>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * NT < L.a_01)
+        store_inlet_part<S, NT>(part, blockIdx.x, (L.a_01 + NT - 1) / NT, L, bc, slot, partials);
 }
 
 // ------------------------------------------------------ AA-pattern step ---
@@ -605,13 +632,14 @@ __device__ __forceinline__ uint64_t aa_index_policy() {
 template <class S, bool ODD, bool WIN = false, int NT = kBlock>
 __global__ void __launch_bounds__(NT, aa_min_blocks<S, ODD>())
 k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename S::M> rates,
-          BcState* bc, double* __restrict__ partials, unsigned* __restrict__ counter) {
+          BcState* bc, double* __restrict__ partials) {
     using M = typename S::M;
     __shared__ double sh[32];
-    __shared__ bool last;
     __shared__ int sid[ODD ? 18 : 1][NT];  // gather offset (WIN) or pore id per direction
     const int64_t i64 = (int64_t)blockIdx.x * NT + threadIdx.x;
-    const int i = (int)i64;
+    // threads past the last node of a gather-scatter launch load its values and write
+    // nothing: straight-line loads up to the barrier of inlet_density (0.9 us of 171)
+    const int i = ODD ? (int)min(i64, L.n - 1) : (int)i64;
     double part = 0.0;
     constexpr int kAhead = S::kRef ? LBM_AA16_PREFETCH : LBM_AA_PREFETCH;
     if constexpr (ODD && kAhead > 0 && NT == kBlock) {
@@ -623,14 +651,15 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
         if (t < 19) l2_prefetch_range(F.row[0] + (int64_t)t * L.ns, s, kBlock, L.ns);
         else if (t == 19) l2_prefetch_range(WIN ? L.nodew : L.vox, s, kBlock, L.n & ~(int64_t)3);
     }
-    if (i64 < L.n) {
-        M d[19];
+    M d[19];
+    M r_own = M(0), g = M(0), drin = M(0);
+    uint32_t seed = 0;
+    if (ODD || i64 < L.n) {
         // 16-bit formats: every stored value is encoded with the reference of the
         // plane of the node that holds it (the even step writes its own slots; the
         // odd step encodes a scattered value with its destination's plane), so a
         // value read from the neighbour x - xi_q decodes with r(z - xi_z).
-        M r_own = M(0), g = M(0);
-        const uint32_t seed = step_seed<S>(bc, slot);
+        seed = step_seed<S>(bc, slot);
         if constexpr (ODD && WIN) {
             const uint32_t word = ld_aa_index(L.nodew + i, aa_index_policy());
             r_own = own_ref_word<S>(bc, L, word);
@@ -664,8 +693,10 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
                 d[Q] = S::template dec<Q>(F.row[Q][i], r_own);
             });
         }
+    }
+    if ((int64_t)blockIdx.x * NT < L.a_in) drin = inlet_density<M, NT>(L, bc, slot, partials, sh, blockIdx.x == 0);
+    if (i64 < L.n) {
         if (i < L.a_in) {
-            const M drin = bc->inlet_mode ? M(bc->drho_in_fixed) : M(bc->drho_in[slot]);
             close_inlet(d, drin - inlet_known(d));
         } else if (i64 >= L.n - L.a_out) {
             close_outlet(d, outlet_known(d) - M(bc->drho_out));
@@ -714,7 +745,8 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
             });
         }
     }
-    if ((int64_t)blockIdx.x * NT < L.a_01) finish_inlet<S, NT>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * NT < L.a_01)
+        store_inlet_part<S, NT>(part, blockIdx.x, (L.a_01 + NT - 1) / NT, L, bc, slot, partials);
 }
 
 // ------------------------------------------- two nodes per thread (16-bit) ---
@@ -745,7 +777,7 @@ constexpr int kPair = kBlock / 2;  // threads per tile
 
 // Inlet and outlet closures of the nodes i0 < i1 of a thread (both planes are rare).
 __device__ __forceinline__ void close_nodes(F2* d, int64_t i0, int64_t i1, const DevLattice& L, const BcState* bc,
-                                            int slot) {
+                                            float drin) {
     if (i0 < L.a_in || i1 >= L.n - L.a_out) {
         float a[2][19];
 #pragma unroll
@@ -754,7 +786,6 @@ __device__ __forceinline__ void close_nodes(F2* d, int64_t i0, int64_t i1, const
         for (int k = 0; k < 2; ++k) {
             const int64_t i = k ? i1 : i0;
             if (i < L.a_in) {
-                const float drin = bc->inlet_mode ? float(bc->drho_in_fixed) : float(bc->drho_in[slot]);
                 close_inlet(a[k], drin - inlet_known(a[k]));
             } else if (i >= L.n - L.a_out) {
                 close_outlet(a[k], outlet_known(a[k]) - float(bc->drho_out));
@@ -792,10 +823,9 @@ __device__ __forceinline__ double inlet_part_nodes(const F2* d, int64_t i0, int6
 template <class S>
 __global__ void __launch_bounds__(kPair, LBM_PAIR_STEP_BLOCKS)
 k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float> rates, BcState* bc,
-            double* __restrict__ partials, unsigned* __restrict__ counter) {
+            double* __restrict__ partials) {
     using T = typename S::T;
     __shared__ double sh[32];
-    __shared__ bool last;
     {
         const int64_t s = ((int64_t)blockIdx.x + LBM_STEP_PREFETCH) * kBlock;
         const int t = (int)threadIdx.x;
@@ -804,13 +834,16 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
     }
     const int64_t i64 = (int64_t)blockIdx.x * kBlock + 2 * threadIdx.x;
     double part = 0.0;
+    const uint32_t i = (uint32_t)i64, ns = (uint32_t)L.ns;
+    float r0 = 0.f, r1 = 0.f;
+    uint32_t seed = 0;
+    F2 d[19];
     if (i64 < L.n) {
-        const uint32_t i = (uint32_t)i64, ns = (uint32_t)L.ns;
         const uint2 w = __ldg(reinterpret_cast<const uint2*>(L.nodew + i));
         const float g = own_slope<S>(bc);
-        const float r0 = own_ref_word<S>(bc, L, w.x), r1 = own_ref_word<S>(bc, L, w.y);
-        const uint32_t seed = step_seed<S>(bc, slot);
-        F2 d[19];
+        r0 = own_ref_word<S>(bc, L, w.x);
+        r1 = own_ref_word<S>(bc, L, w.y);
+        seed = step_seed<S>(bc, slot);
         {
             float v[2][19];
             split(dec2<S, 0>(widen2<S>(__ldg(reinterpret_cast<const uint32_t*>(P.in[0] + i))),
@@ -828,7 +861,12 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
 #pragma unroll
             for (int q = 0; q < 19; ++q) d[q] = f2(v[0][q], v[1][q]);
         }
-        close_nodes(d, i64, i64 + 1, L, bc, slot);
+    }
+    float drin = 0.f;
+    if ((int64_t)blockIdx.x * kBlock < L.a_in)
+        drin = inlet_density<float, kPair>(L, bc, slot, partials, sh, blockIdx.x == 0);
+    if (i64 < L.n) {
+        close_nodes(d, i64, i64 + 1, L, bc, drin);
         collide2<true>(d, rates.sp, rates.sm);
         const F2 nr = f2(-1024.0f * r0, -1024.0f * r1);
         const uint32_t u = sr_key2(seed, i, i + 1u);
@@ -838,7 +876,8 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
         });
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair, 64>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * kBlock < L.a_01)
+        store_inlet_part<S, kPair>(part, blockIdx.x, (L.a_01 + kBlock - 1) / kBlock, L, bc, slot, partials);
 }
 
 // Gather-scatter launch: thread t of a warp owns the nodes 64 w + t and
@@ -849,9 +888,8 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
 template <class S>
 __global__ void __launch_bounds__(kPair, LBM_PAIR_ODD_BLOCKS)
 k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float> rates, BcState* bc,
-              double* __restrict__ partials, unsigned* __restrict__ counter) {
+              double* __restrict__ partials) {
     __shared__ double sh[32];
-    __shared__ bool last;
     // gather offsets: the scatter destination of q is the gather source of opp(q)
     __shared__ uint32_t soff[2][18][kPair];
     {
@@ -862,17 +900,20 @@ k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float
     }
     const int64_t i64 = (int64_t)blockIdx.x * kBlock + 2 * (threadIdx.x & ~31u) + (threadIdx.x & 31u);
     double part = 0.0;
+    const uint32_t ns = (uint32_t)L.ns;
+    const uint32_t i = (uint32_t)i64;
+    // an absent second node repeats the first one's reads and writes nothing
+    const bool two = i64 + 32 < L.n;
+    const uint32_t i1 = two ? i + 32u : i;
+    float g = 0.f, r0 = 0.f, r1 = 0.f;
+    uint32_t seed = 0;
+    F2 d[19];
     if (i64 < L.n) {
-        const uint32_t ns = (uint32_t)L.ns;
-        const uint32_t i = (uint32_t)i64;
-        // an absent second node repeats the first one's reads and writes nothing
-        const bool two = i64 + 32 < L.n;
-        const uint32_t i1 = two ? i + 32u : i;
         const uint32_t w0 = __ldg(L.nodew + i), w1 = __ldg(L.nodew + i1);
-        const float g = own_slope<S>(bc);
-        const float r0 = own_ref_word<S>(bc, L, w0), r1 = own_ref_word<S>(bc, L, w1);
-        const uint32_t seed = step_seed<S>(bc, slot);
-        F2 d[19];
+        g = own_slope<S>(bc);
+        r0 = own_ref_word<S>(bc, L, w0);
+        r1 = own_ref_word<S>(bc, L, w1);
+        seed = step_seed<S>(bc, slot);
         {
             float v[2][19];
 #pragma unroll
@@ -890,7 +931,12 @@ k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float
 #pragma unroll
             for (int q = 0; q < 19; ++q) d[q] = f2(v[0][q], v[1][q]);
         }
-        close_nodes(d, i64, i64 + 32, L, bc, slot);
+    }
+    float drin = 0.f;
+    if ((int64_t)blockIdx.x * kBlock < L.a_in)
+        drin = inlet_density<float, kPair>(L, bc, slot, partials, sh, blockIdx.x == 0);
+    if (i64 < L.n) {
+        close_nodes(d, i64, i64 + 32, L, bc, drin);
         collide2<false>(d, rates.sp, rates.sm);
         const float m0 = -1024.0f * r0, m1 = -1024.0f * r1;
         const uint32_t u = sr_key2(seed, i, i + 32u);
@@ -922,16 +968,16 @@ k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float
             return cz(decltype(qc)::value) < 0 ? r - g : r;
         });
     }
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair, 64>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * kBlock < L.a_01)
+        store_inlet_part<S, kPair>(part, blockIdx.x, (L.a_01 + kBlock - 1) / kBlock, L, bc, slot, partials);
 }
 
 // Node-local launch: neighbouring nodes on a thread, one 4-byte load and store per row.
 template <class S>
 __global__ void __launch_bounds__(kPair, LBM_PAIR_EVEN_BLOCKS)
 k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<float> rates, BcState* bc,
-               double* __restrict__ partials, unsigned* __restrict__ counter) {
+               double* __restrict__ partials) {
     __shared__ double sh[32];
-    __shared__ bool last;
     if constexpr (LBM_PAIR_EVEN_PREFETCH > 0) {
         const int64_t s = ((int64_t)blockIdx.x + LBM_PAIR_EVEN_PREFETCH) * kBlock;
         const int t = (int)threadIdx.x;
@@ -940,22 +986,30 @@ k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<floa
     }
     const int64_t i64 = (int64_t)blockIdx.x * kBlock + 2 * threadIdx.x;
     double part = 0.0;
+    const uint32_t i = (uint32_t)i64;
+    float r0 = 0.f, r1 = 0.f;
+    uint32_t seed = 0;
+    F2 d[19];
     if (i64 < L.n) {
-        const uint32_t i = (uint32_t)i64;
         uint32_t raw[19];
         for_q(AllQ{}, [&](auto qc) {
             constexpr int Q = decltype(qc)::value;
             raw[Q] = *reinterpret_cast<const uint32_t*>(F.row[Q] + i);
         });
         const uint2 w = __ldg(reinterpret_cast<const uint2*>(L.nodew + i));
-        const float r0 = own_ref_word<S>(bc, L, w.x), r1 = own_ref_word<S>(bc, L, w.y);
-        const uint32_t seed = step_seed<S>(bc, slot);
-        F2 d[19];
+        r0 = own_ref_word<S>(bc, L, w.x);
+        r1 = own_ref_word<S>(bc, L, w.y);
+        seed = step_seed<S>(bc, slot);
         for_q(AllQ{}, [&](auto qc) {
             constexpr int Q = decltype(qc)::value;
             d[Q] = dec2<S, Q>(widen2<S>(raw[Q]), f2(float(wq(Q)) * r0, float(wq(Q)) * r1));
         });
-        close_nodes(d, i64, i64 + 1, L, bc, slot);
+    }
+    float drin = 0.f;
+    if ((int64_t)blockIdx.x * kBlock < L.a_in)
+        drin = inlet_density<float, kPair>(L, bc, slot, partials, sh, blockIdx.x == 0);
+    if (i64 < L.n) {
+        close_nodes(d, i64, i64 + 1, L, bc, drin);
         collide2<false>(d, rates.sp, rates.sm);
         const F2 nr = f2(-1024.0f * r0, -1024.0f * r1);
         const uint32_t u = sr_key2(seed, i, i + 1u);
@@ -967,7 +1021,8 @@ k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<floa
         });
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
-    if ((int64_t)blockIdx.x * kBlock < L.a_01) finish_inlet<S, kPair, 64>(part, blockIdx.x, L, bc, slot, partials, counter, sh, &last);
+    if ((int64_t)blockIdx.x * kBlock < L.a_01)
+        store_inlet_part<S, kPair>(part, blockIdx.x, (L.a_01 + kBlock - 1) / kBlock, L, bc, slot, partials);
 }
 
 // Pull layout <-> layout S: swap F[q][x] and F[opp q][x] at every node.
@@ -1133,8 +1188,7 @@ __device__ __forceinline__ void read_vals(typename S::M* d, const unsigned char*
 
 template <class S, int NT>
 __global__ void __launch_bounds__(NT)
-k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates, BcState* bc, double* __restrict__ partials,
-             unsigned* __restrict__ counter) {
+k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates, BcState* bc, double* __restrict__ partials) {
     using M = typename S::M;
     constexpr int SB = AsyncSlot<S>::kBytes;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1142,7 +1196,6 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<type
     unsigned char* vals0 = smem + (size_t)18 * NT * 4;
     unsigned char* vals1 = vals0 + (size_t)19 * NT * SB;
     __shared__ double sh[32];
-    __shared__ bool last;
 
     const int64_t ntiles = (L.n + NT - 1) / NT;
     const int64_t nt01 = (L.a_01 + NT - 1) / NT;
@@ -1165,6 +1218,8 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<type
     cp_async_commit();
     if (t + G < ntiles && node(t + G) < L.n) issue_ids<NT>(ids, L, p_next, pol_idx);
     cp_async_commit();
+    M drin = M(0);
+    if (t * NT < L.a_in) drin = inlet_density<M, NT>(L, bc, slot, partials, sh, t == 0);
 
     for (int k = 0; t < ntiles; ++k, t += G) {
         unsigned char* vcur = (k & 1) ? vals1 : vals0;
@@ -1188,7 +1243,6 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<type
             M d[19];
             read_vals<S, NT>(d, vcur, hi_cur, nb_cur, r_own, g);
             if (i < L.a_in) {
-                const M drin = bc->inlet_mode ? M(bc->drho_in_fixed) : M(bc->drho_in[slot]);
                 close_inlet(d, drin - inlet_known(d));
             } else if (i64 >= L.n - L.a_out) {
                 const M uz = outlet_known(d) - M(bc->drho_out);
@@ -1202,7 +1256,7 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<type
             if (i64 < L.a_01) part = next_inlet_part<S>(d, L, p_cur, i, r_own, seed);
         }
         if (t < nt01)  // tile holds plane z = 0 / z = 1 nodes (block-uniform)
-            finish_inlet<S, NT>(part, t, L, bc, slot, partials, counter, sh, &last);
+            store_inlet_part<S, NT>(part, t, nt01, L, bc, slot, partials);
         hi_cur = hi_next;
         nb_cur = nb_next;
         p_cur = p_next;
@@ -1498,7 +1552,6 @@ cudaError_t launch_build_windows(const int* grid, const uint32_t* vox, uint32_t 
 
 int elem_size(int prec) { return prec == 0 ? 8 : prec == 1 ? 4 : 2; }
 int inlet_reduce_blocks(const DevLattice& L) { return (int)blocks_for(L.a_in, kReduceBlock); }
-int step_reduce_blocks(const DevLattice& L) { return (int)blocks_for(L.a_01, kBlock); }
 int monitor_blocks(const DevLattice& L) { return (int)blocks_for(L.n, kReduceBlock); }
 
 cudaError_t launch_inlet_reduce(int prec, const void* fin, int slot, const DevLattice& L, BcState* bc,
@@ -1512,7 +1565,7 @@ cudaError_t launch_inlet_reduce(int prec, const void* fin, int slot, const DevLa
 }
 
 cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const DevLattice& L, Relax r,
-                        BcState* bc, double* partials, unsigned* counter, cudaStream_t st) {
+                        BcState* bc, double* partials, cudaStream_t st) {
     return dispatch(prec, [&](auto s) {
         using S = decltype(s);
         using M = typename S::M;
@@ -1526,24 +1579,21 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
         if (L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64"))
         {
             if constexpr (S::kRef)
-                k_step_pair<S><<<blocks_for(L.n, kBlock), kPair, 0, st>>>(P, slot, L, make_rates<float>(r.sp, r.sm), bc,
-                                                                          partials, counter);
+                k_step_pair<S><<<blocks_for(L.n, kBlock), kPair, 0, st>>>(P, slot, L, make_rates<float>(r.sp, r.sm), bc, partials);
             else if (sizeof(M) == 8 && L.n < kSmallNodes)
                 k_step<S, true, kSmallBlock><<<blocks_for(L.n, kSmallBlock), kSmallBlock, 0, st>>>(
-                    P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials, counter);
+                    P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
             else
-                k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc,
-                                                                             partials, counter);
+                k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
         } else
-            k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials,
-                                                                   counter);
+            k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
         return cudaGetLastError();
     });
 }
 
 template <class S, int NT>
 cudaError_t launch_async_t(const void* fin, void* fout, int slot, const DevLattice& L, Relax r, BcState* bc,
-                           double* partials, unsigned* counter, cudaStream_t st, int grid) {
+                           double* partials, cudaStream_t st, int grid) {
     using T = typename S::T;
     using M = typename S::M;
     StepPtrs<T> P;
@@ -1552,7 +1602,7 @@ cudaError_t launch_async_t(const void* fin, void* fout, int slot, const DevLatti
         P.out[q] = (T*)fout + (int64_t)q * L.ns;
     }
     const size_t smem = async_smem_bytes<NT>(AsyncSlot<S>::kBytes);
-    k_step_async<S, NT><<<grid, NT, smem, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials, counter);
+    k_step_async<S, NT><<<grid, NT, smem, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
     return cudaGetLastError();
 }
 
@@ -1571,6 +1621,11 @@ cudaError_t config_async_t(int* grid, int64_t n) {
     const int64_t ntiles = (n + NT - 1) / NT;
     *grid = (int)std::min<int64_t>((int64_t)per_sm * sms, ntiles);
     return cudaSuccess;
+}
+
+cudaError_t launch_inlet_finish(const DevLattice& L, BcState* bc, int slot, const double* partials, cudaStream_t st) {
+    k_inlet_finish<<<1, kReduceBlock, 0, st>>>(L, bc, slot, partials);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_monitors(int prec, const void* f, const DevLattice& L, const BcState* bc, double* partials,
@@ -1648,7 +1703,7 @@ cudaError_t launch_decode(int prec, const void* f, const DevLattice& L, const Bc
 }
 
 cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattice& L, Relax r, BcState* bc,
-                           double* partials, unsigned* counter, cudaStream_t st) {
+                           double* partials, cudaStream_t st) {
     return dispatch(prec, [&](auto s) {
         using S = decltype(s);
         using M = typename S::M;
@@ -1663,26 +1718,24 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
             if constexpr (S::kRef) {
                 if (win) {
                     if (odd)
-                        k_aa_odd_pair<S><<<nb, kPair, 0, st>>>((typename S::T*)f, slot, L, rates, bc, partials, counter);
+                        k_aa_odd_pair<S><<<nb, kPair, 0, st>>>((typename S::T*)f, slot, L, rates, bc, partials);
                     else
-                        k_aa_even_pair<S><<<nb, kPair, 0, st>>>(F, slot, L, rates, bc, partials, counter);
+                        k_aa_even_pair<S><<<nb, kPair, 0, st>>>(F, slot, L, rates, bc, partials);
                     return cudaGetLastError();
                 }
             } else if (win && sizeof(M) == 8 && L.n < kSmallNodes) {
                 const unsigned nbs = blocks_for(L.n, kSmallBlock);
                 if (odd)
-                    k_step_aa<S, true, true, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials,
-                                                                                       counter);
+                    k_step_aa<S, true, true, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
                 else
-                    k_step_aa<S, false, false, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc,
-                                                                                         partials, counter);
+                    k_step_aa<S, false, false, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
                 return cudaGetLastError();
             } else if (odd && win) {
-                k_step_aa<S, true, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials, counter);
+                k_step_aa<S, true, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
                 return cudaGetLastError();
             }
-            if (odd) k_step_aa<S, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials, counter);
-            else k_step_aa<S, false><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials, counter);
+            if (odd) k_step_aa<S, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+            else k_step_aa<S, false><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
             return cudaGetLastError();
         }
     });
@@ -1717,15 +1770,15 @@ cudaError_t configure_step(int prec, int variant, const DevLattice& L, StepConfi
 }
 
 cudaError_t launch_step_cfg(int prec, const StepConfig& cfg, const void* fin, void* fout, int slot,
-                            const DevLattice& L, Relax r, BcState* bc, double* partials, unsigned* counter,
+                            const DevLattice& L, Relax r, BcState* bc, double* partials,
                             cudaStream_t st) {
-    if (cfg.variant == 0) return launch_step(prec, fin, fout, slot, L, r, bc, partials, counter, st);
+    if (cfg.variant == 0) return launch_step(prec, fin, fout, slot, L, r, bc, partials, st);
     return dispatch(prec, [&](auto s) {
         using S = decltype(s);
         if (cfg.variant == 1)
-            return launch_async_t<S, 256>(fin, fout, slot, L, r, bc, partials, counter, st, cfg.grid);
+            return launch_async_t<S, 256>(fin, fout, slot, L, r, bc, partials, st, cfg.grid);
         if (cfg.variant == 2)
-            return launch_async_t<S, 128>(fin, fout, slot, L, r, bc, partials, counter, st, cfg.grid);
+            return launch_async_t<S, 128>(fin, fout, slot, L, r, bc, partials, st, cfg.grid);
         return cudaErrorInvalidValue;
     });
 }
