@@ -104,7 +104,7 @@ __host__ __device__ constexpr double mnorm2(int k) {
 
 // Bound by memory.  N_A and N_B are stored for the step, which would otherwise read
 // the 14 values again: 60 -> 68 bytes here and 268 -> 220 there per FP32 node; on a
-// 128x128x256 pack (1.6 M pores) the step took 72.5 us and takes 65.7.  Two nodes
+// 128x128x256 pack (1.6 M pores) the step went from 72.5 to 65.7 us.  Two nodes
 // per thread with 8-byte loads measured slower (23.4 against 20.2 us here).
 template <class T>
 __global__ void __launch_bounds__(kCB)
@@ -193,12 +193,15 @@ struct ColorRows {
     T* bout[7];
 };
 
+// Resident blocks per SM (FP32), measured on a 128x128x256 pack with the row windows:
+// 70.7, 64.2, 62.6 and 65.9 us per step at 3, 4, 5 and 6.
 #ifndef LBM_COLOR_MIN_BLOCKS
-#define LBM_COLOR_MIN_BLOCKS 4
+#define LBM_COLOR_MIN_BLOCKS 5
 #endif
 // LBM_COLOR_PREFETCH: the step asks L2 for the rows of the block that many
 // blocks ahead (bulk prefetch, nothing waited for); 0 = off.  Measured on the
-// 192x192x384 pack: 32 best (-5.6 % per step), 256 slower than none.
+// 192x192x384 pack: 32 best (-5.6 % per step), 256 slower than none; with the row
+// windows, 128x128x256 pack: 68.2 us with none, 64.4 at 16, 64.2 at 32, 63.6 at 128.
 #ifndef LBM_COLOR_PREFETCH
 #define LBM_COLOR_PREFETCH 32
 #endif
@@ -207,48 +210,89 @@ constexpr int color_min_blocks() {
     return sizeof(T) == 8 ? 1 : LBM_COLOR_MIN_BLOCKS;
 }
 
-// OFF32 (buffers of 19 ns < 2^32 elements): a gathered momentum value and a
-// pushed D3Q7 value are addressed as row 0 plus one 32-bit element offset, the
-// row chosen by a 32-bit select (as in the single-fluid gather-scatter step).
-template <class T, bool OFF32 = false>
+constexpr uint32_t kNoPush = 0xFFFFFFFFu;  // not an element of 7 ns < 2^32
+// Bit of the box faces that a node lies on: its neighbours beyond them are outside.
+enum : unsigned { kFaceX0 = 1, kFaceX1 = 2, kFaceY0 = 4, kFaceY1 = 8, kFaceZ0 = 16, kFaceZ1 = 32 };
+// Faces beyond which the pull source x - xi_q of a node lies.
+__host__ __device__ constexpr unsigned faces_of(int q) {
+    return (cx(q) > 0 ? kFaceX0 : cx(q) < 0 ? kFaceX1 : 0u) | (cy(q) > 0 ? kFaceY0 : cy(q) < 0 ? kFaceY1 : 0u) |
+           (cz(q) > 0 ? kFaceZ0 : cz(q) < 0 ? kFaceZ1 : 0u);
+}
+__global__ void k_color_faces(DevLattice L, uint8_t* __restrict__ faces) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= L.n) return;
+    const uint32_t p = L.vox[i], sy = (uint32_t)L.sy, sz = (uint32_t)L.sz;
+    const int z = (int)(p / sz), y = (int)(p % sz / sy), x = (int)(p % sy);
+    faces[i] = (uint8_t)((x == 1 ? kFaceX0 : 0u) | (x == L.nx ? kFaceX1 : 0u) | (y == 1 ? kFaceY0 : 0u) |
+                         (y == L.ny ? kFaceY1 : 0u) | (z == 1 ? kFaceZ0 : 0u) | (z == L.nz ? kFaceZ1 : 0u));
+}
+
+// WIN (buffers of 19 ns < 2^32 elements, and a row-window table): the neighbours
+// come from the row windows and the node's face bits -- 9 loads where the id grid
+// takes 18, and 6 again for the push, whose destinations are staged in shared memory
+// here -- and a gathered or pushed value is addressed as row 0 plus one 32-bit
+// element offset.  Bound by the latency of the gathers behind the index loads (68 %
+// of DRAM bandwidth on the id grid at 64 registers); without the id loads the kernel
+// fits 48 registers, so 5 blocks per SM instead of 4: 65.5 -> 62.6 us on a
+// 128x128x256 pack (1.6 M pores), bitwise equal states.  Otherwise (19 ns >= 2^32 or
+// 2^27 windows and more) the id grid and 64-bit row pointers.
+template <class T, bool WIN = false>
 __global__ void __launch_bounds__(kCB, color_min_blocks<T>())
-k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, const ColorParams* __restrict__ prm,
-             Rates<T> rates, T alpha, T beta, T phi_s) {
+k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, const uint8_t* __restrict__ faces,
+             const ColorParams* __restrict__ prm, Rates<T> rates, T alpha, T beta, T phi_s) {
+    __shared__ uint32_t push[WIN ? 7 : 1][WIN ? kCB : 1];  // [Q]: push destination (element of the D3Q7 rows)
     const int64_t i64 = (int64_t)blockIdx.x * kCB + threadIdx.x;
     if constexpr (LBM_COLOR_PREFETCH > 0) {
         // threads 0..18: momentum rows, 19..20: N_A and N_B (rows of ns elements
-        // from row 0, as launched), 21: phi, 22: the voxel list cut to a multiple
-        // of 4 entries
+        // from row 0, as launched), 21: phi, 22: the node or voxel list cut to a
+        // multiple of 4 entries, 23: the face bits cut to a multiple of 16
         const int64_t s = ((int64_t)blockIdx.x + LBM_COLOR_PREFETCH) * kCB;
         const int t = (int)threadIdx.x;
         if (t < 19) l2_prefetch_range(R.fin[0] + (int64_t)t * L.ns, s, kCB, L.ns);
         else if (t < 21) l2_prefetch_range(R.nab[0] + (int64_t)(t - 19) * L.ns, s, kCB, L.ns);
         else if (t == 21) l2_prefetch_range(phi, s, kCB, L.ns);
-        else if (t == 22) l2_prefetch_range(L.vox, s, kCB, L.n & ~(int64_t)3);
+        else if (t == 22) l2_prefetch_range(WIN ? L.nodew : L.vox, s, kCB, L.n & ~(int64_t)3);
+        else if (WIN && t == 23) l2_prefetch_range(faces, s, kCB, L.n & ~(int64_t)15);
     }
     if (i64 >= L.n) return;
     const int i = (int)i64;
     const uint64_t pol = l2_policy_evict_last();  // index structures stay in L2
-    const uint32_t p = ld_hint(reinterpret_cast<const unsigned*>(L.vox) + i, pol);
     const T phi_own = phi[i];
-    T d[19];
-    T cgx = 0, cgy = 0, cgz = 0;
+    T d[19], ph[19];
     d[0] = R.fin[0][i];
-    for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
-        constexpr int Q = decltype(qc)::value + 1;
-        const int id = ld_hint(L.grid + (uint32_t)(p + (uint32_t)grid_off<Q>(L.sy, L.sz)), pol);
-        if constexpr (OFF32)
-            d[Q] = R.fin[0][id >= 0 ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)id
-                                    : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)i];
-        else
+    if constexpr (WIN) {
+        const uint32_t word = ld_hint(reinterpret_cast<const unsigned*>(L.nodew) + i, pol);
+        const unsigned face = __ldg(faces + i);
+        for_links(L.win, word, L.wy, L.wz, (uint32_t)i, [&](auto qc, bool pore, uint32_t id) {
+            constexpr int Q = decltype(qc)::value;
+            const uint32_t ns = (uint32_t)L.ns;
+            d[Q] = R.fin[0][pore ? (uint32_t)Q * ns + id : (uint32_t)opp(Q) * ns + (uint32_t)i];
+            ph[Q] = pore ? phi[id] : ((face & faces_of(Q)) ? phi_own : phi_s);
+            if constexpr (Q <= 6) {
+                // the push of opp(Q) goes to this neighbour: a pore, bounce-back from a
+                // solid voxel or lateral box face, or lost through the inlet or outlet
+                uint32_t to = pore ? (uint32_t)opp(Q) * ns + id : (uint32_t)Q * ns + (uint32_t)i;
+                if (cz(Q) != 0 && !pore && (face & faces_of(Q))) to = kNoPush;
+                push[opp(Q)][threadIdx.x] = to;
+            }
+        });
+    } else {
+        const uint32_t p = ld_hint(reinterpret_cast<const unsigned*>(L.vox) + i, pol);
+        for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
+            constexpr int Q = decltype(qc)::value + 1;
+            const int id = ld_hint(L.grid + (uint32_t)(p + (uint32_t)grid_off<Q>(L.sy, L.sz)), pol);
             d[Q] = id >= 0 ? R.fin[Q][id] : R.fin[opp(Q)][i];
+            ph[Q] = id >= 0 ? phi[id] : (id == SOLID ? phi_s : phi_own);  // box faces: own phi
+        });
+    }
+    T cgx = 0, cgy = 0, cgz = 0;
+    for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
         // colour-gradient neighbour x + xi_opp(Q) is the pull source of Q
-        const T ph = id >= 0 ? phi[id] : (id == SOLID ? phi_s : phi_own);  // box faces: own phi
-        constexpr int Rq = opp(Q);  // this neighbour sits at x + xi_Rq
+        constexpr int Q = decltype(qc)::value + 1, Rq = opp(Q);
         const T wq3 = T(3.0 * wq(Rq));
-        if (cx(Rq)) cgx += wq3 * T(cx(Rq)) * ph;
-        if (cy(Rq)) cgy += wq3 * T(cy(Rq)) * ph;
-        if (cz(Rq)) cgz += wq3 * T(cz(Rq)) * ph;
+        if (cx(Rq)) cgx += wq3 * T(cx(Rq)) * ph[Q];
+        if (cy(Rq)) cgy += wq3 * T(cy(Rq)) * ph[Q];
+        if (cz(Rq)) cgz += wq3 * T(cz(Rq)) * ph[Q];
     });
     if (i < L.a_in) {
         close_inlet(d, T(prm->drho_in) - inlet_known(d));
@@ -280,7 +324,8 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
     // D3Q7 mass transport with recolouring (push); destinations looked up again
     const T na = R.nab[0][j], nb = R.nab[1][j];
     const bool inlet = j < L.a_in, outlet = (int64_t)j >= L.n - L.a_out;
-    const uint32_t ps = ld_hint(reinterpret_cast<const unsigned*>(L.vox) + j, pol);
+    uint32_t ps = 0;
+    if constexpr (!WIN) ps = ld_hint(reinterpret_cast<const unsigned*>(L.vox) + j, pol);
     for_q(std::make_integer_sequence<int, 7>{}, [&](auto qc) {
         constexpr int Q = decltype(qc)::value;
         const T xu = T(cx(Q)) * jx + T(cy(Q)) * jy + T(cz(Q)) * jz;
@@ -290,17 +335,16 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
         if constexpr (Q == 0) {
             R.aout[0][j] = va;
             R.bout[0][j] = vb;
+        } else if constexpr (WIN) {
+            const uint32_t off = *(volatile uint32_t*)&push[Q][threadIdx.x];
+            if (off != kNoPush) {
+                R.aout[0][off] = va;
+                R.bout[0][off] = vb;
+            }
         } else {
             // push destination x + xi_Q is the pull source of opp(Q)
             const int id = ld_hint(L.grid + (uint32_t)(ps + (uint32_t)grid_off<opp(Q)>(L.sy, L.sz)), pol);
-            if constexpr (OFF32) {
-                if (id != ZOUT) {  // a pore, or bounce-back from a solid voxel or lateral box face
-                    const uint32_t off = id >= 0 ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)id
-                                                 : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)j;
-                    R.aout[0][off] = va;
-                    R.bout[0][off] = vb;
-                }
-            } else if (id >= 0) {
+            if (id >= 0) {
                 R.aout[Q][id] = va;
                 R.bout[Q][id] = vb;
             } else if (id != ZOUT) {  // solid voxel or lateral box face: bounce back
@@ -407,6 +451,9 @@ struct lbm_color {
     int cur = 0;
     uint32_t* d_vox = nullptr;
     int* d_grid = nullptr;
+    uint2* d_win = nullptr;      // row windows, node words and face bits; null for the id-grid form
+    uint32_t* d_nodew = nullptr;
+    uint8_t* d_faces = nullptr;
     int64_t* d_voxel = nullptr;  // unpadded voxel of each pore node
     lbm::ColorParams h_prm{};
     lbm::ColorParams* d_prm = nullptr;
@@ -460,6 +507,9 @@ void crelease(lbm_color* c) {
     cudaFree(c->nab);
     cudaFree(c->d_vox);
     cudaFree(c->d_grid);
+    cudaFree(c->d_win);
+    cudaFree(c->d_nodew);
+    cudaFree(c->d_faces);
     cudaFree(c->d_voxel);
     cudaFree(c->d_prm);
     cudaFree(c->d_partials);
@@ -500,11 +550,13 @@ int cstep_once(lbm_color* c) {
             R.aout[q] = (T*)c->A[k ^ 1] + (int64_t)q * c->L.ns;
             R.bout[q] = (T*)c->B[k ^ 1] + (int64_t)q * c->L.ns;
         }
-        if (19 * (uint64_t)c->L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_COLOR_ADDR64"))
-            lbm::k_color_step<T, true><<<nb, lbm::kCB, 0, c->stream>>>(
-                R, (const T*)c->phi, c->L, c->d_prm, lbm::make_rates<T>(c->sp, c->sm), (T)c->alpha, (T)c->beta, (T)c->phi_s);
-        else
-            lbm::k_color_step<T><<<nb, lbm::kCB, 0, c->stream>>>(R, (const T*)c->phi, c->L, c->d_prm, lbm::make_rates<T>(c->sp, c->sm), (T)c->alpha, (T)c->beta, (T)c->phi_s);
+        const auto launch = [&](auto kernel) {
+            kernel<<<nb, lbm::kCB, 0, c->stream>>>(R, (const T*)c->phi, c->L, c->d_faces, c->d_prm,
+                                                   lbm::make_rates<T>(c->sp, c->sm), (T)c->alpha, (T)c->beta,
+                                                   (T)c->phi_s);
+        };
+        if (c->L.win && !std::getenv("GB300_LBM_COLOR_ADDR64")) launch(lbm::k_color_step<T, true>);
+        else launch(lbm::k_color_step<T, false>);
         return cudaGetLastError();
     });
     COLOR_CUDA(c, e);
@@ -582,6 +634,13 @@ int lbm_color_create(const uint8_t* mask, int nx, int ny, int nz, double tau, do
     c->L.nz = nz;
     c->L.sy = (int)px;
     c->L.sz = (int)(px * py);
+    // row windows, where a window index fits the node's word and an element a 32-bit offset
+    const int64_t nwin = (int64_t)lbm::windows_per_row(nx) * py * pz;
+    const bool windows = nwin < (int64_t)1 << 27 && 19 * (uint64_t)c->L.ns <= 0xFFFFFFFFull;
+    if (windows) {
+        c->L.wy = lbm::windows_per_row(nx);
+        c->L.wz = c->L.wy * (int)py;
+    }
     const int es = precision == LBM_PREC_FP64 ? 8 : 4;
     const size_t fb = (size_t)19 * c->L.ns * es, ab = (size_t)7 * c->L.ns * es;
     cudaError_t e = cudaSuccess;
@@ -597,6 +656,11 @@ int lbm_color_create(const uint8_t* mask, int nx, int ny, int nz, double tau, do
     Al(&c->nab, (size_t)2 * c->L.ns * es);
     Al(&c->d_vox, vox.size() * 4);
     Al(&c->d_grid, grid.size() * 4);
+    if (windows) {
+        Al(&c->d_win, (size_t)nwin * sizeof(uint2));
+        Al(&c->d_nodew, (size_t)c->L.ns * sizeof(uint32_t));
+        Al(&c->d_faces, (size_t)c->L.ns);
+    }
     Al(&c->d_voxel, c->pore_voxel.size() * 8);
     Al(&c->d_prm, sizeof(lbm::ColorParams));
     Al(&c->d_partials, (size_t)((n + lbm::kCB - 1) / lbm::kCB + 1) * sizeof(double));
@@ -605,9 +669,17 @@ int lbm_color_create(const uint8_t* mask, int nx, int ny, int nz, double tau, do
     Al(&c->d_out, sizeof(double));
     c->L.vox = c->d_vox;
     c->L.grid = c->d_grid;
+    c->L.win = c->d_win;
+    c->L.nodew = c->d_nodew;
     c->h_prm = lbm::ColorParams{0.0, 0.0, 0.0, 1.0};
     if (e == cudaSuccess) e = cudaMemcpy(c->d_vox, vox.data(), vox.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_grid, grid.data(), grid.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && windows)
+        e = lbm::launch_build_windows(c->d_grid, c->d_vox, 0u, n, c->L.ns, nx, ny, nz, 0u, c->d_win, c->d_nodew, 0);
+    if (e == cudaSuccess && windows) {
+        lbm::k_color_faces<<<(unsigned)((n + 255) / 256), 256>>>(c->L, c->d_faces);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess)
         e = cudaMemcpy(c->d_voxel, c->pore_voxel.data(), c->pore_voxel.size() * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_prm, &c->h_prm, sizeof c->h_prm, cudaMemcpyHostToDevice);

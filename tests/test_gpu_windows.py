@@ -95,3 +95,26 @@ def test_inlet_density_of_parts_equals_the_plane_sum(shape, prec, tol, variant):
     (a, fa), (b, fb) = run(False), run(True)
     np.testing.assert_allclose(a, b, rtol=0, atol=tol)
     np.testing.assert_allclose(fa, fb, rtol=0, atol=tol * mask.shape[1] * mask.shape[2])
+
+
+@pytest.mark.parametrize("shape", [(1, 6, 5), (30, 1, 4), (31, 4, 3), (61, 5, 5), (92, 3, 4)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_colour_windows_equal_id_grid(monkeypatch, shape, prec):
+    """Colour step on the row windows and face bits against the id grid: boxes of one
+    voxel across, pores on every face and edge, runs across window borders."""
+    from paper_1806_10589_gb300 import ColorLattice
+
+    mask = random_mask(*shape, 0.3, 13)
+    phi = np.where(uniform_field(mask.shape, 5) > 0, 0.75, -0.5)
+
+    def run():
+        with ColorLattice(mask, 0.8, 0.01, 0.9, -0.5, prec) as c:
+            c.set_flux_bc(0.002, 1.0)
+            c.set_phase(phi)
+            c.step(6)
+            return c.state()
+
+    got = run()
+    monkeypatch.setenv("GB300_LBM_COLOR_ADDR64", "1")
+    for a, b in zip(got, run()):
+        np.testing.assert_array_equal(a, b)
