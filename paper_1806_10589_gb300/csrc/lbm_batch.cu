@@ -153,28 +153,32 @@ __device__ __forceinline__ typename S::M pull_b(const typename S::T* fin, int64_
 }
 
 // Same contribution rule as the single-lattice step (see lbm_kernels.cu).
-template <class S>
+// Sum: the pair kernel, where registers are short, adds in FP64 (63.8 against 64.9 us
+// per step of six packs); the others as the single lattice does (four packs with
+// edges 24..40: FP32 9.9 -> 8.6 us per step, FP16-dev 10.3 -> 9.2).
+template <class S, class Sum = InletSum<typename S::M>>
 __device__ __forceinline__ double next_inlet_part_b(const typename S::M* d, const int* __restrict__ grid,
                                                     const Member& m, int64_t p, int64_t il,
                                                     typename S::M r_own, uint32_t seed, int64_t i) {
-    double s = 0.0;
-    auto val = [&](auto qc) -> double {
+    using M = typename S::M;
+    Sum s;
+    auto val = [&](auto qc) -> M {
         constexpr int Q = decltype(qc)::value;
-        return (double)S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i)), r_own);
+        return S::template dec<Q>(S::template enc_sr<Q>(d[Q], r_own, sr_key<S>(seed, i)), r_own);
     };
     auto dest_is_pore = [&](auto qc) -> bool {
         constexpr int Q = decltype(qc)::value;
         return __ldg(grid + p + m.goff[opp(Q)]) >= 0;
     };
     if (il < m.a_in) {
-        for_q(std::integer_sequence<int, 0, 1, 2, 3, 4, 7, 8, 9, 10>{}, [&](auto qc) { s += val(qc); });
+        for_q(std::integer_sequence<int, 0, 1, 2, 3, 4, 7, 8, 9, 10>{}, [&](auto qc) { s.add(val(qc)); });
         for_q(std::integer_sequence<int, 5, 11, 14, 15, 18>{},
-              [&](auto qc) { if (!dest_is_pore(qc)) s += 2.0 * val(qc); });
+              [&](auto qc) { if (!dest_is_pore(qc)) s.add(M(2) * val(qc)); });
     } else {
         for_q(std::integer_sequence<int, 6, 12, 13, 16, 17>{},
-              [&](auto qc) { if (dest_is_pore(qc)) s += 2.0 * val(qc); });
+              [&](auto qc) { if (dest_is_pore(qc)) s.add(M(2) * val(qc)); });
     }
-    return s;
+    return s.value();
 }
 
 // Per-member reduction of `part` over the member's tiles [0, ntiles_member):
@@ -280,7 +284,7 @@ __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typena
             constexpr int Q = decltype(qc)::value;
             fout[(int64_t)Q * ns + i] = v;
         });
-        if (il < m.a_01) part = next_inlet_part_b<S>(d, K.grid, m, K.vox[i], il, r_own, seed, i);
+        if (il < m.a_01) part = next_inlet_part_b<S>(d, K.grid, m, WIN ? __ldg(K.vox + i) : p, il, r_own, seed, i);
     }
     batch_finish<S, COH>(part, slot, tile, mi, members, partials, counters, sh);
 }
@@ -394,7 +398,7 @@ k_batch_pair(const typename S::T* __restrict__ fin, typename S::T* __restrict__ 
 #pragma unroll
             for (int k = 0; k < 2; ++k)
                 if (il + k < m.a_01)
-                    part += next_inlet_part_b<S>(v[k], K.grid, m, K.vox[i64 + k], il + k, k ? r1 : r0, seed, i64 + k);
+                    part += next_inlet_part_b<S, SumF64>(v[k], K.grid, m, K.vox[i64 + k], il + k, k ? r1 : r0, seed, i64 + k);
         }
     }
     batch_finish<S, false>(part, slot, tile, mi, members, partials, counters, sh);

@@ -11,6 +11,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <type_traits>
 #include <utility>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -302,6 +303,38 @@ __device__ __forceinline__ void for_links(const uint2* __restrict__ win, uint32_
     row_links<-1, 1>(vmp, b, low, i, f);
     row_links<1, 1>(vpp, b, low, i, f);
 }
+
+// ------------------------------------------------------- inlet sums ---
+// Sum of a node's values that enter the next inlet sum.  FP32 values are added
+// without error in three FP32 words (two chained two-sums, Knuth's) and reach FP64
+// once per node: a conversion and an FP64 addition per value, at two FP64 operations
+// per clock and SM, made the inlet tiles the tail of every step of a small lattice
+// (61x67x72, 112 k nodes: 9.1 -> 8.0 us per step).
+struct SumF32 {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    __device__ __forceinline__ static void two_sum(float& s, float x, float& err) {
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+        s = t;
+    }
+    __device__ __forceinline__ void add(float x) {
+        float e, f;
+        two_sum(hi, x, e);
+        two_sum(mid, e, f);
+        lo = __fadd_rn(lo, f);
+    }
+    // an infinite or NaN sum has no error terms
+    __device__ __forceinline__ double value() const {
+        return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
+    }
+};
+struct SumF64 {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <class M>
+using InletSum = std::conditional_t<sizeof(M) == 8, SumF64, SumF32>;
 
 // ------------------------------------------------------- cache hints ---
 // L2 eviction-priority hints (PTX createpolicy / .L2::cache_hint): the streamed

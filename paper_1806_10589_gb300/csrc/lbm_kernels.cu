@@ -325,37 +325,10 @@ k_inlet_reduce(const typename S::T* __restrict__ fin, int slot, DevLattice L, Bc
 //   z = 1:  twice each xi_z = -1 value whose destination on z = 0 is a pore.
 // `val(Q)` returns the stored value of direction Q exactly as the next step
 // will decode it.
-//   FP32 values are added without error in three FP32 words (two chained two-sums,
-// Knuth's) and reach FP64 once per node: a conversion and an FP64 addition per
-// value, at two FP64 operations per clock and SM, made the inlet tiles the tail of
-// every step of a small lattice (61x67x72, 112 k nodes: 9.1 -> 8.0 us per step).
-struct SumF32 {
-    float hi = 0.f, mid = 0.f, lo = 0.f;
-    __device__ __forceinline__ static void two_sum(float& s, float x, float& err) {
-        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-        err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
-        s = t;
-    }
-    __device__ __forceinline__ void add(float x) {
-        float e, f;
-        two_sum(hi, x, e);
-        two_sum(mid, e, f);
-        lo = __fadd_rn(lo, f);
-    }
-    // an infinite or NaN sum has no error terms
-    __device__ __forceinline__ double value() const {
-        return isfinite(hi) ? (double)hi + ((double)mid + (double)lo) : (double)hi;
-    }
-};
-struct SumF64 {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double x) { s += x; }
-    __device__ __forceinline__ double value() const { return s; }
-};
 template <class S, class V>
 __device__ __forceinline__ double inlet_contribution(const DevLattice& L, uint32_t p, int i, V&& val) {
     using M = typename S::M;
-    std::conditional_t<sizeof(M) == 8, SumF64, SumF32> s;
+    InletSum<M> s;
     auto dest_is_pore = [&](auto qc) -> bool {
         constexpr int Q = decltype(qc)::value;  // destination i + xi_Q = pull source of opp(Q)
         return __ldg(L.grid + (uint32_t)(p + (uint32_t)L.goff[opp(Q)])) >= 0;
