@@ -29,13 +29,18 @@ namespace {
 constexpr int kBlock = 256;
 constexpr int kReduceBlock = 256;
 // Resident 256-thread blocks per SM the step kernel is compiled for (caps its
-// registers at 65536 / (256 * n)); FP64 arithmetic is left unconstrained.
+// registers at 65536 / (256 * n)); FP64 arithmetic is left unconstrained.  On the row
+// windows FP32 fits 48 registers without spills: 100 steps of a 100^3 pack 1142, 1101
+// and 1101 us at 4, 5 and 6 blocks, of a 180x160x200 one 5817, 5595 and 5640.
 #ifndef LBM_STEP_MIN_BLOCKS
 #define LBM_STEP_MIN_BLOCKS 4
 #endif
-template <class S>
+#ifndef LBM_STEP_WIN_BLOCKS
+#define LBM_STEP_WIN_BLOCKS 5
+#endif
+template <class S, bool WIN = false>
 constexpr int step_min_blocks() {
-    return sizeof(typename S::M) == 8 ? 1 : LBM_STEP_MIN_BLOCKS;
+    return sizeof(typename S::M) == 8 ? 1 : (WIN && !S::kRef) ? LBM_STEP_WIN_BLOCKS : LBM_STEP_MIN_BLOCKS;
 }
 
 template <int... Qs, class F>
@@ -447,7 +452,7 @@ k_inlet_finish(DevLattice L, BcState* bc, int slot, const double* __restrict__ p
 // offset (buffers of 19 ns < 2^32 elements), as in the gather-scatter AA step.  NT
 // nodes per block.
 template <class S, bool WIN = false, int NT = kBlock>
-__global__ void __launch_bounds__(NT, step_min_blocks<S>())
+__global__ void __launch_bounds__(NT, step_min_blocks<S, WIN>())
 k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates,
        BcState* bc, double* __restrict__ partials) {
     using M = typename S::M;
