@@ -69,7 +69,7 @@ def workload():
 
 # the step kernels and their launch configurations; the host API (lbm_api.cu)
 # only sequences launches and does not change the traffic of one
-STEP_KERNEL_SOURCES = ("lbm_device.cuh", "lbm_internal.h", "lbm_kernels.cu")
+STEP_KERNEL_SOURCES = ("lbm_device.cuh", "lbm_internal.h", "lbm_kernels.cu", "lbm_pair.cuh")
 
 
 def strip_c_comments(src):
@@ -97,7 +97,7 @@ def strip_c_comments(src):
     return "".join(out)
 
 
-BATCH_KERNEL_SOURCES = ("lbm_batch.cu", "lbm_device.cuh", "lbm_internal.h")
+BATCH_KERNEL_SOURCES = ("lbm_batch.cu", "lbm_device.cuh", "lbm_internal.h", "lbm_pair.cuh")
 PROFILE_BATCH = os.path.join(ROOT, "profiles", "k_batch_step_fp16_ensemble64.md")
 CONV_KERNEL_SOURCES = ("wsnet.cu", "tc_util.cuh")
 PROFILE_CONV = os.path.join(ROOT, "profiles", "k_conv_wgrad_bf16_32x32.md")
@@ -550,7 +550,7 @@ def run_ensemble(stream, prec="fp16dev", steps=2000, warmup=64, steady_steps=Tru
                          "frac": round(ach / peak, 4),
                          "traffic": profiled_traffic(kernel_sources_sha(BATCH_KERNEL_SOURCES), path=PROFILE_BATCH)
                          if best in (0, 1) else None,
-                         "kernel": {2: "k_batch_persistent", 3: "k_batch_persistent", 4: "k_batch_aa", 5: "k_batch_aa"}.get(best, "k_batch_step"),
+                         "kernel": {2: "k_batch_persistent", 3: "k_batch_persistent", 4: "k_batch_aa", 5: "k_batch_aa"}.get(best, "k_batch_pair"),
                          "kernel_ms": round(k_ms, 5), "bytes_per_unit": 2 * 19 * s},
             "autotune": {"chosen": BATCH_CONFIGS[best],
                          "ms_per_step": {BATCH_CONFIGS[c]: round(t, 5) for c, t in enumerate(trial_ms)}},
@@ -614,7 +614,9 @@ def run_two_fluid(stream, steps=500, warmup=20, total_steps=50000):
         c.step(total_steps - warmup - steps)
         q_in_end, rho_in_end = c.get_flux(4)
     n = int((mask == 0).sum())
-    unit = 82 * 4  # FP32 values per node and step as built: f 19+19, A/B 14+14, phase 1, pre-pass A/B 14 + phi 1
+    # FP32 values per node and step as built: f 19+19, A/B pushed 14, N_A, N_B and phi read 3; pre-pass A/B 14, phi,
+    # N_A and N_B written 3
+    unit = 72 * 4
     unit_min = 66 * 4  # a single pass: f 19+19, A/B 14+14
     peak, _ = measured_hbm_peak()
     ach = unit * n / (ms * 1e-3 / steps) / 1e9
@@ -630,7 +632,7 @@ def run_two_fluid(stream, steps=500, warmup=20, total_steps=50000):
                          "single_pass": {"bytes_per_unit": unit_min, "achieved": round(ach_min, 1),
                                          "frac": round(ach_min / peak, 4),
                                          "note": "against the 66 values a single-pass step must move; the "
-                                                 "pre-pass re-reads the 14 D3Q7 values and writes and reads phi"}},
+                                                 "pre-pass stores phi, N_A and N_B for the step"}},
             "inlet_flux_rel_err": abs(q_in - Q) / Q,
             "run_to_step": total_steps,
             "inlet_flux_rel_err_end": abs(q_in_end - Q) / Q, "rho_in_end": rho_in_end}
@@ -924,7 +926,7 @@ def conv_roofline(stream, side=64, batch=8, reps=20):
     return {"bound": "tensor", "unit": "TFLOP/s", "peak": peak, "peak_source": kind,
             "shape": "3x3x3 conv 32 -> 32 channels, %d x %d^3 voxels (BF16, FP32 accumulate)" % (batch, side),
             "flops_per_launch": flops, "per_kernel": per, "achieved": per["forward"]["achieved"],
-            "frac": per["forward"]["frac"], "kernel": "k_conv<32,32> (forward)",
+            "frac": per["forward"]["frac"], "kernel": "k_conv_march<32,32> (forward)",
             "traffic": profiled_traffic(kernel_sources_sha(CONV_KERNEL_SOURCES), path=PROFILE_CONV)}
 
 

@@ -383,7 +383,8 @@ int lbm_wsnet_train(lbm_wsnet* net, const uint8_t* masks, const float* targets, 
                     int nz, int epochs, int batch, float lr, const int* order, float* loss_history);
 /* Predicted fields (host, 4*nz*ny*nx floats) of one geometry; 0 at solids. */
 int lbm_wsnet_predict(lbm_wsnet* net, const uint8_t* mask, int nx, int ny, int nz, float* y);
-/* Free the activation buffers kept between calls (sized for the last batch and volume). */
+/* Free the activation buffers kept between calls (sized for the last batch and volume),
+ * and the scratch of up to 16 MB per device that lbm_conv3d_bf16 keeps between calls. */
 int lbm_wsnet_release_buffers(lbm_wsnet* net);
 int lbm_wsnet_destroy(lbm_wsnet* net);
 const char* lbm_wsnet_last_error(const lbm_wsnet* net);
