@@ -321,7 +321,8 @@ constexpr int batch_min_blocks() {
 // latencies, where one node per thread and the id grid (resident in L2) are
 // shorter.  Per step, FP16-dev, id grid against windows with pairs: 83,816 pores 9.3
 // and 10.0 us, 365,138 pores 11.3 and 11.2, 707,421 pores 19.1 and 15.4; FP32 8.8
-// and 9.1, 10.5 and 10.3, 22.1 and 20.8.
+// and 9.1, 10.5 and 10.3, 22.1 and 20.8 (before the id-grid form's inlet tiles got 0.7
+// to 1.4 us shorter, see next_inlet_part_b; from 1,216 tiles they hide behind the rest).
 #ifndef LBM_WINDOW_TILES
 #define LBM_WINDOW_TILES (8 * 152)
 #endif
