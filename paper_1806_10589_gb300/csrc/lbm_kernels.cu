@@ -436,8 +436,11 @@ __device__ __forceinline__ M density_of_parts(const DevLattice& L, BcState* bc, 
 template <class M, int NT>
 __device__ __forceinline__ M inlet_density(const DevLattice& L, BcState* bc, int slot, const double* __restrict__ partials,
                                            double* sh, bool first) {
-    if (bc->inlet_mode) return M(bc->drho_in_fixed);
-    return density_of_parts<M, NT>(L, bc, slot, partials, sh, first);
+    // in pressure mode the first block still records the density that the flux would need
+    const int fixed = bc->inlet_mode;
+    if (fixed && !first) return M(bc->drho_in_fixed);
+    const M drho = density_of_parts<M, NT>(L, bc, slot, partials, sh, first);
+    return fixed ? M(bc->drho_in_fixed) : drho;
 }
 
 // drho_in[slot] from its parts, for readers between steps (the 16-bit reference,
