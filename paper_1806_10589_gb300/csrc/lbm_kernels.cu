@@ -390,14 +390,64 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 // fence, a ticket and a second round of loads at the end of every step: 8.5 us per
 // step of a 10k-node FP32 lattice against 6.7, 8.8 against 7.5 at 173k nodes, 11.0
 // against 9.1 at 365k.)
-template <class S, int NT>
-__device__ __forceinline__ void store_inlet_part(double part, int64_t tile, int64_t tiles, const DevLattice& L,
-                                                 BcState* bc, int slot, double* __restrict__ partials) {
-    constexpr int W = NT / 32;
-    const double v = warp_sum(part);
-    if ((threadIdx.x & 31) == 0) partials[(slot ^ 1) * L.part_stride + tile * W + (threadIdx.x >> 5)] = v;
+//   Every block with inlet nodes adds all parts, which costs the square of the inlet
+// area: with one part per warp throughout, an open FP32 lattice of 1024x1024x3 took
+// 602 us per step, of 512x512x16 139.  Above 32 LBM_WARP_PARTS nodes on the planes a
+// tile therefore leaves one part for all its warps (112x112x24, AA pattern: 10.5 ->
+// 9.7 us; 256x256x16: 25.5 -> 24.3; below, the block's sum would only lengthen the
+// step's tail), and above LBM_PARTS_DIRECT of those a kernel behind the step adds them
+// to kFolded ones first, the count stored as its negative (512x512x16, 2,048 parts:
+// 117.4 us without that kernel and 118.7 with it, 600x600x16, 2,813 parts: 167.5 and
+// 165.2; 1024x1024x3 125, 2047x2047x4 8,590 -> 613).
+#ifndef LBM_WARP_PARTS
+#define LBM_WARP_PARTS 512
+#endif
+#ifndef LBM_PARTS_DIRECT
+#define LBM_PARTS_DIRECT 2048
+#endif
+constexpr int kPartsDirect = LBM_PARTS_DIRECT;
+constexpr int kFolded = kFoldedParts;
+// Parts of a tile of NT threads, and of a step of blocks of `nodes` nodes.
+template <int NT>
+__host__ __device__ __forceinline__ int tile_parts(const DevLattice& L) {
+    return L.a_01 <= 32 * LBM_WARP_PARTS ? NT / 32 : 1;
+}
+template <int NT>
+__host__ __device__ __forceinline__ int step_parts(const DevLattice& L, int nodes) {
+    return (int)((L.a_01 + nodes - 1) / nodes) * tile_parts<NT>(L);
+}
+template <class P>
+__device__ __forceinline__ P* folded(const DevLattice& L, P* partials, int slot) {
+    return partials + 2 * L.part_stride + slot * kFolded;
+}
+__global__ void __launch_bounds__(kReduceBlock)
+k_inlet_fold(DevLattice L, int n, int slot, double* __restrict__ partials) {
+    __shared__ double sh[32];
+    const double* p = partials + slot * L.part_stride;
+    double s = 0.0;
+    for (int j = blockIdx.x * kReduceBlock + threadIdx.x; j < n; j += kFolded * kReduceBlock) s += p[j];
+    s = block_sum<kReduceBlock>(s, sh);
+    if (threadIdx.x == 0) folded(L, partials, slot)[blockIdx.x] = s;
+}
+// Behind a step that reads buffer `slot`, in blocks of NT threads and `nodes` nodes.
+template <int NT>
+inline cudaError_t fold_parts(const DevLattice& L, int slot, double* partials, int nodes, cudaStream_t st) {
+    const int n = step_parts<NT>(L, nodes);
+    if (n > kPartsDirect) k_inlet_fold<<<kFolded, kReduceBlock, 0, st>>>(L, n, slot ^ 1, partials);
+    return cudaGetLastError();
+}
+template <class S, int NT, int NODES>
+__device__ __forceinline__ void store_inlet_part(double part, int64_t tile, const DevLattice& L, BcState* bc, int slot,
+                                                 double* __restrict__ partials, double* sh) {
+    const int w = tile_parts<NT>(L);
+    double v;
+    if (NT > 32 && w == 1) v = block_sum<NT>(part, sh);
+    else v = warp_sum(part);
+    if ((threadIdx.x & 31) == 0 && (int)(threadIdx.x >> 5) < w)
+        partials[(slot ^ 1) * L.part_stride + tile * w + (threadIdx.x >> 5)] = v;
     if (tile == 0 && threadIdx.x == 0) {
-        bc->parts[slot ^ 1] = (int)(tiles * W);
+        const int n = step_parts<NT>(L, NODES);
+        bc->parts[slot ^ 1] = n > kPartsDirect ? -n : n;
         if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
     }
 }
@@ -410,9 +460,13 @@ template <class M, int NT>
 __device__ __forceinline__ M density_of_parts(const DevLattice& L, BcState* bc, int slot,
                                               const double* __restrict__ partials, double* sh, bool first) {
     constexpr int W = NT / 32;
-    const int n = bc->parts[slot];
+    int n = bc->parts[slot];
     if (n == 0) return M(bc->drho_in[slot]);
     const double* p = partials + slot * L.part_stride;
+    if (n < 0) {  // folded behind the step that left them
+        p = folded(L, partials, slot);
+        n = kFolded;
+    }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int vw = wid; vw < 8; vw += W) {
         double s = 0.0;
@@ -513,7 +567,7 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
         }
     }
     if ((int64_t)blockIdx.x * NT < L.a_01)
-        store_inlet_part<S, NT>(part, blockIdx.x, (L.a_01 + NT - 1) / NT, L, bc, slot, partials);
+        store_inlet_part<S, NT, NT>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // ------------------------------------------------------ AA-pattern step ---
@@ -727,7 +781,7 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
         }
     }
     if ((int64_t)blockIdx.x * NT < L.a_01)
-        store_inlet_part<S, NT>(part, blockIdx.x, (L.a_01 + NT - 1) / NT, L, bc, slot, partials);
+        store_inlet_part<S, NT, NT>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // ------------------------------------------- two nodes per thread (16-bit) ---
@@ -858,7 +912,7 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
     if ((int64_t)blockIdx.x * kBlock < L.a_01)
-        store_inlet_part<S, kPair>(part, blockIdx.x, (L.a_01 + kBlock - 1) / kBlock, L, bc, slot, partials);
+        store_inlet_part<S, kPair, kBlock>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // Gather-scatter launch: thread t of a warp owns the nodes 64 w + t and
@@ -950,7 +1004,7 @@ k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float
         });
     }
     if ((int64_t)blockIdx.x * kBlock < L.a_01)
-        store_inlet_part<S, kPair>(part, blockIdx.x, (L.a_01 + kBlock - 1) / kBlock, L, bc, slot, partials);
+        store_inlet_part<S, kPair, kBlock>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // Node-local launch: neighbouring nodes on a thread, one 4-byte load and store per row.
@@ -1003,7 +1057,7 @@ k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<floa
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
     if ((int64_t)blockIdx.x * kBlock < L.a_01)
-        store_inlet_part<S, kPair>(part, blockIdx.x, (L.a_01 + kBlock - 1) / kBlock, L, bc, slot, partials);
+        store_inlet_part<S, kPair, kBlock>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // Pull layout <-> layout S: swap F[q][x] and F[opp q][x] at every node.
@@ -1237,7 +1291,7 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<type
             if (i64 < L.a_01) part = next_inlet_part<S>(d, L, p_cur, i, r_own, seed);
         }
         if (t < nt01)  // tile holds plane z = 0 / z = 1 nodes (block-uniform)
-            store_inlet_part<S, NT>(part, t, nt01, L, bc, slot, partials);
+            store_inlet_part<S, NT, NT>(part, t, L, bc, slot, partials, sh);
         hi_cur = hi_next;
         nb_cur = nb_next;
         p_cur = p_next;
@@ -1506,6 +1560,7 @@ __global__ void k_node_words(const uint32_t* __restrict__ vox, uint32_t vox0, in
 // 112 k nodes) measured slower: 1.01 ms in blocks of 256, 1.02 in 128, 1.17 in 64.
 constexpr int64_t kSmallNodes = 152 * 256;
 constexpr int kSmallBlock = 32;
+static_assert(kSmallNodes / kSmallBlock <= LBM_PARTS_DIRECT, "a step in small blocks leaves no parts to fold");
 
 inline unsigned blocks_for(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
@@ -1559,16 +1614,17 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
         // GB300_LBM_STEP_ADDR64 forces the id-grid form with 64-bit addresses (tests)
         if (L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64"))
         {
-            if constexpr (S::kRef)
+            if constexpr (S::kRef) {
                 k_step_pair<S><<<blocks_for(L.n, kBlock), kPair, 0, st>>>(P, slot, L, make_rates<float>(r.sp, r.sm), bc, partials);
-            else if (sizeof(M) == 8 && L.n < kSmallNodes)
+                return fold_parts<kPair>(L, slot, partials, kBlock, st);
+            } else if (sizeof(M) == 8 && L.n < kSmallNodes)
                 k_step<S, true, kSmallBlock><<<blocks_for(L.n, kSmallBlock), kSmallBlock, 0, st>>>(
                     P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
             else
                 k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
         } else
             k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-        return cudaGetLastError();
+        return fold_parts<kBlock>(L, slot, partials, kBlock, st);
     });
 }
 
@@ -1584,7 +1640,7 @@ cudaError_t launch_async_t(const void* fin, void* fout, int slot, const DevLatti
     }
     const size_t smem = async_smem_bytes<NT>(AsyncSlot<S>::kBytes);
     k_step_async<S, NT><<<grid, NT, smem, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-    return cudaGetLastError();
+    return fold_parts<NT>(L, slot, partials, NT, st);
 }
 
 template <class S, int NT>
@@ -1702,7 +1758,7 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
                         k_aa_odd_pair<S><<<nb, kPair, 0, st>>>((typename S::T*)f, slot, L, rates, bc, partials);
                     else
                         k_aa_even_pair<S><<<nb, kPair, 0, st>>>(F, slot, L, rates, bc, partials);
-                    return cudaGetLastError();
+                    return fold_parts<kPair>(L, slot, partials, kBlock, st);
                 }
             } else if (win && sizeof(M) == 8 && L.n < kSmallNodes) {
                 const unsigned nbs = blocks_for(L.n, kSmallBlock);
@@ -1713,11 +1769,11 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
                 return cudaGetLastError();
             } else if (odd && win) {
                 k_step_aa<S, true, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-                return cudaGetLastError();
+                return fold_parts<kBlock>(L, slot, partials, kBlock, st);
             }
             if (odd) k_step_aa<S, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
             else k_step_aa<S, false><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-            return cudaGetLastError();
+            return fold_parts<kBlock>(L, slot, partials, kBlock, st);
         }
     });
 }
