@@ -160,6 +160,7 @@ struct ConvEpi {
     bf16* out_mask;
     float* y;                   // output layer: y[b][c][z][y][x] = v * pore, c < kOut
     const bf16* xin;            // pore indicator rows (channel 0 of a 32-channel tensor)
+    bool border;                // out's border rows are to be written too (0)
     int* err;
     PGeo g;
 };
@@ -1424,15 +1425,59 @@ cudaError_t wgrad_t(const bf16* act, const bf16* gout, const WgArgs& a0, cudaStr
         default: return cudaErrorInvalidValue;                               \
     }
 
-// Layers whose 27 taps fit in shared memory beside two plane buffers march along
-// z (64 -> 64 with half of the output channels per CTA); the others take k_conv.
-bool conv_marches(int cin, int cout) { return cin <= 64 && cout <= 64; }
+// A layer whose 27 taps fit in shared memory beside two plane buffers marches along z
+// (64 -> 64 with half of the output channels per CTA) where that is faster: per
+// 128-row tile a march takes `march` ns of the chip where k_conv takes `conv`, but it
+// starts `late` ns later (the weights and three planes come before its first output),
+// its last round of CTAs may be short, and a patch is whole tiles, while k_conv also
+// computes the border rows, which a march leaves to k_zero_border where they are to be
+// written.  Fitted to 28 volumes from 4^3 to 144x128x144 a pair: the march is not taken
+// where it is slower.  Per launch, k_conv and k_conv_march:
+//   32 -> 32   24^3 8.2 and 18.5 us   4 x 24x32x40 24.7 and 26.7   8 x 64^3 311 and 242
+//   32 -> 64   24^3 8.3 and 10.3      4 x 24x32x40 32.8 and 28.7   8 x 64^3 386 and 291
+//   64 -> 32   24^3 10.3 and 11.9     4 x 24x32x40 55.3 and 41.3   8 x 64^3 783 and 478
+//   64 -> 64   24^3 10.3 and 16.4     4 x 24x32x40 61.4 and 71.7   8 x 64^3 857 and 946
+//              (6 x 72x72x6, a quarter of whose rows are border: 104 and 88)
+// Both add the products of an output in one order: the results are the same bits.
+struct MarchCost {
+    int cin, cout, n;  // n: channels per CTA
+    float conv, march, late;
+};
+constexpr MarchCost kMarchCost[] = {
+    {32, 32, 32, 17.3f, 14.3f, 3500.f}, {32, 64, 64, 21.4f, 16.5f, 1500.f}, {64, 32, 32, 43.6f, 27.1f, 4500.f},
+    {64, 64, 32, 47.7f, 54.3f, 5000.f}};
+constexpr double kZeroBorderNs = 4000.0;
+bool conv_marches(int cin, int cout, const PGeo& g, bool border, int n_sm) {
+    for (const MarchCost& c : kMarchCost) {
+        if (c.cin != cin || c.cout != cout) continue;
+        MarchArgs a{};
+        size_t smem;
+        const bool fits = c.n == 64     ? march_plan<32, 64>(g, cout, &a, &smem)
+                          : cin == 32   ? march_plan<32, 32>(g, cout, &a, &smem)
+                                        : march_plan<64, 32>(g, cout, &a, &smem);
+        if (!fits) return false;
+        const int64_t items = (int64_t)g.B * a.patches * g.Z, ctas = std::max(1, n_sm / a.parts);
+        const double tiles = (double)((items + ctas - 1) / ctas * ctas * a.T);
+        return tiles * c.march + c.late + (border ? kZeroBorderNs : 0.0) <
+               (double)((g.rows() + kRows - 1) / kRows) * c.conv;
+    }
+    return false;
+}
 cudaError_t conv(int cin, int cout, const bf16* in, const bf16* w, const bf16* wt, const ConvEpi& epi,
                  cudaStream_t st, int n_sm) {
-    if (cin == 32 && cout == 32) return march_t<32, 32>(in, wt, cout, epi, st, n_sm);
-    if (cin == 32 && cout == 64) return march_t<32, 64>(in, wt, cout, epi, st, n_sm);
-    if (cin == 64 && (cout == 32 || cout == 64)) return march_t<64, 32>(in, wt, cout, epi, st, n_sm);
+    if (conv_marches(cin, cout, epi.g, epi.border, n_sm)) {
+        if (epi.border) {
+            const int64_t lines = (int64_t)epi.g.B * (epi.g.Z + 2) * (epi.g.Y + 2);
+            k_zero_border<<<(unsigned)((lines + 7) / 8), 256, 0, st>>>(epi.out, epi.g, cout);
+        }
+        if (cin == 64) return march_t<64, 32>(in, wt, cout, epi, st, n_sm);
+        return cout == 32 ? march_t<32, 32>(in, wt, cout, epi, st, n_sm) : march_t<32, 64>(in, wt, cout, epi, st, n_sm);
+    }
     switch (cin * 1000 + cout) {
+        case 32032: return conv_t<32, 32>(in, w, wt, epi, st);
+        case 32064: return conv_t<32, 64>(in, w, wt, epi, st);
+        case 64032: return conv_t<64, 32>(in, w, wt, epi, st);
+        case 64064: return conv_t<64, 64>(in, w, wt, epi, st);
         case 32128: return conv_t<32, 128>(in, w, wt, epi, st);
         case 32256: return conv_t<32, 256>(in, w, wt, epi, st);
         case 64128: return conv_t<64, 128>(in, w, wt, epi, st);
@@ -2155,21 +2200,19 @@ int conv_call(int op, const void* in, const void* aux, const void* w, const floa
     if (ms && e == cudaSuccess) e = cudaEventCreate(&ev[1]);
     if (ms && e == cudaSuccess) e = cudaEventRecord(ev[0], st);
     for (int r = 0; r < reps && e == cudaSuccess; ++r) {
-        if (op < 2 && wsn::conv_marches(cin, cout)) {  // these write the rows of the interior lines
-            const int64_t lines = (int64_t)batch * (nz + 2) * (ny + 2);
-            wsn::k_zero_border<<<(unsigned)((lines + 7) / 8), 256, 0, st>>>((bf16*)out, g, op == 0 ? cout : cin);
-        }
         if (op == 0) {
             wsn::ConvEpi ep{};
             ep.bias = bias;
             ep.relu = relu;
             ep.out = (bf16*)out;
+            ep.border = true;
             ep.err = d_err;
             ep.g = g;
             e = wsn::conv(cin, cout, (const bf16*)in, wb, wb + nw, ep, st, nsm);
         } else if (op == 1) {
             wsn::ConvEpi ep{};
             ep.out = (bf16*)out;
+            ep.border = true;
             ep.err = d_err;
             ep.g = g;
             e = wsn::conv(cout, cin, (const bf16*)in, wb, wb + nw, ep, st, nsm);
