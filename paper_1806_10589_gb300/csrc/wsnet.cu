@@ -685,8 +685,8 @@ k_wgrad(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensor
 // interior lines, rounded up to 16 rows of zeros.
 //   The tensor core truncates as it adds, so the error of a sum grows with the
 // products added in one accumulator.  An accumulator is therefore drained (added
-// to the CTA's partial sums in FP32) before it has taken more than a split of
-// k_wgrad would, or 64 products of 16 rows: on 64 -> 64 channels, 4 x 44x52x36
+// to the CTA's partial sums in FP32) before it has taken more products of 16 rows
+// than a split of k_wgrad would: on 64 -> 64 channels, 4 x 44x52x36
 // voxels, the error against 64 bits is 1.5e-6 of the gradient, 1.6e-6 with k_wgrad
 // (6.2e-6 with one drain per CTA).
 template <int CIN, int COUT>
@@ -1327,16 +1327,25 @@ cudaError_t march_t(const bf16* in, const bf16* wt, int cout, const ConvEpi& epi
 }
 
 // Patch of a marching weight gradient: the largest T for which the resident
-// planes and one more of each kind fit (more tiles: fewer halo rows).  The zero
+// planes and one more of each kind fit (more tiles: fewer halo rows), cut to the
+// smallest with as many patches (even patches: a CTA's share is counted in patches).
+// Volumes whose accumulators would take under kMarchProducts products stay with
+// k_wgrad: a march would add more products in one accumulator than its row splits do
+// (at a limit of 64 throughout, 32 -> 64 channels on 8 x 24^3 voxels were off by
+// 5.8e-7 of the gradient instead of 3.7e-7) or drain it at every step (28.7 us
+// instead of 22.6 on 24^3).  The zero
 // rows after a patch (up to 16) have to end before the next plane's interior:
 // padded lines of 8 rows or more.
+constexpr int kMarchProducts = 64;
 template <int CIN, int COUT>
 bool wm_plan(const PGeo& g, int n_sm, WmArgs* out, size_t* smem) {
     using K = WmCfg<CIN, COUT>;
-    if (g.xp() < 8) return false;
+    const int64_t limit = g.rows() / wgrad_splits(CIN, COUT, g.rows(), n_sm) / 16;
+    if (g.xp() < 8 || limit < kMarchProducts) return false;
     const int64_t lines = (int64_t)g.Y * g.xp();
+    const auto patches_of = [&](int T) { return (lines + T * kRows - 1) / (T * kRows); };
     for (int T = 4; T >= 1; --T) {
-        if (T > 1 && (T - 1) * kRows >= lines) continue;
+        if (T > 1 && patches_of(T - 1) == patches_of(T)) continue;
         for (int nseg = 1; nseg <= 3; nseg += 2) {
             const int rows = nseg == 1 ? T * kRows + 2 * g.xp() : T * kRows;
             WmArgs a{};
@@ -1352,7 +1361,7 @@ bool wm_plan(const PGeo& g, int n_sm, WmArgs* out, size_t* smem) {
             a.gbytes = (int)(((size_t)a.gnbox * a.gbox * K::GROW + 1023) / 1024 * 1024);
             a.na = K::ND + 1;
             a.ng = 2;
-            a.patches = (int)((lines + T * kRows - 1) / (T * kRows));
+            a.patches = (int)patches_of(T);
             // the unused block of the activation operand reads up to one segment past
             // its plane: into the buffers after it, and at the end into this slack
             const size_t used = (size_t)a.na * a.abytes + (size_t)a.ng * a.gbytes + 256;
@@ -1360,7 +1369,7 @@ bool wm_plan(const PGeo& g, int n_sm, WmArgs* out, size_t* smem) {
             const size_t slack = over > (size_t)a.ng * a.gbytes ? over - (size_t)a.ng * a.gbytes : 0;
             const size_t total = 1024 + used + slack;
             if (total > K::SMEM_MAX) continue;
-            a.limit = (int)std::max<int64_t>(64, g.rows() / wgrad_splits(CIN, COUT, g.rows(), n_sm) / 16);
+            a.limit = (int)limit;
             *out = a;
             *smem = total;
             return true;
