@@ -1068,11 +1068,24 @@ __global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, 
 }
 
 // gw[w] += sum over k of part[k][w] in a fixed order (the deterministic finish of
-// the weight- and bias-gradient kernels): 8 threads per w each add every eighth
-// split, then the eight sums are added in order.  One thread per w left the card
-// waiting on its chain of loads (19 us a layer on average, 16 MB read).
+// the weight- and bias-gradient kernels).  One thread per w reads coalesced rows and
+// is enough where there are many weights or few splits.  Of few weights and many
+// splits (the narrow layers) it left the card waiting on its chain of loads: there 8
+// threads per w each add every eighth split, then the eight sums are added in order.
+// Gradient of the 4-level network, us, one thread / eight / by the rule below: 1 x
+// 16^3 1335 (previous kernels), 1421, 1340; 8 x 32^3 - , 2986, 2860; 8 x 64^3 -, 8807,
+// 8661 (a rule at 16 splits and 300,000 weights: 1332, 2866, 8676).
 __global__ void __launch_bounds__(256)
-k_split_sum(const float* __restrict__ part, int64_t splits, int64_t nw, float* __restrict__ gw) {
+k_split_sum1(const float* __restrict__ part, int64_t splits, int64_t nw, float* __restrict__ gw) {
+    const int64_t w = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (w >= nw) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int64_t k = 0; k < splits; ++k) s += part[k * nw + w];
+    gw[w] += s;
+}
+__global__ void __launch_bounds__(256)
+k_split_sum8(const float* __restrict__ part, int64_t splits, int64_t nw, float* __restrict__ gw) {
     __shared__ float sh[8][32];
     const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
     const int64_t w = (int64_t)blockIdx.x * 32 + lane;
@@ -1089,7 +1102,8 @@ k_split_sum(const float* __restrict__ part, int64_t splits, int64_t nw, float* _
     }
 }
 inline cudaError_t split_sum(const float* part, int64_t splits, int64_t nw, float* gw, cudaStream_t st) {
-    k_split_sum<<<(unsigned)((nw + 31) / 32), 256, 0, st>>>(part, splits, nw, gw);
+    if (splits >= 64 && nw <= 100000) k_split_sum8<<<(unsigned)((nw + 31) / 32), 256, 0, st>>>(part, splits, nw, gw);
+    else k_split_sum1<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(part, splits, nw, gw);
     return cudaGetLastError();
 }
 
