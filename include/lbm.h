@@ -384,7 +384,7 @@ int lbm_wsnet_train(lbm_wsnet* net, const uint8_t* masks, const float* targets, 
 /* Predicted fields (host, 4*nz*ny*nx floats) of one geometry; 0 at solids. */
 int lbm_wsnet_predict(lbm_wsnet* net, const uint8_t* mask, int nx, int ny, int nz, float* y);
 /* Free the activation buffers kept between calls (sized for the last batch and volume),
- * and the scratch of up to 16 MB per device that lbm_conv3d_bf16 keeps between calls. */
+ * and the scratch that lbm_conv3d_bf16 keeps (lbm_conv3d_release). */
 int lbm_wsnet_release_buffers(lbm_wsnet* net);
 int lbm_wsnet_destroy(lbm_wsnet* net);
 const char* lbm_wsnet_last_error(const lbm_wsnet* net);
@@ -406,10 +406,13 @@ const char* lbm_wsnet_last_error(const lbm_wsnet* net);
  *          channels, zero on border rows; out: FP32 [cout][27][cin], added to
  *          with FP32 atomics, one per row split: the order of those additions,
  *          and so the last bits, may vary between calls)
- * Returns LBM_EINVAL for bad arguments, LBM_ECUDA for a CUDA error and
- * LBM_ETIMEOUT if a pipeline wait ran out. */
+ * Returns LBM_EINVAL for bad arguments, LBM_ECUDA for a CUDA error (a stream that
+ * records a graph among them) and LBM_ETIMEOUT if a pipeline wait ran out. */
 int lbm_conv3d_bf16(int op, const void* in, const void* aux, const void* w, const float* bias, int relu, void* out,
                     int batch, int nx, int ny, int nz, int cin, int cout, void* cuda_stream);
+/* Free the scratch that the convolution calls keep on the current device between
+ * calls: at most 16 MB of device memory, shared by all threads and streams. */
+int lbm_conv3d_release(void);
 /* The same convolution launched `reps` times back to back on `cuda_stream`,
  * bracketed by CUDA events on that stream; *ms_per_call = the mean time of
  * one launch.  For op 2 the weight gradient is added `reps` times. */

@@ -1198,46 +1198,83 @@ __global__ void k_pack_layer(const bf16* __restrict__ w, int cin, int cout, int 
 }
 
 // ------------------------------------------------------- host helpers ---
-// Scratch of a single convolution call, stream-ordered from one pool per device:
-// the pool keeps at most kScratchKept bytes between calls (a cudaMalloc and a
-// cudaFree per call took 170 us, about as long as a layer), shared by all threads
-// and streams; lbm_wsnet_release_buffers gives them back.
-constexpr uint64_t kScratchKept = 16u << 20;
-constexpr int kMaxDevices = 64;
-cudaMemPool_t g_scratch[kMaxDevices] = {};
+// Scratch of a single convolution call: a buffer that is the call's own until it
+// returns (it has synchronised its stream by then), from a few that are kept, at most
+// kScratchKept bytes per device (a layer of 256 x 256 channels takes 7 MB), shared by
+// all threads and streams; lbm_conv3d_release gives them back.  A cudaMalloc and a
+// cudaFree per call took 170 us, about as long as a layer.  A stream-ordered pool saved
+// that only until the next synchronisation: it grows by 32 MB, more than it was to
+// keep, and unmapped them there (a weight gradient of 6^3 voxels after a
+// synchronisation: 170 us with cudaMalloc, 220 from such a pool, 37 here).
+constexpr size_t kScratchKept = 16u << 20;
+struct Scratch {
+    void* p;
+    size_t bytes;
+    int dev;
+    bool busy;
+};
+constexpr int kScratchSlots = 64;
+Scratch g_scratch[kScratchSlots] = {};  // p == nullptr: free slot
 std::mutex g_scratch_mutex;
 
-cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+// A buffer of `bytes` or more on the current device; a call that finds no slot gets one
+// that scratch_give frees.
+cudaError_t scratch_take(void** p, size_t bytes) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    cudaMemPool_t pool;
     {
         std::lock_guard<std::mutex> lock(g_scratch_mutex);
-        if (!g_scratch[dev]) {
-            cudaMemPoolProps props{};
-            props.allocType = cudaMemAllocationTypePinned;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = dev;
-            cudaMemPool_t made = nullptr;
-            if ((e = cudaMemPoolCreate(&made, &props)) != cudaSuccess) return e;
-            uint64_t kept = kScratchKept;
-            if ((e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &kept)) != cudaSuccess) {
-                cudaMemPoolDestroy(made);
-                return e;
-            }
-            g_scratch[dev] = made;
+        Scratch* best = nullptr;
+        for (Scratch& s : g_scratch)
+            if (s.p && !s.busy && s.dev == dev && s.bytes >= bytes && (!best || s.bytes < best->bytes)) best = &s;
+        if (best) {
+            best->busy = true;
+            *p = best->p;
+            return cudaSuccess;
         }
-        pool = g_scratch[dev];
     }
-    return cudaMallocFromPoolAsync(p, bytes, pool, st);
-}
-void scratch_trim() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kMaxDevices) return;
+    if ((e = cudaMalloc(p, bytes)) != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(g_scratch_mutex);
-    if (g_scratch[dev]) cudaMemPoolTrimTo(g_scratch[dev], 0);
+    for (Scratch& s : g_scratch)
+        if (!s.p) {
+            s = Scratch{*p, bytes, dev, true};
+            break;
+        }
+    return cudaSuccess;
+}
+// Frees buffers of the device that no call holds until `room` bytes may be added.
+void scratch_make_room(int dev, size_t room) {
+    size_t kept = 0;
+    for (const Scratch& s : g_scratch)
+        if (s.p && !s.busy && s.dev == dev) kept += s.bytes;
+    for (Scratch& s : g_scratch)
+        if (s.p && !s.busy && s.dev == dev && kept + room > kScratchKept) {
+            kept -= s.bytes;
+            cudaFree(s.p);
+            s = Scratch{};
+        }
+}
+// `idle`: nothing on the device uses the buffer any more.
+cudaError_t scratch_give(void* p, bool idle) {
+    std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    for (Scratch& s : g_scratch)
+        if (s.p == p) {
+            if (idle && s.bytes <= kScratchKept) {
+                scratch_make_room(s.dev, s.bytes);
+                s.busy = false;
+                return cudaSuccess;
+            }
+            s = Scratch{};
+            break;
+        }
+    return cudaFree(p);  // waits for work in flight
+}
+void scratch_release() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return;
+    std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    scratch_make_room(dev, kScratchKept + 1);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
@@ -2158,7 +2195,7 @@ int lbm_wsnet_release_buffers(lbm_wsnet* n) {
     if (rc) return rc;
     cudaStreamSynchronize(n->stream);
     free_buffers(n);
-    wsn::scratch_trim();
+    wsn::scratch_release();
     cudaFree(n->part);
     n->part = nullptr;
     n->part_cap = 0;
@@ -2202,8 +2239,14 @@ int conv_call(int op, const void* in, const void* aux, const void* w, const floa
     // forward [cout][27][cin] and [27][cout][cin]; data gradient (flipped taps)
     // [cin][27][cout] and [27][cin][cout]
     const size_t nw = (size_t)cout * 27 * cin;
+    // the call ends with a synchronisation, which a stream that records a graph refuses
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return LBM_ECUDA;
+    }
     void* scratch = nullptr;
-    cudaError_t e = wsn::scratch_alloc(&scratch, 256 + (op < 2 ? 2 * nw * sizeof(bf16) : 0), st);
+    cudaError_t e = wsn::scratch_take(&scratch, 256 + (op < 2 ? 2 * nw * sizeof(bf16) : 0));
     if (e != cudaSuccess) {
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
@@ -2260,7 +2303,8 @@ int conv_call(int op, const void* in, const void* aux, const void* w, const floa
     }
     for (auto& x : ev)
         if (x) cudaEventDestroy(x);
-    if (cudaFreeAsync(scratch, st) != cudaSuccess && e == cudaSuccess) e = cudaErrorUnknown;
+    const cudaError_t e_give = wsn::scratch_give(scratch, e == cudaSuccess);
+    if (e == cudaSuccess) e = e_give;
     if (e != cudaSuccess) return LBM_ECUDA;
     return h ? LBM_ETIMEOUT : LBM_OK;
 }
@@ -2273,6 +2317,11 @@ int lbm_conv3d_bf16(int op, const void* in, const void* aux, const void* w, cons
                     int batch, int nx, int ny, int nz, int cin, int cout, void* stream) {
     return conv_call(op, in, aux, w, bias, relu, out, batch, nx, ny, nz, cin, cout, 1, nullptr,
                      (cudaStream_t)stream);
+}
+
+int lbm_conv3d_release(void) {
+    wsn::scratch_release();
+    return LBM_OK;
 }
 
 int lbm_conv3d_bf16_time(int op, const void* in, const void* aux, const void* w, const float* bias, int relu,

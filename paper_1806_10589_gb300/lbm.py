@@ -100,6 +100,7 @@ SIGNATURES = {
     "lbm_wsnet_last_error": (C.c_char_p, [_P]),
     "lbm_conv3d_bf16": (C.c_int, [C.c_int, _P, _P, _P, _FP, C.c_int, _P, C.c_int, C.c_int, C.c_int, C.c_int,
                                   C.c_int, C.c_int, _P]),
+    "lbm_conv3d_release": (C.c_int, []),
     "lbm_conv3d_bf16_time": (C.c_int, [C.c_int, _P, _P, _P, _FP, C.c_int, _P, C.c_int, C.c_int, C.c_int, C.c_int,
                                        C.c_int, C.c_int, C.c_int, _FP, _P]),
 }
@@ -493,6 +494,11 @@ def conv3d_bf16(op, inp, aux, w, bias, relu, out, batch, nx, ny, nz, cin, cout, 
     if st != LBM_OK:
         raise LBMError(st, "lbm_conv3d_bf16(op %d, cin %d, cout %d)" % (op, cin, cout))
     return ms
+
+
+def conv3d_release():
+    """lbm_conv3d_release: free the scratch kept between convolution calls on the current device."""
+    load_library().lbm_conv3d_release()
 
 
 class ColorLattice:
