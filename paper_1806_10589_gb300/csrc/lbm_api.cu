@@ -14,6 +14,7 @@
 #include <new>
 #include <cstdio>
 #include <algorithm>
+#include <cstdlib>
 #include <cstring>
 #include <string>
 #include <vector>
@@ -356,9 +357,9 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
         c->L.sz_magic = (uint64_t)(two64 / szq + (two64 % szq != 0 ? 1 : 0));
     }
 
-    // row windows, where a window index fits the node's word
+    // row windows, where a window index fits the node's word (GB300_LBM_NO_WINDOWS: none, for tests)
     const int64_t nwin = (int64_t)lbm::windows_per_row(nx) * py * pz;
-    const bool windows = nwin < (int64_t)1 << 27;
+    const bool windows = nwin < (int64_t)1 << 27 && !std::getenv("GB300_LBM_NO_WINDOWS");
     if (windows) {
         c->L.wy = lbm::windows_per_row(nx);
         c->L.wz = c->L.wy * (int)py;

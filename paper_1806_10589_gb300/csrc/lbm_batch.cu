@@ -232,9 +232,6 @@ __device__ __forceinline__ void batch_finish(double part, int slot, int64_t tile
 
 // One 256-node tile of one step: the single-lattice step with the member's own
 // boundary scalars, and the member's next inlet density.
-// FORM: kGrid64 the id grid with 64-bit addresses, kGrid32 the id grid and kWindows
-// the row windows, both with fin plus one 32-bit element offset per source.
-enum { kGrid64 = 0, kGrid32 = 1, kWindows = 2 };
 template <class S, bool COH, int FORM = kGrid64>
 __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typename S::T* fout, int64_t ns, int slot,
                                                 int64_t tile, const Links& K, const int* __restrict__ tile_member,
@@ -1049,10 +1046,10 @@ int bstep_once(lbm_batch* b, cudaStream_t st) {
         // GB300_LBM_BATCH_ADDR64 forces the id-grid form (tests)
         const bool off32 = 19 * (uint64_t)b->ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_BATCH_ADDR64");
         const bool capped = cfg_capped(b->config);
-        if (off32 && b->ntiles < lbm::kWindowTiles) {
+        if (off32 && (b->ntiles < lbm::kWindowTiles || !b->d_win)) {
             capped ? launch(lbm::k_batch_step<S, 5, lbm::kGrid32>, lbm::kTile)
                    : launch(lbm::k_batch_step<S, 4, lbm::kGrid32>, lbm::kTile);
-        } else if (off32 && b->d_win) {
+        } else if (off32) {
             if constexpr (S::kRef)
                 capped ? launch(lbm::k_batch_pair<S, 6>, lbm::kTile / 2) : launch(lbm::k_batch_pair<S, 5>, lbm::kTile / 2);
             else
@@ -1297,7 +1294,7 @@ int lbm_batch_create(int n_members, const uint8_t* const* masks, const int* dims
     A(&b->f[1], fbytes);
     A(&b->d_vox, vox.size() * 4);
     A(&b->d_grid, grid.size() * 4);
-    const bool windows = wbase < (int64_t)1 << 27;
+    const bool windows = wbase < (int64_t)1 << 27 && !std::getenv("GB300_LBM_NO_WINDOWS");
     if (windows) {
         A(&b->d_win, (size_t)wbase * sizeof(uint2));
         A(&b->d_nodew, (size_t)base * sizeof(uint32_t));

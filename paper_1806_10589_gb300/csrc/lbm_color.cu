@@ -227,19 +227,19 @@ __global__ void k_color_faces(DevLattice L, uint8_t* __restrict__ faces) {
                          (y == L.ny ? kFaceY1 : 0u) | (z == 1 ? kFaceZ0 : 0u) | (z == L.nz ? kFaceZ1 : 0u));
 }
 
-// WIN (buffers of 19 ns < 2^32 elements, and a row-window table): the neighbours
+// FORM: see lbm_device.cuh.  With the row windows the neighbours
 // come from the row windows and the node's face bits -- 9 loads where the id grid
 // takes 18, and 6 again for the push, whose destinations are staged in shared memory
 // here -- and a gathered or pushed value is addressed as row 0 plus one 32-bit
 // element offset.  Bound by the latency of the gathers behind the index loads (68 %
 // of DRAM bandwidth on the id grid at 64 registers); without the id loads the kernel
 // fits 48 registers, so 5 blocks per SM instead of 4: 65.5 -> 62.6 us on a
-// 128x128x256 pack (1.6 M pores), bitwise equal states.  Otherwise (19 ns >= 2^32 or
-// 2^27 windows and more) the id grid and 64-bit row pointers.
-template <class T, bool WIN = false>
+// 128x128x256 pack (1.6 M pores), bitwise equal states.
+template <class T, int FORM>
 __global__ void __launch_bounds__(kCB, color_min_blocks<T>())
 k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, const uint8_t* __restrict__ faces,
              const ColorParams* __restrict__ prm, Rates<T> rates, T alpha, T beta, T phi_s) {
+    constexpr bool WIN = FORM == kWindows, OFF32 = FORM != kGrid64;
     __shared__ uint32_t push[WIN ? 7 : 1][WIN ? kCB : 1];  // [Q]: push destination (element of the D3Q7 rows)
     const int64_t i64 = (int64_t)blockIdx.x * kCB + threadIdx.x;
     if constexpr (LBM_COLOR_PREFETCH > 0) {
@@ -281,7 +281,11 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
         for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
             constexpr int Q = decltype(qc)::value + 1;
             const int id = ld_hint(L.grid + (uint32_t)(p + (uint32_t)grid_off<Q>(L.sy, L.sz)), pol);
-            d[Q] = id >= 0 ? R.fin[Q][id] : R.fin[opp(Q)][i];
+            if constexpr (OFF32)
+                d[Q] = R.fin[0][id >= 0 ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)id
+                                        : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)i];
+            else
+                d[Q] = id >= 0 ? R.fin[Q][id] : R.fin[opp(Q)][i];
             ph[Q] = id >= 0 ? phi[id] : (id == SOLID ? phi_s : phi_own);  // box faces: own phi
         });
     }
@@ -344,7 +348,14 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
         } else {
             // push destination x + xi_Q is the pull source of opp(Q)
             const int id = ld_hint(L.grid + (uint32_t)(ps + (uint32_t)grid_off<opp(Q)>(L.sy, L.sz)), pol);
-            if (id >= 0) {
+            if constexpr (OFF32) {
+                if (id != ZOUT) {  // a pore, or bounce-back from a solid voxel or lateral box face
+                    const uint32_t off = id >= 0 ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)id
+                                                 : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)j;
+                    R.aout[0][off] = va;
+                    R.bout[0][off] = vb;
+                }
+            } else if (id >= 0) {
                 R.aout[Q][id] = va;
                 R.bout[Q][id] = vb;
             } else if (id != ZOUT) {  // solid voxel or lateral box face: bounce back
@@ -555,8 +566,11 @@ int cstep_once(lbm_color* c) {
                                                    lbm::make_rates<T>(c->sp, c->sm), (T)c->alpha, (T)c->beta,
                                                    (T)c->phi_s);
         };
-        if (c->L.win && !std::getenv("GB300_LBM_COLOR_ADDR64")) launch(lbm::k_color_step<T, true>);
-        else launch(lbm::k_color_step<T, false>);
+        // GB300_LBM_COLOR_ADDR64 forces the id-grid form with 64-bit addresses (tests)
+        const bool off32 = 19 * (uint64_t)c->L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_COLOR_ADDR64");
+        if (off32 && c->L.win) launch(lbm::k_color_step<T, lbm::kWindows>);
+        else if (off32) launch(lbm::k_color_step<T, lbm::kGrid32>);
+        else launch(lbm::k_color_step<T, lbm::kGrid64>);
         return cudaGetLastError();
     });
     COLOR_CUDA(c, e);
@@ -636,7 +650,8 @@ int lbm_color_create(const uint8_t* mask, int nx, int ny, int nz, double tau, do
     c->L.sz = (int)(px * py);
     // row windows, where a window index fits the node's word and an element a 32-bit offset
     const int64_t nwin = (int64_t)lbm::windows_per_row(nx) * py * pz;
-    const bool windows = nwin < (int64_t)1 << 27 && 19 * (uint64_t)c->L.ns <= 0xFFFFFFFFull;
+    const bool windows =
+        nwin < (int64_t)1 << 27 && 19 * (uint64_t)c->L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_NO_WINDOWS");
     if (windows) {
         c->L.wy = lbm::windows_per_row(nx);
         c->L.wz = c->L.wy * (int)py;

@@ -269,7 +269,14 @@ __device__ __forceinline__ M ref_slope(const BcState* bc) {
 // -> 16.19 ms, BF16-dev two-buffer on a 157x149x171 pack 4.08 -> 3.90 ms, bitwise
 // equal states.  The id grid stays for boxes of 2^27 windows or more (and for the
 // inlet sums and conversions).
-constexpr int kWinVoxels = 30;
+// How a step kernel finds and addresses the neighbours: kGrid64 the id grid and 64-bit
+// row pointers, kGrid32 the id grid and kWindows the row windows, both with row 0 plus
+// one 32-bit element offset per neighbour (buffers of 19 ns < 2^32 elements).
+// kGrid32 serves boxes and ensembles of 2^27 windows or more, near the limit of 2^32
+// voxels, and small ensembles.  Per step of a 251x243x262 pack, kWindows, kGrid32 and
+// kGrid64: FP32 AA pattern 151, 160 and 172 us, FP16-dev 108, 137 and 157, two-buffer
+// 111, 148 and 168; FP16-dev ensemble of four 128x120x140 packs 70, 91 and 105.
+enum Form { kGrid64 = 0, kGrid32 = 1, kWindows = 2 };
 // Direction with velocity (x, y, z), -1 if there is none.
 __host__ __device__ constexpr int dir_of(int x, int y, int z) {
     for (int q = 0; q < 19; ++q)

@@ -132,7 +132,7 @@ __device__ __forceinline__ void st_stream(T* a, T v, uint64_t pol) {
 // Pull all 19 values of node i (padded voxel p): a pore source gives its own
 // value, a solid or outside source the node's opposite value (halfway
 // bounce-back; the z-outside ones are replaced by the closure).
-template <class S>
+template <class S, bool OFF32>
 __device__ __forceinline__ void pull_step(typename S::M* d, const StepPtrs<typename S::T>& P,
                                           const DevLattice& L, uint32_t p, int i, uint64_t pol_f,
                                           uint64_t pol_idx, typename S::M r_own, typename S::M g) {
@@ -144,7 +144,12 @@ __device__ __forceinline__ void pull_step(typename S::M* d, const StepPtrs<typen
         } else {
             // padded voxel indices fit in 32 bits (checked at creation)
             const int id = ld_index(L.grid + (uint32_t)(p + (uint32_t)L.goff[Q]), pol_idx);
-            const typename S::T* a = id >= 0 ? P.in[Q] + id : P.in[opp(Q)] + i;
+            const typename S::T* a;
+            if constexpr (OFF32)
+                a = P.in[0] + (id >= 0 ? (uint32_t)Q * (uint32_t)L.ns + (uint32_t)id
+                                       : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)i);
+            else
+                a = id >= 0 ? P.in[Q] + id : P.in[opp(Q)] + i;
             // a pulled value was written on plane z - xi_z (reference r_own - g xi_z)
             const M r = (cz(Q) != 0 && id >= 0) ? r_own - M(cz(Q)) * g : r_own;
             d[Q] = S::template dec<Q>(ld_stream(a, pol_f), r);
@@ -505,14 +510,13 @@ k_inlet_finish(DevLattice L, BcState* bc, int slot, const double* __restrict__ p
     density_of_parts<double, kReduceBlock>(L, bc, slot, partials, sh, true);
 }
 
-// WIN: pulls from the row windows, addressed as row 0 plus a 32-bit element
-// offset (buffers of 19 ns < 2^32 elements), as in the gather-scatter AA step.  NT
-// nodes per block.
-template <class S, bool WIN = false, int NT = kBlock>
-__global__ void __launch_bounds__(NT, step_min_blocks<S, WIN>())
+// FORM: see Form in lbm_device.cuh.  NT nodes per block.
+template <class S, int FORM = kGrid64, int NT = kBlock>
+__global__ void __launch_bounds__(NT, step_min_blocks<S, FORM == kWindows>())
 k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates,
        BcState* bc, double* __restrict__ partials) {
     using M = typename S::M;
+    constexpr bool WIN = FORM == kWindows;
     __shared__ double sh[32];
     const int64_t i64 = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int i = (int)i64;
@@ -546,7 +550,7 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
         r_own = WIN ? own_ref_word<S>(bc, L, p) : own_ref<S>(bc, L, p);
         seed = step_seed<S>(bc, slot);
         if constexpr (WIN) pull_step_win<S>(d, P, L, p, i, pol_f, r_own, g);
-        else pull_step<S>(d, P, L, p, i, pol_f, pol_idx, r_own, g);
+        else pull_step<S, FORM == kGrid32>(d, P, L, p, i, pol_f, pol_idx, r_own, g);
     }
     if ((int64_t)blockIdx.x * NT < L.a_in) drin = inlet_density<M, NT>(L, bc, slot, partials, sh, blockIdx.x == 0);
     if (i64 < L.n) {
@@ -655,22 +659,22 @@ __device__ __forceinline__ uint64_t aa_index_policy() {
 #endif
 }
 
-// WIN (gather-scatter launch, buffers of 19 ns < 2^32 elements): neighbours from
-// the row windows, every neighbour address row 0 plus one 32-bit element offset,
-// and each direction's gather offset staged in shared memory.  The scatter
+// FORM (of the gather-scatter launch; see lbm_device.cuh): with 32-bit offsets, each
+// direction's gather offset is staged in shared memory.  The scatter
 // destination of q is the gather source of opp(q) -- F[q][x + xi_q] for a pore
 // there, else the bounce-back slot F[opp q][x], both read by the gather of
 // opp(q) -- so the scatter reads its offset as it is and needs no id test or
 // offset arithmetic (the launch on the 256^3 pack, ids staged -> offsets staged:
 // 0.2006 -> 0.1825 ms FP16-dev, 0.2013 -> 0.1972 ms FP32).  Otherwise the ids of
 // the id grid are staged and the rows addressed by 64-bit pointers.
-template <class S, bool ODD, bool WIN = false, int NT = kBlock>
+template <class S, bool ODD, int FORM = kGrid64, int NT = kBlock>
 __global__ void __launch_bounds__(NT, aa_min_blocks<S, ODD>())
 k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename S::M> rates,
           BcState* bc, double* __restrict__ partials) {
     using M = typename S::M;
     __shared__ double sh[32];
-    __shared__ int sid[ODD ? 18 : 1][NT];  // gather offset (WIN) or pore id per direction
+    constexpr bool WIN = FORM == kWindows, OFF32 = FORM != kGrid64;
+    __shared__ int sid[ODD ? 18 : 1][NT];  // gather offset (OFF32) or pore id per direction
     const int64_t i64 = (int64_t)blockIdx.x * NT + threadIdx.x;
     // threads past the last node of a gather-scatter launch load its values and write
     // nothing: straight-line loads up to the barrier of inlet_density (0.9 us of 171)
@@ -716,9 +720,16 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
             for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
                 constexpr int Q = decltype(qc)::value + 1;
                 const int id = ld_aa_index(L.grid + (uint32_t)(p + (uint32_t)L.goff[Q]), pol_idx);
-                sid[Q - 1][threadIdx.x] = id;
-                d[Q] = id >= 0 ? S::template dec<Q>(F.row[opp(Q)][id], r_own - M(cz(Q)) * g)
-                               : S::template dec<Q>(F.row[Q][i], r_own);
+                if constexpr (OFF32) {
+                    const uint32_t off = id >= 0 ? (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)id
+                                                 : (uint32_t)Q * (uint32_t)L.ns + (uint32_t)i;
+                    sid[Q - 1][threadIdx.x] = (int)off;
+                    d[Q] = S::template dec<Q>(F.row[0][off], id >= 0 ? r_own - M(cz(Q)) * g : r_own);
+                } else {
+                    sid[Q - 1][threadIdx.x] = id;
+                    d[Q] = id >= 0 ? S::template dec<Q>(F.row[opp(Q)][id], r_own - M(cz(Q)) * g)
+                                   : S::template dec<Q>(F.row[Q][i], r_own);
+                }
             });
         } else {
             if constexpr (S::kRef)
@@ -741,7 +752,7 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
         // 19 64-bit addresses live across the collision
         int j;
         asm volatile("mov.b32 %0, %1;" : "=r"(j) : "r"(i));
-        if constexpr (ODD && WIN) {
+        if constexpr (ODD && OFF32) {
             F.row[0][j] = S::template enc_sr<0>(d[0], r_own, sr_key<S>(seed, i));
             // a pore destination lies in row Q, a bounce-back one in row opp(Q)
             for_q(std::make_integer_sequence<int, 18>{}, [&](auto qc) {
@@ -1612,17 +1623,19 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
             P.out[q] = (T*)fout + (int64_t)q * L.ns;
         }
         // GB300_LBM_STEP_ADDR64 forces the id-grid form with 64-bit addresses (tests)
-        if (L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64"))
-        {
+        const bool off32 = 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64");
+        if (L.win && off32) {
             if constexpr (S::kRef) {
                 k_step_pair<S><<<blocks_for(L.n, kBlock), kPair, 0, st>>>(P, slot, L, make_rates<float>(r.sp, r.sm), bc, partials);
                 return fold_parts<kPair>(L, slot, partials, kBlock, st);
             } else if (sizeof(M) == 8 && L.n < kSmallNodes)
-                k_step<S, true, kSmallBlock><<<blocks_for(L.n, kSmallBlock), kSmallBlock, 0, st>>>(
+                k_step<S, kWindows, kSmallBlock><<<blocks_for(L.n, kSmallBlock), kSmallBlock, 0, st>>>(
                     P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
             else
-                k_step<S, true><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-        } else
+                k_step<S, kWindows><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
+        } else if (off32)
+            k_step<S, kGrid32><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
+        else
             k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
         return fold_parts<kBlock>(L, slot, partials, kBlock, st);
     });
@@ -1747,9 +1760,10 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
         {
             AAPtrs<typename S::T> F;
             for (int q = 0; q < 19; ++q) F.row[q] = (typename S::T*)f + (int64_t)q * L.ns;
-            // row windows, and every element offset of the buffer in 32 bits; the
-            // environment variable GB300_LBM_AA_ADDR64 forces the id-grid form (for tests)
-            const bool win = L.win && 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_AA_ADDR64");
+            // every element offset of the buffer in 32 bits; the environment variable
+            // GB300_LBM_AA_ADDR64 forces the id-grid form with 64-bit addresses (tests)
+            const bool off32 = 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_AA_ADDR64");
+            const bool win = L.win && off32;
             const unsigned nb = blocks_for(L.n, kBlock);
             const auto rates = make_rates<M>(r.sp, r.sm);
             if constexpr (S::kRef) {
@@ -1763,15 +1777,16 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
             } else if (win && sizeof(M) == 8 && L.n < kSmallNodes) {
                 const unsigned nbs = blocks_for(L.n, kSmallBlock);
                 if (odd)
-                    k_step_aa<S, true, true, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                    k_step_aa<S, true, kWindows, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
                 else
-                    k_step_aa<S, false, false, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                    k_step_aa<S, false, kGrid64, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
                 return cudaGetLastError();
             } else if (odd && win) {
-                k_step_aa<S, true, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                k_step_aa<S, true, kWindows><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
                 return fold_parts<kBlock>(L, slot, partials, kBlock, st);
             }
-            if (odd) k_step_aa<S, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+            if (odd && off32) k_step_aa<S, true, kGrid32><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+            else if (odd) k_step_aa<S, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
             else k_step_aa<S, false><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
             return fold_parts<kBlock>(L, slot, partials, kBlock, st);
         }
