@@ -383,7 +383,7 @@ int lbm_create(const uint8_t* mask, int nx, int ny, int nz, double tau, int mode
         (rc = dev_alloc(c, &c->d_bc, sizeof(lbm::BcState))) ||
         (rc = dev_alloc(c, &c->d_red_partials, (size_t)nb_red * sizeof(double))) ||
         (rc = dev_alloc(c, &c->d_red_counter, sizeof(unsigned))) ||
-        (rc = dev_alloc(c, &c->d_parts, (size_t)2 * (c->L.part_stride + lbm::kFoldedParts) * sizeof(double))) ||
+        (rc = dev_alloc(c, &c->d_parts, (size_t)3 * c->L.part_stride * sizeof(double))) ||
         (rc = dev_alloc(c, &c->d_mon_partials, (size_t)5 * nb_mon * sizeof(double))) ||
         (rc = dev_alloc(c, &c->d_mon_counter, sizeof(unsigned))) ||
         (rc = dev_alloc(c, &c->d_mon, sizeof(lbm::MonitorOut)))) {

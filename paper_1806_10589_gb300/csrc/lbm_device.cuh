@@ -216,8 +216,7 @@ __device__ __forceinline__ void encode_node(const typename S::M* d, uint32_t see
 // drho_in[c] is the inlet density (Eq. potential) for the step that reads
 // distribution buffer c.  A step leaves the parts of the next step's inlet sum
 // (parts[c] of them, c the buffer the next step reads) and the next step adds them
-// and records drho_in[c]; parts[c] = 0 means that drho_in[c] is already set, parts[c] < 0 that
-// -parts[c] parts were added to fewer behind that step.
+// and records drho_in[c]; parts[c] = 0 means that drho_in[c] is already set.
 struct BcState {
     double Q;              // prescribed inlet flux (Eq. flux)
     double drho_in_fixed;  // inlet density when the inlet is in pressure mode

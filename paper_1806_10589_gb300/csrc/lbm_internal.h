@@ -57,11 +57,9 @@ struct MonitorOut {
 // over the inlet plane; used whenever the state or Q changes outside a step.
 cudaError_t launch_inlet_reduce(int prec, const void* fin, int slot, const DevLattice& L, BcState* bc,
                                 double* partials, unsigned* counter, cudaStream_t st);
-// Behind a step that leaves many parts of the inlet sum, they are added to this many.
-constexpr int kFoldedParts = 128;
 // One full step fin (parity `slot`) -> fout; also leaves the parts of the inlet sum
-// of the step after it in partials (two parities of L.part_stride doubles, then two
-// of kFoldedParts).
+// of the step after it in partials (two parities of L.part_stride doubles, then one
+// such row for the parts of a step that are folded behind it).
 cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const DevLattice& L, Relax r,
                         BcState* bc, double* partials, cudaStream_t st);
 // drho_in[slot] from the parts the last step left, if it left any.

@@ -401,7 +401,7 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 // tile therefore leaves one part for all its warps (112x112x24, AA pattern: 10.5 ->
 // 9.7 us; 256x256x16: 25.5 -> 24.3; below, the block's sum would only lengthen the
 // step's tail), and above LBM_PARTS_DIRECT of those a kernel behind the step adds them
-// to kFolded ones first, the count stored as its negative (512x512x16, 2,048 parts:
+// to kFolded ones first (512x512x16, 2,048 parts:
 // 117.4 us without that kernel and 118.7 with it, 600x600x16, 2,813 parts: 167.5 and
 // 165.2; 1024x1024x3 125, 2047x2047x4 8,590 -> 613).
 #ifndef LBM_WARP_PARTS
@@ -411,48 +411,48 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 #define LBM_PARTS_DIRECT 2048
 #endif
 constexpr int kPartsDirect = LBM_PARTS_DIRECT;
-constexpr int kFolded = kFoldedParts;
-// Parts of a tile of NT threads, and of a step of blocks of `nodes` nodes.
-template <int NT>
-__host__ __device__ __forceinline__ int tile_parts(const DevLattice& L) {
-    return L.a_01 <= 32 * LBM_WARP_PARTS ? NT / 32 : 1;
+constexpr int kFolded = 128;
+// TILES: one part per tile.  Both forms are compiled: as a branch of one kernel it cost
+// the steps of small lattices up to 2 % (61x67x72 FP32 7.05 -> 7.15 us).  f(TILES).
+template <class F>
+cudaError_t with_parts(const DevLattice& L, F&& f) {
+    return L.a_01 > 32 * LBM_WARP_PARTS ? f(std::true_type{}) : f(std::false_type{});
 }
-template <int NT>
+// Parts that a step in blocks of NT threads and `nodes` nodes leaves.
+template <int NT, bool TILES>
 __host__ __device__ __forceinline__ int step_parts(const DevLattice& L, int nodes) {
-    return (int)((L.a_01 + nodes - 1) / nodes) * tile_parts<NT>(L);
+    return (int)((L.a_01 + nodes - 1) / nodes) * (TILES ? 1 : NT / 32);
 }
-template <class P>
-__device__ __forceinline__ P* folded(const DevLattice& L, P* partials, int slot) {
-    return partials + 2 * L.part_stride + slot * kFolded;
-}
+// The parts of a step that folds them lie behind the two parities.
 __global__ void __launch_bounds__(kReduceBlock)
 k_inlet_fold(DevLattice L, int n, int slot, double* __restrict__ partials) {
     __shared__ double sh[32];
-    const double* p = partials + slot * L.part_stride;
+    const double* p = partials + 2 * L.part_stride;
     double s = 0.0;
     for (int j = blockIdx.x * kReduceBlock + threadIdx.x; j < n; j += kFolded * kReduceBlock) s += p[j];
     s = block_sum<kReduceBlock>(s, sh);
-    if (threadIdx.x == 0) folded(L, partials, slot)[blockIdx.x] = s;
+    if (threadIdx.x == 0) partials[slot * L.part_stride + blockIdx.x] = s;
 }
 // Behind a step that reads buffer `slot`, in blocks of NT threads and `nodes` nodes.
-template <int NT>
+template <int NT, bool TILES>
 inline cudaError_t fold_parts(const DevLattice& L, int slot, double* partials, int nodes, cudaStream_t st) {
-    const int n = step_parts<NT>(L, nodes);
-    if (n > kPartsDirect) k_inlet_fold<<<kFolded, kReduceBlock, 0, st>>>(L, n, slot ^ 1, partials);
+    const int n = step_parts<NT, TILES>(L, nodes);
+    if (TILES && n > kPartsDirect) k_inlet_fold<<<kFolded, kReduceBlock, 0, st>>>(L, n, slot ^ 1, partials);
     return cudaGetLastError();
 }
-template <class S, int NT, int NODES>
+template <class S, int NT, int NODES, bool TILES>
 __device__ __forceinline__ void store_inlet_part(double part, int64_t tile, const DevLattice& L, BcState* bc, int slot,
                                                  double* __restrict__ partials, double* sh) {
-    const int w = tile_parts<NT>(L);
+    constexpr int W = TILES ? 1 : NT / 32;
     double v;
-    if (NT > 32 && w == 1) v = block_sum<NT>(part, sh);
+    if constexpr (TILES) v = block_sum<NT>(part, sh);
     else v = warp_sum(part);
-    if ((threadIdx.x & 31) == 0 && (int)(threadIdx.x >> 5) < w)
-        partials[(slot ^ 1) * L.part_stride + tile * w + (threadIdx.x >> 5)] = v;
+    const int n = step_parts<NT, TILES>(L, NODES);
+    const bool fold = TILES && n > kPartsDirect;
+    if ((threadIdx.x & 31) == 0 && (!TILES || threadIdx.x == 0))
+        partials[(fold ? 2 : slot ^ 1) * L.part_stride + tile * W + (threadIdx.x >> 5)] = v;
     if (tile == 0 && threadIdx.x == 0) {
-        const int n = step_parts<NT>(L, NODES);
-        bc->parts[slot ^ 1] = n > kPartsDirect ? -n : n;
+        bc->parts[slot ^ 1] = fold ? kFolded : n;
         if constexpr (S::kRef) bc->sr_seed[slot ^ 1] = sr_next(bc->sr_seed[slot]);
     }
 }
@@ -465,17 +465,23 @@ template <class M, int NT>
 __device__ __forceinline__ M density_of_parts(const DevLattice& L, BcState* bc, int slot,
                                               const double* __restrict__ partials, double* sh, bool first) {
     constexpr int W = NT / 32;
-    int n = bc->parts[slot];
+    const int n = bc->parts[slot];
     if (n == 0) return M(bc->drho_in[slot]);
-    const double* p = partials + slot * L.part_stride;
-    if (n < 0) {  // folded behind the step that left them
-        p = folded(L, partials, slot);
-        n = kFolded;
-    }
+    // a 32-bit offset in the two-node kernels (NT = 128): with a pointer k_aa_even_pair
+    // spilled 40 bytes (2 % of a 45x50x60 pack's step); with an offset the FP32
+    // gather-scatter kernel spilled 8
+    using Row = std::conditional_t<NT == kBlock / 2, int, const double*>;
+    Row row;
+    if constexpr (std::is_same<Row, int>::value) row = slot * (int)L.part_stride;
+    else row = partials + slot * L.part_stride;
+    const auto part = [&](int j) {
+        if constexpr (std::is_same<Row, int>::value) return partials[row + j];
+        else return row[j];
+    };
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int vw = wid; vw < 8; vw += W) {
         double s = 0.0;
-        for (int j = vw * 32 + lane; j < n; j += 256) s += p[j];
+        for (int j = vw * 32 + lane; j < n; j += 256) s += part(j);
         s = warp_sum(s);
         if (lane == 0) sh[vw] = s;
     }
@@ -511,7 +517,7 @@ k_inlet_finish(DevLattice L, BcState* bc, int slot, const double* __restrict__ p
 }
 
 // FORM: see Form in lbm_device.cuh.  NT nodes per block.
-template <class S, int FORM = kGrid64, int NT = kBlock>
+template <class S, int FORM, int NT, bool TILES>
 __global__ void __launch_bounds__(NT, step_min_blocks<S, FORM == kWindows>())
 k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates,
        BcState* bc, double* __restrict__ partials) {
@@ -571,7 +577,7 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
         }
     }
     if ((int64_t)blockIdx.x * NT < L.a_01)
-        store_inlet_part<S, NT, NT>(part, blockIdx.x, L, bc, slot, partials, sh);
+        store_inlet_part<S, NT, NT, TILES>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // ------------------------------------------------------ AA-pattern step ---
@@ -667,7 +673,7 @@ __device__ __forceinline__ uint64_t aa_index_policy() {
 // offset arithmetic (the launch on the 256^3 pack, ids staged -> offsets staged:
 // 0.2006 -> 0.1825 ms FP16-dev, 0.2013 -> 0.1972 ms FP32).  Otherwise the ids of
 // the id grid are staged and the rows addressed by 64-bit pointers.
-template <class S, bool ODD, int FORM = kGrid64, int NT = kBlock>
+template <class S, bool ODD, int FORM, int NT, bool TILES>
 __global__ void __launch_bounds__(NT, aa_min_blocks<S, ODD>())
 k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename S::M> rates,
           BcState* bc, double* __restrict__ partials) {
@@ -792,7 +798,7 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
         }
     }
     if ((int64_t)blockIdx.x * NT < L.a_01)
-        store_inlet_part<S, NT, NT>(part, blockIdx.x, L, bc, slot, partials, sh);
+        store_inlet_part<S, NT, NT, TILES>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // ------------------------------------------- two nodes per thread (16-bit) ---
@@ -866,7 +872,7 @@ __device__ __forceinline__ double inlet_part_nodes(const F2* d, int64_t i0, int6
     return s;
 }
 
-template <class S>
+template <class S, bool TILES>
 __global__ void __launch_bounds__(kPair, LBM_PAIR_STEP_BLOCKS)
 k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float> rates, BcState* bc,
             double* __restrict__ partials) {
@@ -923,7 +929,7 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
     if ((int64_t)blockIdx.x * kBlock < L.a_01)
-        store_inlet_part<S, kPair, kBlock>(part, blockIdx.x, L, bc, slot, partials, sh);
+        store_inlet_part<S, kPair, kBlock, TILES>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // Gather-scatter launch: thread t of a warp owns the nodes 64 w + t and
@@ -931,7 +937,7 @@ k_step_pair(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<float
 // cover consecutive slots (with neighbouring nodes on a thread every store leaves
 // half of each sector to the next one: L2 throughput 65 % and the launch slower
 // than one node per thread).
-template <class S>
+template <class S, bool TILES>
 __global__ void __launch_bounds__(kPair, LBM_PAIR_ODD_BLOCKS)
 k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float> rates, BcState* bc,
               double* __restrict__ partials) {
@@ -1015,11 +1021,11 @@ k_aa_odd_pair(typename S::T* __restrict__ f, int slot, DevLattice L, Rates<float
         });
     }
     if ((int64_t)blockIdx.x * kBlock < L.a_01)
-        store_inlet_part<S, kPair, kBlock>(part, blockIdx.x, L, bc, slot, partials, sh);
+        store_inlet_part<S, kPair, kBlock, TILES>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // Node-local launch: neighbouring nodes on a thread, one 4-byte load and store per row.
-template <class S>
+template <class S, bool TILES>
 __global__ void __launch_bounds__(kPair, LBM_PAIR_EVEN_BLOCKS)
 k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<float> rates, BcState* bc,
                double* __restrict__ partials) {
@@ -1068,7 +1074,7 @@ k_aa_even_pair(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<floa
         part = inlet_part_nodes<S>(d, i64, i64 + 1, L, seed, [&](int k, auto) { return k ? r1 : r0; });
     }
     if ((int64_t)blockIdx.x * kBlock < L.a_01)
-        store_inlet_part<S, kPair, kBlock>(part, blockIdx.x, L, bc, slot, partials, sh);
+        store_inlet_part<S, kPair, kBlock, TILES>(part, blockIdx.x, L, bc, slot, partials, sh);
 }
 
 // Pull layout <-> layout S: swap F[q][x] and F[opp q][x] at every node.
@@ -1232,7 +1238,7 @@ __device__ __forceinline__ void read_vals(typename S::M* d, const unsigned char*
     });
 }
 
-template <class S, int NT>
+template <class S, int NT, bool TILES>
 __global__ void __launch_bounds__(NT)
 k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S::M> rates, BcState* bc, double* __restrict__ partials) {
     using M = typename S::M;
@@ -1302,7 +1308,7 @@ k_step_async(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<type
             if (i64 < L.a_01) part = next_inlet_part<S>(d, L, p_cur, i, r_own, seed);
         }
         if (t < nt01)  // tile holds plane z = 0 / z = 1 nodes (block-uniform)
-            store_inlet_part<S, NT, NT>(part, t, L, bc, slot, partials, sh);
+            store_inlet_part<S, NT, NT, TILES>(part, t, L, bc, slot, partials, sh);
         hi_cur = hi_next;
         nb_cur = nb_next;
         p_cur = p_next;
@@ -1624,20 +1630,32 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
         }
         // GB300_LBM_STEP_ADDR64 forces the id-grid form with 64-bit addresses (tests)
         const bool off32 = 19 * (uint64_t)L.ns <= 0xFFFFFFFFull && !std::getenv("GB300_LBM_STEP_ADDR64");
-        if (L.win && off32) {
-            if constexpr (S::kRef) {
-                k_step_pair<S><<<blocks_for(L.n, kBlock), kPair, 0, st>>>(P, slot, L, make_rates<float>(r.sp, r.sm), bc, partials);
-                return fold_parts<kPair>(L, slot, partials, kBlock, st);
-            } else if (sizeof(M) == 8 && L.n < kSmallNodes)
-                k_step<S, kWindows, kSmallBlock><<<blocks_for(L.n, kSmallBlock), kSmallBlock, 0, st>>>(
-                    P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-            else
-                k_step<S, kWindows><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-        } else if (off32)
-            k_step<S, kGrid32><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-        else
-            k_step<S><<<blocks_for(L.n, kBlock), kBlock, 0, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-        return fold_parts<kBlock>(L, slot, partials, kBlock, st);
+        const bool win = L.win && off32;
+        const unsigned nb = blocks_for(L.n, kBlock);
+        const auto rates = make_rates<M>(r.sp, r.sm);
+        if constexpr (sizeof(M) == 8) {
+            if (win && L.n < kSmallNodes) {
+                k_step<S, kWindows, kSmallBlock, false><<<blocks_for(L.n, kSmallBlock), kSmallBlock, 0, st>>>(
+                    P, slot, L, rates, bc, partials);
+                return cudaGetLastError();
+            }
+        }
+        return with_parts(L, [&](auto tiles) {
+            constexpr bool TILES = decltype(tiles)::value;
+            if (win) {
+                if constexpr (S::kRef) {
+                    k_step_pair<S, TILES><<<nb, kPair, 0, st>>>(P, slot, L, rates, bc, partials);
+                    return fold_parts<kPair, TILES>(L, slot, partials, kBlock, st);
+                } else {
+                    k_step<S, kWindows, kBlock, TILES><<<nb, kBlock, 0, st>>>(P, slot, L, rates, bc, partials);
+                }
+            } else if (off32) {
+                k_step<S, kGrid32, kBlock, TILES><<<nb, kBlock, 0, st>>>(P, slot, L, rates, bc, partials);
+            } else {
+                k_step<S, kGrid64, kBlock, TILES><<<nb, kBlock, 0, st>>>(P, slot, L, rates, bc, partials);
+            }
+            return fold_parts<kBlock, TILES>(L, slot, partials, kBlock, st);
+        });
     });
 }
 
@@ -1652,25 +1670,30 @@ cudaError_t launch_async_t(const void* fin, void* fout, int slot, const DevLatti
         P.out[q] = (T*)fout + (int64_t)q * L.ns;
     }
     const size_t smem = async_smem_bytes<NT>(AsyncSlot<S>::kBytes);
-    k_step_async<S, NT><<<grid, NT, smem, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
-    return fold_parts<NT>(L, slot, partials, NT, st);
+    return with_parts(L, [&](auto tiles) {
+        constexpr bool TILES = decltype(tiles)::value;
+        k_step_async<S, NT, TILES><<<grid, NT, smem, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
+        return fold_parts<NT, TILES>(L, slot, partials, NT, st);
+    });
 }
 
 template <class S, int NT>
-cudaError_t config_async_t(int* grid, int64_t n) {
+cudaError_t config_async_t(int* grid, const DevLattice& L) {
     const size_t smem = async_smem_bytes<NT>(AsyncSlot<S>::kBytes);
-    cudaError_t e = cudaFuncSetAttribute(k_step_async<S, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0, dev = 0, sms = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_async<S, NT>, NT, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    const int64_t ntiles = (n + NT - 1) / NT;
-    *grid = (int)std::min<int64_t>((int64_t)per_sm * sms, ntiles);
-    return cudaSuccess;
+    return with_parts(L, [&](auto tiles) {
+        auto* kernel = k_step_async<S, NT, decltype(tiles)::value>;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        int per_sm = 0, dev = 0, sms = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, smem);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        const int64_t ntiles = (L.n + NT - 1) / NT;
+        *grid = (int)std::min<int64_t>((int64_t)per_sm * sms, ntiles);
+        return cudaSuccess;
+    });
 }
 
 cudaError_t launch_inlet_finish(const DevLattice& L, BcState* bc, int slot, const double* partials, cudaStream_t st) {
@@ -1766,29 +1789,35 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
             const bool win = L.win && off32;
             const unsigned nb = blocks_for(L.n, kBlock);
             const auto rates = make_rates<M>(r.sp, r.sm);
-            if constexpr (S::kRef) {
-                if (win) {
+            if constexpr (sizeof(M) == 8) {
+                if (win && L.n < kSmallNodes) {
+                    const unsigned nbs = blocks_for(L.n, kSmallBlock);
                     if (odd)
-                        k_aa_odd_pair<S><<<nb, kPair, 0, st>>>((typename S::T*)f, slot, L, rates, bc, partials);
+                        k_step_aa<S, true, kWindows, kSmallBlock, false><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
                     else
-                        k_aa_even_pair<S><<<nb, kPair, 0, st>>>(F, slot, L, rates, bc, partials);
-                    return fold_parts<kPair>(L, slot, partials, kBlock, st);
+                        k_step_aa<S, false, kGrid64, kSmallBlock, false><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                    return cudaGetLastError();
                 }
-            } else if (win && sizeof(M) == 8 && L.n < kSmallNodes) {
-                const unsigned nbs = blocks_for(L.n, kSmallBlock);
-                if (odd)
-                    k_step_aa<S, true, kWindows, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-                else
-                    k_step_aa<S, false, kGrid64, kSmallBlock><<<nbs, kSmallBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-                return cudaGetLastError();
-            } else if (odd && win) {
-                k_step_aa<S, true, kWindows><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-                return fold_parts<kBlock>(L, slot, partials, kBlock, st);
             }
-            if (odd && off32) k_step_aa<S, true, kGrid32><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-            else if (odd) k_step_aa<S, true><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-            else k_step_aa<S, false><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
-            return fold_parts<kBlock>(L, slot, partials, kBlock, st);
+            return with_parts(L, [&](auto tiles) {
+                constexpr bool TILES = decltype(tiles)::value;
+                if constexpr (S::kRef) {
+                    if (win) {
+                        if (odd)
+                            k_aa_odd_pair<S, TILES><<<nb, kPair, 0, st>>>((typename S::T*)f, slot, L, rates, bc, partials);
+                        else
+                            k_aa_even_pair<S, TILES><<<nb, kPair, 0, st>>>(F, slot, L, rates, bc, partials);
+                        return fold_parts<kPair, TILES>(L, slot, partials, kBlock, st);
+                    }
+                } else if (odd && win) {
+                    k_step_aa<S, true, kWindows, kBlock, TILES><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                    return fold_parts<kBlock, TILES>(L, slot, partials, kBlock, st);
+                }
+                if (odd && off32) k_step_aa<S, true, kGrid32, kBlock, TILES><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                else if (odd) k_step_aa<S, true, kGrid64, kBlock, TILES><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                else k_step_aa<S, false, kGrid64, kBlock, TILES><<<nb, kBlock, 0, st>>>(F, slot, L, rates, bc, partials);
+                return fold_parts<kBlock, TILES>(L, slot, partials, kBlock, st);
+            });
         }
     });
 }
@@ -1815,8 +1844,8 @@ cudaError_t configure_step(int prec, int variant, const DevLattice& L, StepConfi
     if (variant == 0) return cudaSuccess;
     return dispatch(prec, [&](auto s) {
         using S = decltype(s);
-        if (variant == 1) return config_async_t<S, 256>(&cfg->grid, L.n);
-        if (variant == 2) return config_async_t<S, 128>(&cfg->grid, L.n);
+        if (variant == 1) return config_async_t<S, 256>(&cfg->grid, L);
+        if (variant == 2) return config_async_t<S, 128>(&cfg->grid, L);
         return cudaErrorInvalidValue;
     });
 }
