@@ -61,10 +61,10 @@ struct Member {
     uint32_t sr_seed[2];        // stochastic-rounding seed of the step reading buffer c (16-bit)
 };
 
-// LBM_BATCH16_PAIR_SCATTER: as LBM_AA16_PAIR_SCATTER, for the ensemble's
-// gather-scatter step.  Measured on the 64-pack FP16-dev ensemble, the
-// opposite order from the single lattice: its AA step takes 1.234 ms with one
-// conversion per pair and 1.243 ms with one per value.
+// LBM_BATCH16_PAIR_SCATTER: 1 = the ensemble's 16-bit gather-scatter step rounds each
+// opposite pair with one conversion before its two stores, 0 = one conversion per
+// value next to its store.  Measured on the 64-pack FP16-dev ensemble: its AA step
+// takes 1.234 ms with one conversion per pair and 1.243 ms with one per value.
 #ifndef LBM_BATCH16_PAIR_SCATTER
 #define LBM_BATCH16_PAIR_SCATTER 1
 #endif
@@ -246,16 +246,19 @@ __device__ __forceinline__ void batch_tile_step(const typename S::T* fin, typena
     double part = 0.0;
     if (il < m.n) {
         const uint32_t p = WIN ? __ldg(K.nodew + i) : K.vox[i];  // node word or padded voxel
-        const M r_own = WIN ? member_ref_word<S>(m, p) : member_ref<S>(m, p), g = member_slope<S>(m);
+        M r_own = M(0);
+        if constexpr (!WIN) r_own = member_ref<S>(m, p);
+        const M g = member_slope<S>(m);
         const uint32_t seed = S::kRef ? ld_state<COH>(&m.sr_seed[slot]) : 0u;
         M d[19];
         if constexpr (WIN) {
-            d[0] = S::template dec<0>(fin[i], r_own);
+            static_assert(!S::kRef, "k_batch_pair");
+            d[0] = fin[i];
             for_links(K.win, p, m.wy, m.wz, (uint32_t)i, [&](auto qc, bool pore, uint32_t id) {
                 constexpr int Q = decltype(qc)::value;
                 const uint32_t off =
                     pore ? (uint32_t)Q * (uint32_t)ns + id : (uint32_t)opp(Q) * (uint32_t)ns + (uint32_t)i;
-                d[Q] = S::template dec<Q>(fin[off], (cz(Q) != 0 && pore) ? r_own - M(cz(Q)) * g : r_own);
+                d[Q] = fin[off];
             });
         } else {
             for_q(AllQ{}, [&](auto qc) {
@@ -316,10 +319,10 @@ constexpr int batch_min_blocks() {
 
 // Ensembles of fewer tiles (8 a SM) fit one or two waves: their step is a chain of
 // latencies, where one node per thread and the id grid (resident in L2) are
-// shorter.  Per step, FP16-dev, id grid against windows with pairs: 83,816 pores 9.3
-// and 10.0 us, 365,138 pores 11.3 and 11.2, 707,421 pores 19.1 and 15.4; FP32 8.8
-// and 9.1, 10.5 and 10.3, 22.1 and 20.8 (before the id-grid form's inlet tiles got 0.7
-// to 1.4 us shorter, see next_inlet_part_b; from 1,216 tiles they hide behind the rest).
+// shorter.  Per step, FP16-dev, id grid against windows with pairs: 697 tiles 9.7 and
+// 10.8 us, 1,021 12.3 and 13.3, 1,523 14.4 and 14.2, 2,035 16.9 and 16.5, 3,313 24.4 and
+// 21.3; FP32 8.9 and 8.6 (8.5 and 8.7 at 48 registers), 11.4 and 11.3, 13.5 and 13.4,
+// 17.2 and 16.1, 30.3 and 28.5.
 #ifndef LBM_WINDOW_TILES
 #define LBM_WINDOW_TILES (8 * 152)
 #endif

@@ -325,7 +325,8 @@ k_color_step(const ColorRows<T> R, const T* __restrict__ phi, DevLattice L, cons
                      T(mrow(14, Q) / mnorm2(14)) * dm14 + T(mrow(15, Q) / mnorm2(15)) * dm15;
         R.fout[Q][j] = d[Q] + sp * df;
     });
-    // D3Q7 mass transport with recolouring (push); destinations looked up again
+    // D3Q7 mass transport with recolouring (push); the destinations were staged above
+    // (row windows) or are looked up again (id grid)
     const T na = R.nab[0][j], nb = R.nab[1][j];
     const bool inlet = j < L.a_in, outlet = (int64_t)j >= L.n - L.a_out;
     uint32_t ps = 0;

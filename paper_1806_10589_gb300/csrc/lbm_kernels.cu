@@ -6,12 +6,16 @@
 //                   collision (Appendix A) and the store.  The same launch also
 //                   forms the NEXT step's inlet density: every stored value that
 //                   the next step pulls into an inlet node's known sum (Eq.
-//                   inlet) is added, in FP64, by the node that produces it, then
-//                   deterministic per-warp parts that the next step adds.
+//                   inlet) is added by the node that produces it (FP32 values
+//                   without error in FP32 words, FP64 values in FP64), and each
+//                   warp or tile stores its FP64 part of the sum, which the next
+//                   step adds in a fixed order.
+//   k_step_pair     the same for the 16-bit formats, two nodes per thread.
 //   k_inlet_reduce  the same density by a pull over the inlet plane, for states
 //                   set from outside a step (creation, set_*, a new Q).
-//   k_step_aa       the same step on ONE buffer (AA pattern, FP64/FP32), with
-//                   the layout swaps k_aa_swap / k_aa_unstream around a call.
+//   k_step_aa       the same step on ONE buffer (AA pattern), with the layout swaps
+//                   k_aa_swap / k_aa_unstream around a call; k_aa_odd_pair and
+//                   k_aa_even_pair for the 16-bit formats.
 //   k_monitors      FP64 mass / flux / max|u| / NaN reductions of a state.
 //   k_export, k_init_eq, k_encode, k_decode   field and state conversions.
 #include <algorithm>
@@ -38,9 +42,9 @@ constexpr int kReduceBlock = 256;
 #ifndef LBM_STEP_WIN_BLOCKS
 #define LBM_STEP_WIN_BLOCKS 5
 #endif
-template <class S, bool WIN = false>
+template <class S, bool WIN>
 constexpr int step_min_blocks() {
-    return sizeof(typename S::M) == 8 ? 1 : (WIN && !S::kRef) ? LBM_STEP_WIN_BLOCKS : LBM_STEP_MIN_BLOCKS;
+    return sizeof(typename S::M) == 8 ? 1 : WIN ? LBM_STEP_WIN_BLOCKS : LBM_STEP_MIN_BLOCKS;
 }
 
 template <int... Qs, class F>
@@ -84,7 +88,8 @@ struct StepPtrs {
 
 // The per-node kernel forms the next step's inlet contribution from the
 // registers (FP32/FP64: measured faster) or by reloading the values it has just
-// stored (16-bit formats: frees the decode state, measured faster).
+// stored (16-bit formats, which it serves where there are no row windows: frees the
+// decode state, measured faster).
 // LBM_CONTRIB_RELOAD = 0 / 1 forces one way for every format.
 template <class S>
 __host__ __device__ constexpr bool contrib_reload() {
@@ -158,19 +163,17 @@ __device__ __forceinline__ void pull_step(typename S::M* d, const StepPtrs<typen
 }
 
 // The same from the row windows: every source is row 0 plus one 32-bit element
-// offset (rows are ns apart, buffers of fewer than 2^32 elements).
+// offset (rows are ns apart, buffers of fewer than 2^32 elements).  FP32 and FP64: the
+// 16-bit formats take two nodes per thread there.
 template <class S>
 __device__ __forceinline__ void pull_step_win(typename S::M* d, const StepPtrs<typename S::T>& P, const DevLattice& L,
-                                              uint32_t word, int i, uint64_t pol_f, typename S::M r_own,
-                                              typename S::M g) {
-    using M = typename S::M;
-    d[0] = S::template dec<0>(ld_stream(P.in[0] + i, pol_f), r_own);
+                                              uint32_t word, int i, uint64_t pol_f) {
+    static_assert(!S::kRef, "k_step_pair");
+    d[0] = ld_stream(P.in[0] + i, pol_f);
     for_links(L.win, word, L.wy, L.wz, (uint32_t)i, [&](auto qc, bool pore, uint32_t id) {
         constexpr int Q = decltype(qc)::value;
         const uint32_t off = pore ? (uint32_t)Q * (uint32_t)L.ns + id : (uint32_t)opp(Q) * (uint32_t)L.ns + (uint32_t)i;
-        // a pulled value was written on plane z - xi_z (reference r_own - g xi_z)
-        const M r = (cz(Q) != 0 && pore) ? r_own - M(cz(Q)) * g : r_own;
-        d[Q] = S::template dec<Q>(ld_stream(P.in[0] + off, pol_f), r);
+        d[Q] = ld_stream(P.in[0] + off, pol_f);
     });
 }
 
@@ -553,9 +556,9 @@ k_step(const StepPtrs<typename S::T> P, int slot, DevLattice L, Rates<typename S
     if (i64 < L.n) {
         p = ld_index((WIN ? L.nodew : L.vox) + i, pol_idx);  // node word or padded voxel
         const M g = own_slope<S>(bc);
-        r_own = WIN ? own_ref_word<S>(bc, L, p) : own_ref<S>(bc, L, p);
+        if constexpr (!WIN) r_own = own_ref<S>(bc, L, p);
         seed = step_seed<S>(bc, slot);
-        if constexpr (WIN) pull_step_win<S>(d, P, L, p, i, pol_f, r_own, g);
+        if constexpr (WIN) pull_step_win<S>(d, P, L, p, i, pol_f);
         else pull_step<S, FORM == kGrid32>(d, P, L, p, i, pol_f, pol_idx, r_own, g);
     }
     if ((int64_t)blockIdx.x * NT < L.a_in) drin = inlet_density<M, NT>(L, bc, slot, partials, sh, blockIdx.x == 0);
@@ -706,16 +709,15 @@ k_step_aa(const AAPtrs<typename S::T> F, int slot, DevLattice L, Rates<typename 
         // value read from the neighbour x - xi_q decodes with r(z - xi_z).
         seed = step_seed<S>(bc, slot);
         if constexpr (ODD && WIN) {
+            static_assert(!S::kRef, "k_aa_odd_pair");
             const uint32_t word = ld_aa_index(L.nodew + i, aa_index_policy());
-            r_own = own_ref_word<S>(bc, L, word);
-            g = own_slope<S>(bc);
-            d[0] = S::template dec<0>(F.row[0][i], r_own);
+            d[0] = F.row[0][i];
             for_links(L.win, word, L.wy, L.wz, (uint32_t)i, [&](auto qc, bool pore, uint32_t id) {
                 constexpr int Q = decltype(qc)::value;
                 const uint32_t off =
                     pore ? (uint32_t)opp(Q) * (uint32_t)L.ns + id : (uint32_t)Q * (uint32_t)L.ns + (uint32_t)i;
                 sid[Q - 1][threadIdx.x] = (int)off;
-                d[Q] = S::template dec<Q>(F.row[0][off], (S::kRef && pore) ? r_own - M(cz(Q)) * g : r_own);
+                d[Q] = F.row[0][off];
             });
         } else if constexpr (ODD) {
             const uint64_t pol_idx = aa_index_policy();
@@ -1573,7 +1575,9 @@ __global__ void k_node_words(const uint32_t* __restrict__ vox, uint32_t vox0, in
 
 // FP64 lattices of at most one wave of 256-node blocks (152 SMs, one such block
 // resident) run in small blocks, so that every SM's FP64 units get an even share:
-// 16x16x64 duct, 12,544 nodes, 100 steps 2.05 -> 1.64 ms.  FP32 (61x67x72 pack,
+// 16x16x64 duct, 12,544 nodes, 100 steps 2.05 -> 1.64 ms.  Near the line, per step in
+// small blocks and before them: 30x30x48 duct, 37,632 nodes 16.5 and 22.2 us; above it
+// (32x32x48, 43,200 nodes, two waves of 256-node blocks) 23.8 and 31.8 us.  FP32 (61x67x72 pack,
 // 112 k nodes) measured slower: 1.01 ms in blocks of 256, 1.02 in 128, 1.17 in 64.
 constexpr int64_t kSmallNodes = 152 * 256;
 constexpr int kSmallBlock = 32;

@@ -29,9 +29,13 @@
 //     A: activation rows (K-major), B: weights [Cout][27*Cin] (K-major); K
 //     streamed through a TMA -> shared memory -> tcgen05 pipeline in chunks
 //     of 64 (or 32) channels of one tap.
+//     k_conv_march keeps a narrow layer's weights resident and marches along z.
 //   weight gradient (k_wgrad):  D[(tap, ci) x co] = sum_rows act[r + off(tap)][ci] g[r][co]
 //     A: 128 (tap, channel) pairs of shifted activation rows (MN-major),
-//     B: output-gradient rows (MN-major); split over rows, FP32 atomics.
+//     B: output-gradient rows (MN-major); split over rows into partial sums
+//     (network) or FP32 atomics (single calls).
+//   weight gradient of narrow layers on large volumes (k_wgrad_march):
+//     D[(dy, ci) x (dx, co)] per dz, planes resident along z.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -126,12 +130,10 @@ struct ConvCfg {
     // (AW * 2 bytes) apart, so a tile loads its input rows 9 times instead of 27.
     // Wide outputs keep one tap per stage (128 rows): their weights, not the
     // activations, dominate the bytes.  Measured on the 32 -> 32 layer, 8 x 64^3
-    // voxels, per forward launch: 0.474 ms one tap per stage, 0.390 ms with the
-    // window as four unswizzled 8-channel planes, 0.318 ms as one swizzled box,
-    // 0.311 ms with the three taps' weights as one box of the tap-major copy;
-    // slower: a persistent form with two TMEM accumulators (0.416 ms), weights
-    // kept resident in shared memory (0.557 ms one tile per CTA, 0.458 ms
-    // persistent).
+    // voxels, per forward launch of this kernel: 0.474 ms one tap per stage, 0.390 ms
+    // with the window as four unswizzled 8-channel planes, 0.318 ms as one swizzled
+    // box, 0.311 ms with the three taps' weights as one box of the tap-major copy
+    // (k_conv_march, which takes that layer there: 0.242 ms).
     static constexpr bool FUSE = COUT <= 64;
     static constexpr int NITER = (FUSE ? 9 : 27) * KSUB;
     static constexpr int HALO = kRows + 2;
@@ -324,10 +326,10 @@ k_conv(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorM
 // every input plane of the patch (with a halo of one row line and one row) is
 // loaded once and used for all 27 taps, adding to the three output planes z - 1,
 // z, z + 1, each with its own accumulators in tensor memory (3 T N columns).  Row
-// lines y = -1, Y and planes z = -1, Z of the output are not written.  A finished output plane drains while the MMAs of the next input plane run.  The
-// taps of an output accumulate in k_conv's order (dz, dy, dx, channel), so the
+// lines y = -1, Y and planes z = -1, Z of the output are not written.  A finished output
+// plane drains while the MMAs of the next input plane run.  The taps of an output accumulate in k_conv's order (dz, dy, dx, channel), so the
 // results are bitwise the same.  Measured, 32 -> 32 channels on 8 x 64^3 voxels:
-// 316 -> 242 us; 64 -> 32 at 128x120x136: 903 -> about 500 us.  What is left is the
+// 311 -> 242 us; 64 -> 32: 783 -> 478 us (where it is slower: MarchCost).  What is left is the
 // tensor core's own pace: 65 cycles for each 128 x 32 x 16 product (86 % of the
 // cycles), against 16 of arithmetic.
 //   The operand of tap (dy, dx) and tile t is the resident plane started
@@ -1072,9 +1074,9 @@ __global__ void k_mse(const float* __restrict__ Y, const float* __restrict__ T, 
 // is enough where there are many weights or few splits.  Of few weights and many
 // splits (the narrow layers) it left the card waiting on its chain of loads: there 8
 // threads per w each add every eighth split, then the eight sums are added in order.
-// Gradient of the 4-level network, us, one thread / eight / by the rule below: 1 x
-// 16^3 1335 (previous kernels), 1421, 1340; 8 x 32^3 - , 2986, 2860; 8 x 64^3 -, 8807,
-// 8661 (a rule at 16 splits and 300,000 weights: 1332, 2866, 8676).
+// Gradient of the 4-level network, eight threads throughout and by split_sum's rule: 1 x
+// 16^3 1421 and 1340 us, 8 x 32^3 2986 and 2860, 8 x 64^3 8807 and 8661 (the line at 16
+// splits and 300,000 weights: 1332, 2866 and 8676).
 __global__ void __launch_bounds__(256)
 k_split_sum1(const float* __restrict__ part, int64_t splits, int64_t nw, float* __restrict__ gw) {
     const int64_t w = (int64_t)blockIdx.x * 256 + threadIdx.x;
