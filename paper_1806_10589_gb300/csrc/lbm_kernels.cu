@@ -400,15 +400,16 @@ __device__ __forceinline__ double next_inlet_part_stored(const StepPtrs<typename
 // against 9.1 at 365k.)
 //   Every block with inlet nodes adds all parts, which costs the square of the inlet
 // area: with one part per warp throughout, an open FP32 lattice of 1024x1024x3 took
-// 602 us per step, of 512x512x16 139.  Above 32 LBM_WARP_PARTS nodes on the planes a
-// tile therefore leaves one part for all its warps (112x112x24, AA pattern: 10.5 ->
-// 9.7 us; 256x256x16: 25.5 -> 24.3; below, the block's sum would only lengthen the
-// step's tail), and above LBM_PARTS_DIRECT of those a kernel behind the step adds them
-// to kFolded ones first (512x512x16, 2,048 parts:
-// 117.4 us without that kernel and 118.7 with it, 600x600x16, 2,813 parts: 167.5 and
-// 165.2; 1024x1024x3 125, 2047x2047x4 8,590 -> 613).
+// 602 us per step, of 512x512x16 139.  Above LBM_WARP_PARTS warps of nodes on the planes
+// (FP64: twice as many, its steps being longer) a tile therefore leaves one part for
+// all its warps (FP32 packs, AA pattern: 140x160x100, 1,400 warps 21.4 us per step with
+// a part per warp and 21.7 with one per tile, 250x250x24, 3,906 warps 24.7 and 24.2;
+// FP64 241.8 and 243.7 there), and above LBM_PARTS_DIRECT of those a kernel behind the
+// step adds them to kFolded ones first (512x512x16, 2,048 parts: 117.4 us without that
+// kernel and 118.7 with it, 600x600x16, 2,813 parts: 167.5 and 165.2; 1024x1024x3 125,
+// 2047x2047x4 8,590 -> 613).
 #ifndef LBM_WARP_PARTS
-#define LBM_WARP_PARTS 512
+#define LBM_WARP_PARTS 2048
 #endif
 #ifndef LBM_PARTS_DIRECT
 #define LBM_PARTS_DIRECT 2048
@@ -417,9 +418,10 @@ constexpr int kPartsDirect = LBM_PARTS_DIRECT;
 constexpr int kFolded = 128;
 // TILES: one part per tile.  Both forms are compiled: as a branch of one kernel it cost
 // the steps of small lattices up to 2 % (61x67x72 FP32 7.05 -> 7.15 us).  f(TILES).
-template <class F>
+template <class M, class F>
 cudaError_t with_parts(const DevLattice& L, F&& f) {
-    return L.a_01 > 32 * LBM_WARP_PARTS ? f(std::true_type{}) : f(std::false_type{});
+    constexpr int64_t kNodes = 32 * LBM_WARP_PARTS * (sizeof(M) == 8 ? 2 : 1);
+    return L.a_01 > kNodes ? f(std::true_type{}) : f(std::false_type{});
 }
 // Parts that a step in blocks of NT threads and `nodes` nodes leaves.
 template <int NT, bool TILES>
@@ -1644,7 +1646,7 @@ cudaError_t launch_step(int prec, const void* fin, void* fout, int slot, const D
                 return cudaGetLastError();
             }
         }
-        return with_parts(L, [&](auto tiles) {
+        return with_parts<M>(L, [&](auto tiles) {
             constexpr bool TILES = decltype(tiles)::value;
             if (win) {
                 if constexpr (S::kRef) {
@@ -1674,7 +1676,7 @@ cudaError_t launch_async_t(const void* fin, void* fout, int slot, const DevLatti
         P.out[q] = (T*)fout + (int64_t)q * L.ns;
     }
     const size_t smem = async_smem_bytes<NT>(AsyncSlot<S>::kBytes);
-    return with_parts(L, [&](auto tiles) {
+    return with_parts<M>(L, [&](auto tiles) {
         constexpr bool TILES = decltype(tiles)::value;
         k_step_async<S, NT, TILES><<<grid, NT, smem, st>>>(P, slot, L, make_rates<M>(r.sp, r.sm), bc, partials);
         return fold_parts<NT, TILES>(L, slot, partials, NT, st);
@@ -1683,8 +1685,9 @@ cudaError_t launch_async_t(const void* fin, void* fout, int slot, const DevLatti
 
 template <class S, int NT>
 cudaError_t config_async_t(int* grid, const DevLattice& L) {
+    using M = typename S::M;
     const size_t smem = async_smem_bytes<NT>(AsyncSlot<S>::kBytes);
-    return with_parts(L, [&](auto tiles) {
+    return with_parts<M>(L, [&](auto tiles) {
         auto* kernel = k_step_async<S, NT, decltype(tiles)::value>;
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1803,7 +1806,7 @@ cudaError_t launch_aa_step(int prec, void* f, int odd, int slot, const DevLattic
                     return cudaGetLastError();
                 }
             }
-            return with_parts(L, [&](auto tiles) {
+            return with_parts<M>(L, [&](auto tiles) {
                 constexpr bool TILES = decltype(tiles)::value;
                 if constexpr (S::kRef) {
                     if (win) {

@@ -1,6 +1,6 @@
-"""Wide inlets (GB300).  A step leaves its parts of the inlet sum per warp, from 16,384
-nodes on the planes z = 0 and z = 1 per 256-node tile, and from 524,288 nodes they are
-added to 128 behind the step."""
+"""Wide inlets (GB300).  A step leaves its parts of the inlet sum per warp, from 65,536
+nodes on the planes z = 0 and z = 1 (FP64: 131,072) per 256-node tile, and from 524,288
+nodes they are added to 128 behind the step."""
 import numpy as np
 import pytest
 
