@@ -687,8 +687,8 @@ k_wgrad(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensor
 // interior lines, rounded up to 16 rows of zeros.
 //   The tensor core truncates as it adds, so the error of a sum grows with the
 // products added in one accumulator.  An accumulator is therefore drained (added
-// to the CTA's partial sums in FP32) before it has taken more products of 16 rows
-// than a split of k_wgrad would: on 64 -> 64 channels, 4 x 44x52x36
+// to the CTA's partial sums in FP32) before it has taken more products of 16 interior
+// rows than a split of k_wgrad would: on 64 -> 64 channels, 4 x 44x52x36
 // voxels, the error against 64 bits is 1.5e-6 of the gradient, 1.6e-6 with k_wgrad
 // (6.2e-6 with one drain per CTA).
 template <int CIN, int COUT>
@@ -1381,24 +1381,31 @@ cudaError_t march_t(const bf16* in, const bf16* wt, int cout, const ConvEpi& epi
 
 // Patch of a marching weight gradient: the largest T for which the resident
 // planes and one more of each kind fit (more tiles: fewer halo rows), cut to the
-// smallest with as many patches (even patches: a CTA's share is counted in patches).
-// Volumes whose accumulators would take under kMarchProducts products stay with
-// k_wgrad: a march would add more products in one accumulator than its row splits do
-// (at a limit of 64 throughout, 32 -> 64 channels on 8 x 24^3 voxels were off by
-// 5.8e-7 of the gradient instead of 3.7e-7) or drain it at every step (28.7 us
-// instead of 22.6 on 24^3).  The zero
-// rows after a patch (up to 16) have to end before the next plane's interior:
-// padded lines of 8 rows or more.
-constexpr int kMarchProducts = 64;
+// smallest with as many patches (even patches: a CTA's share is counted in patches)
+// and, where an accumulator takes few products, to one whose steps fill it to three
+// quarters.  The zero rows after a patch (up to 16) have to end before the next
+// plane's interior: padded lines of 8 rows or more.
+//   An accumulator takes as many products as a row split of k_wgrad has of interior
+// rows, and a sixteenth more (the error against 64 bits is then 0.8 to 1.0 of k_wgrad's
+// on 23 volumes; fewer partial sums make up for it); volumes where that is under
+// march_products stay with k_wgrad.  A longer sum would be less exact (64 products
+// throughout: 32 -> 64 channels on 8 x 24^3 voxels off by 5.8e-7 of the gradient instead
+// of 3.7e-7), and a shorter one is drained so often that the march is the slower form
+// (k_wgrad and march, us: 32 -> 32 on 4 x 24x32x40, 29 products, 43 and 55, on 8 x
+// 16x64x24, 48, 66 and 53, on 64^3, 58, 72 and 49; 64 -> 32 on 24^3 20.5 and 26.7, on
+// 64^3 131 and 88; 32 -> 64 on 4 x 24x48x56, 61, 93 and 98, on 3 x 64x40x48, 82, 115 and
+// 107; 64 -> 64 on 4 x 24x32x40, 58, 93 and 102, on 3 x 40^3, 87, 121 and 95).
+constexpr int march_products(int cout) { return cout == 32 ? 47 : 63; }
 template <int CIN, int COUT>
 bool wm_plan(const PGeo& g, int n_sm, WmArgs* out, size_t* smem) {
     using K = WmCfg<CIN, COUT>;
-    const int64_t limit = g.rows() / wgrad_splits(CIN, COUT, g.rows(), n_sm) / 16;
-    if (g.xp() < 8 || limit < kMarchProducts) return false;
     const int64_t lines = (int64_t)g.Y * g.xp();
+    const int64_t limit = 17 * (g.B * g.Z * lines) / (16 * wgrad_splits(CIN, COUT, g.rows(), n_sm) * 16);
+    if (g.xp() < 8 || limit < march_products(COUT)) return false;
     const auto patches_of = [&](int T) { return (lines + T * kRows - 1) / (T * kRows); };
     for (int T = 4; T >= 1; --T) {
         if (T > 1 && patches_of(T - 1) == patches_of(T)) continue;
+        if (limit < 64 && 4 * (limit / (8 * T) * (8 * T)) < 3 * limit) continue;
         for (int nseg = 1; nseg <= 3; nseg += 2) {
             const int rows = nseg == 1 ? T * kRows + 2 * g.xp() : T * kRows;
             WmArgs a{};

@@ -15,6 +15,8 @@ BOUNDS = {((8, 24, 24, 24), (32, 32)): 3.80e-7, ((8, 24, 24, 24), (32, 64)): 3.7
           ((8, 24, 24, 24), (64, 32)): 3.69e-7, ((1, 48, 48, 48), (32, 64)): 3.74e-7,
           ((3, 30, 20, 60), (64, 64)): 4.99e-7, ((1, 20, 20, 20), (32, 32)): 1.72e-7,
           ((1, 20, 20, 20), (64, 32)): 1.69e-7, ((2, 17, 20, 33), (64, 64)): 2.20e-7,
+          ((1, 64, 64, 64), (32, 32)): 6.39e-7, ((1, 64, 64, 64), (64, 32)): 6.46e-7,
+          ((8, 72, 4, 72), (64, 32)): 4.18e-7, ((8, 72, 4, 72), (64, 64)): 6.34e-7,
           ((8, 40, 40, 40), (32, 64)): 1.25e-6, ((4, 36, 52, 44), (64, 64)): 1.66e-6}
 
 

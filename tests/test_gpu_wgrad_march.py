@@ -9,15 +9,15 @@ from test_gpu_wsnet import _bf16, _he, _padded, torch  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
-SHAPE = (4, 500, 8, 14)  # B, Z, Y, X: planes of 128 rows, 8 products each
+SHAPE = (5, 500, 8, 14)  # B, Z, Y, X: planes of 128 rows, 8 products each
 
 
 def _rule(torch, shape, splits, sets):  # noqa: F811
-    """Products of 16 rows that an accumulator may take, and that a CTA has in all
-    (`sets` CTAs share a plane)."""
+    """Products of 16 interior rows that an accumulator may take, and that a CTA has in
+    all (`sets` CTAs share a plane)."""
     B, Z, Y, X = shape
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    limit = B * (Z + 2) * (Y + 2) * (X + 2) // (splits * sms) // 16
+    limit = 17 * B * Z * Y * (X + 2) // (16 * splits * sms * 16)
     return limit, B * Z * (Y * (X + 2) // 16) // (sms // sets)
 
 
@@ -28,7 +28,7 @@ def test_weight_gradient_with_drains(torch, cin, cout, splits, sets):  # noqa: F
 
     B, Z, Y, X = SHAPE
     limit, products = _rule(torch, SHAPE, splits, sets)
-    assert 64 <= limit < products, (limit, products)
+    assert 63 <= limit < products, (limit, products)
     rng = np.random.default_rng(cin + 3 * cout)
     ta, a = _padded(torch, rng.standard_normal((B, cin, Z, Y, X)))
     tg, g = _padded(torch, rng.standard_normal((B, cout, Z, Y, X)))
@@ -53,7 +53,7 @@ def test_network_gradient_with_drains(torch, base, splits, sets):  # noqa: F811
 
     B, shape = SHAPE[0], SHAPE[1:]
     limit, products = _rule(torch, SHAPE, splits, sets)
-    assert 64 <= limit < products, (limit, products)
+    assert 63 <= limit < products, (limit, products)
     rng = np.random.default_rng(base)
     masks = (rng.random((B,) + shape) < 0.35).astype(np.uint8)
     targets = rng.standard_normal((B, N.NOUT) + shape).astype(np.float32)
