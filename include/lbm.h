@@ -404,8 +404,8 @@ const char* lbm_wsnet_last_error(const lbm_wsnet* net);
  *   op 2, weight gradient:  out[co][t][ci] += sum_v aux[v][co] in[v + t][ci]
  *         (in: the layer input, cin channels; aux: the output gradient, cout
  *          channels, zero on border rows; out: FP32 [cout][27][cin], added to
- *          with FP32 atomics, one per row split: the order of those additions,
- *          and so the last bits, may vary between calls)
+ *          with FP32 atomics, one per row split or drained accumulator: the order
+ *          of those additions, and so the last bits, may vary between calls)
  * Returns LBM_EINVAL for bad arguments, LBM_ECUDA for a CUDA error (a stream that
  * records a graph among them) and LBM_ETIMEOUT if a pipeline wait ran out. */
 int lbm_conv3d_bf16(int op, const void* in, const void* aux, const void* w, const float* bias, int relu, void* out,
